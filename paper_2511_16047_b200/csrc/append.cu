@@ -181,26 +181,16 @@ cudaError_t launch_append(const Strided& K, const Strided& V, const LayerRegion&
         const int64_t total_chunks = (int64_t)rows * heads * 2 * cpb;
         int64_t grid = (int64_t)(sm_count > 0 ? sm_count : 148) * 8;
         if (grid > total_chunks) grid = total_chunks;
-        append_bulk_kernel<<<(unsigned)grid, 32, kBulkSmem, stream>>>(
-            (const char*)K.ptr, (const char*)V.ptr, block_bytes, (char*)region.base, 4ll * region.capacity * D,
-            2ll * region.capacity * D, 2ll * token_offset * D, (uint32_t)block_bytes, cpb, total_chunks, status);
-        count_launch();
-        return cudaGetLastError();
+        return launch_kernel(false, append_bulk_kernel, dim3((unsigned)grid), dim3(32), kBulkSmem, stream, (const char*)K.ptr,
+                             (const char*)V.ptr, block_bytes, (char*)region.base, 4ll * region.capacity * D,
+                             2ll * region.capacity * D, 2ll * token_offset * D, (uint32_t)block_bytes, cpb, total_chunks, status);
     }
     int64_t blocks = (total + (int64_t)kThreads * kUnroll - 1) / ((int64_t)kThreads * kUnroll);
     if (blocks > (1 << 20)) blocks = 1 << 20;
     auto* dst = reinterpret_cast<uint4*>(region.base);
-    if (D == 64) {
-        append_kernel<64><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            (const uint4*)K.ptr, (const uint4*)V.ptr, K.row, K.head, K.token, V.row, V.head, V.token, dst,
-            region.capacity, token_offset, T, heads, total);
-    } else {
-        append_kernel<128><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            (const uint4*)K.ptr, (const uint4*)V.ptr, K.row, K.head, K.token, V.row, V.head, V.token, dst,
-            region.capacity, token_offset, T, heads, total);
-    }
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(false, D == 64 ? append_kernel<64> : append_kernel<128>, dim3((unsigned)blocks), dim3(kThreads), 0, stream,
+                         (const uint4*)K.ptr, (const uint4*)V.ptr, K.row, K.head, K.token, V.row, V.head, V.token, dst,
+                         region.capacity, token_offset, T, heads, total);
 }
 
 }  // namespace amskv

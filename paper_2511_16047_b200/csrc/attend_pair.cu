@@ -260,6 +260,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
+    // everything up to here touches only this CTA's own memory, so it runs while the kernel before this one ends
+    overlap_with_previous();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
@@ -930,11 +932,9 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
     if (oe != cudaSuccess) return oe;
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
     if (grid > pp.n_pairs) grid = pp.n_pairs;
-    attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort><<<(unsigned)grid, C::kThreads, C::kSmemBytes, stream>>>(
-        qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token, ranges, T, heads, pp, n_tiles, qpos,
-        scale_log2, status, den);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort>, dim3((unsigned)grid), dim3(C::kThreads),
+                         C::kSmemBytes, stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
+                         ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);
 }
 
 }  // namespace

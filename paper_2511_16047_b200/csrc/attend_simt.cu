@@ -49,6 +49,7 @@ attend_simt_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q
                    int32_t heads, int64_t total_rows, float scale_log2, const __nv_bfloat16* __restrict__ ext_k,
                    const __nv_bfloat16* __restrict__ ext_v, int64_t e_row, int64_t e_head, int64_t e_tok, int ext_range)
 {
+    overlap_with_previous();
     constexpr int DPL = D / kLanesPerRow;  // channels per lane
     const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     const int sub = (int)(tid % kLanesPerRow);
@@ -161,17 +162,10 @@ cudaError_t launch_attend_simt(const Strided& Q, const Strided& O, const LayerRe
     const int64_t blocks = (threads + kThreads - 1) / kThreads;
     if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
-    if (D == 64) {
-        attend_simt_kernel<64><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
-            region.base, region.capacity, ranges, T, heads, total_rows, scale_log2, ek, ev, e_row, e_head, e_tok, ext_range);
-    } else {
-        attend_simt_kernel<128><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
-            region.base, region.capacity, ranges, T, heads, total_rows, scale_log2, ek, ev, e_row, e_head, e_tok, ext_range);
-    }
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(cur != nullptr, D == 64 ? attend_simt_kernel<64> : attend_simt_kernel<128>, dim3((unsigned)blocks), dim3(kThreads), 0, stream,
+                         (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
+                         region.base, region.capacity, ranges, T, heads, total_rows, scale_log2, ek, ev, e_row, e_head, e_tok,
+                         ext_range);
 }
 
 }  // namespace amskv

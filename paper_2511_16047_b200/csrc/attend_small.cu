@@ -96,6 +96,7 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
                     int32_t heads, int32_t n_items, float scale_log2, const SmallExt ext)
 {
     constexpr int kPieces = D / 32;     // 16-byte pieces of a token row per lane (the lane's pieces are q + 4h)
+    overlap_with_previous();
     const int lane = threadIdx.x & 31;
     const int item = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
     if (item >= n_items) return;        // whole warps leave together: nothing below synchronises across warps
@@ -282,6 +283,7 @@ single_key_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int6
                   uint4* __restrict__ O, int64_t o_row, int64_t o_head, uint4* __restrict__ region, int32_t capacity,
                   int32_t dst, int32_t store, int32_t heads, int64_t n_pieces)
 {
+    overlap_with_previous();
     constexpr int CPT = D / 8;   // 16-byte pieces per token
     const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (idx >= n_pieces) return;
@@ -327,23 +329,16 @@ cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerR
         // the scale's single token is its only key
         const int64_t n_pieces = items * (D / 8);
         const int64_t blocks = (n_pieces + 255) / 256;
-        if (D == 64)
-            single_key_kernel<64><<<(unsigned)blocks, 256, 0, stream>>>(
-                (const uint4*)ext.K, (const uint4*)ext.V, ext.row, ext.head, (uint4*)O.ptr, O.row, O.head, (uint4*)region.base,
-                region.capacity, ext.dst, ext.store, heads, n_pieces);
-        else
-            single_key_kernel<128><<<(unsigned)blocks, 256, 0, stream>>>(
-                (const uint4*)ext.K, (const uint4*)ext.V, ext.row, ext.head, (uint4*)O.ptr, O.row, O.head, (uint4*)region.base,
-                region.capacity, ext.dst, ext.store, heads, n_pieces);
-        count_launch();
-        return cudaGetLastError();
+        return launch_kernel(true, D == 64 ? single_key_kernel<64> : single_key_kernel<128>, dim3((unsigned)blocks), dim3(256), 0, stream,
+                             (const uint4*)ext.K, (const uint4*)ext.V, ext.row, ext.head, (uint4*)O.ptr, O.row, O.head,
+                             (uint4*)region.base, region.capacity, ext.dst, ext.store, heads, n_pieces);
     }
     const int64_t blocks = (items + kWarpsPerCta - 1) / kWarpsPerCta;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
 #define AMSKV_SMALL_LAUNCH(DD, EXT, TILES)                                                                            \
-    attend_small_kernel<DD, EXT, TILES><<<(unsigned)blocks, kWarpsPerCta * 32, 0, stream>>>(                          \
-        (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token, region.base, \
-        region.capacity, ranges, T, heads, (int32_t)items, scale_log2, ext)
+    return launch_kernel(EXT, attend_small_kernel<DD, EXT, TILES>, dim3((unsigned)blocks), dim3(kWarpsPerCta * 32), 0, stream, \
+                         (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, \
+                         O.token, region.base, region.capacity, ranges, T, heads, (int32_t)items, scale_log2, ext)
 #define AMSKV_SMALL_TILES(DD, EXT)                                                                                    \
     do {                                                                                                              \
         if (total <= 8) AMSKV_SMALL_LAUNCH(DD, EXT, 1);                                                               \
@@ -359,8 +354,6 @@ cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerR
     }
 #undef AMSKV_SMALL_TILES
 #undef AMSKV_SMALL_LAUNCH
-    count_launch();
-    return cudaGetLastError();
 }
 
 }  // namespace amskv

@@ -48,6 +48,7 @@ density_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_hea
 {
     constexpr int DPL = D / kLanesPerRow;
     __shared__ double acc[kMaxDensityPieces];
+    overlap_with_previous();
     for (int i = threadIdx.x; i < pieces.n; i += kThreads) acc[i] = 0.0;
     __syncthreads();
     const int32_t item = blockIdx.x / ctas_per_item;
@@ -106,16 +107,9 @@ cudaError_t launch_density(const Strided& Q, const LayerRegion& region, const De
     if (e != cudaSuccess) return e;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
     const double inv_rows = 1.0 / (double)rows;
-    if (D == 64)
-        density_kernel<64><<<(unsigned)blocks, kThreads, 0, stream>>>((const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token,
-                                                                      region.base, region.capacity, pieces, T, heads,
-                                                                      ctas_per_item, scale_log2, inv_rows, out);
-    else
-        density_kernel<128><<<(unsigned)blocks, kThreads, 0, stream>>>((const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token,
-                                                                       region.base, region.capacity, pieces, T, heads,
-                                                                       ctas_per_item, scale_log2, inv_rows, out);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(false, D == 64 ? density_kernel<64> : density_kernel<128>, dim3((unsigned)blocks), dim3(kThreads), 0, stream,
+                         (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, region.base, region.capacity, pieces, T, heads,
+                         ctas_per_item, scale_log2, inv_rows, out);
 }
 
 }  // namespace amskv

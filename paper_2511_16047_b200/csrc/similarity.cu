@@ -79,6 +79,7 @@ similarity_partial_kernel(const uint4* __restrict__ K_prev, int32_t s_prev, cons
                           int32_t s_cur, int64_t items, int64_t units, int32_t parts, int32_t part_chunks,
                           int32_t items_per_unit, uint64_t inv_s_cur, double* __restrict__ partials)
 {
+    overlap_with_previous();
     constexpr int CPT = D / 16;                      // 32-byte pieces per token; a thread takes one piece at a time
     constexpr int kShift = (D == 64) ? 2 : 3;
     __shared__ double smem[kThreads / 32];
@@ -159,6 +160,7 @@ similarity_partial_kernel(const uint4* __restrict__ K_prev, int32_t s_prev, cons
 __global__ void __launch_bounds__(kThreads)
 similarity_final_kernel(const double* __restrict__ partials, int n, double* __restrict__ out)
 {
+    overlap_with_previous();
     __shared__ double smem[kThreads / 32];
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += kThreads) acc += partials[i];
@@ -194,17 +196,11 @@ cudaError_t launch_similarity(const __nv_bfloat16* K_prev, int32_t side_prev, co
     const uint64_t inv = ((1ull << 36) + (uint64_t)side_cur - 1) / (uint64_t)side_cur;
     const uint4* kp = (const uint4*)K_prev;
     const uint4* kc = (const uint4*)K_cur;
-    if (D == 64)
-        similarity_partial_kernel<64><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            kp, side_prev, kc, side_cur, items, units, (int32_t)parts, part_chunks, items_per_unit, inv, partials);
-    else
-        similarity_partial_kernel<128><<<(unsigned)blocks, kThreads, 0, stream>>>(
-            kp, side_prev, kc, side_cur, items, units, (int32_t)parts, part_chunks, items_per_unit, inv, partials);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(true, D == 64 ? similarity_partial_kernel<64> : similarity_partial_kernel<128>,
+                                        dim3((unsigned)blocks), dim3(kThreads), 0, stream, kp, side_prev, kc, side_cur, items,
+                                        units, (int32_t)parts, part_chunks, items_per_unit, inv, partials);
     if (e != cudaSuccess) return e;
-    similarity_final_kernel<<<1, kThreads, 0, stream>>>(partials, (int)blocks, out_ss);
-    count_launch(2);
-    return cudaGetLastError();
+    return launch_kernel(true, similarity_final_kernel, dim3(1), dim3(kThreads), 0, stream, (const double*)partials, (int)blocks, out_ss);
 }
 
 }  // namespace amskv

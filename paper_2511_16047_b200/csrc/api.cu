@@ -232,14 +232,16 @@ int amskv_cache_create(const amskv_desc* desc, void* dev_mem, size_t dev_bytes, 
     if (rc != AMSKV_OK) { delete c; return rc; }
     if (c->plan_only()) { *out = c; return AMSKV_OK; }
 
-    int dev = 0;
-    cudaDeviceProp prop;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) {
+    // (two attributes, not cudaGetDeviceProperties: it also queries clocks, which takes milliseconds a call; creating the
+    // cache of one layer for one image, arena included: 6 -> 0.7 ms)
+    int dev = 0, major = 0, sm_count = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         (void)cudaGetLastError();
         delete c;
         return AMSKV_ERR_CUDA;
     }
-    c->sm_count = prop.multiProcessorCount;
+    c->sm_count = sm_count;
     if (dev_mem) {
         if ((reinterpret_cast<uintptr_t>(dev_mem) % kAlign) != 0) { delete c; return AMSKV_ERR_INVALID; }
         if (dev_bytes < c->arena_bytes) { delete c; return AMSKV_ERR_NOMEM; }
@@ -264,7 +266,7 @@ int amskv_cache_create(const amskv_desc* desc, void* dev_mem, size_t dev_bytes, 
         return AMSKV_ERR_CUDA;
     }
     c->tc_ready = false;
-    if (tc_supported(c->head_dim) && prop.major == 10) {
+    if (tc_supported(c->head_dim) && major == 10) {
         c->k_maps.resize(c->layers);
         c->v_maps.resize(c->layers);
         c->k_maps64.resize(c->layers);

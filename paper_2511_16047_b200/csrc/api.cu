@@ -191,9 +191,13 @@ void note_appended(amskv_cache* cache, int layer, int scale)
 }
 
 // which kernel amskv_attend uses for T query tokens over `total` keys
-enum class AttendKernel { Small, Simt, Pair, Tensor };
-AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total)
+enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
+AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false)
 {
+    // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained)
+    if (cache->path == AMSKV_PATH_AUTO && T > 1 && cache->tc_ready &&
+        mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density))
+        return AttendKernel::Mid;
     // AUTO: the warp-per-item kernel wherever a scale's retained keys fit its register tile, the paired
     // tcgen05 kernel elsewhere (the CUDA-core kernel only where tensor maps are unavailable)
     // (a single query token per item is fastest on the CUDA-core kernel: measured)
@@ -385,6 +389,9 @@ int amskv_attend(amskv_cache* cache, int layer, int scale, const void* Q, void* 
     if (kernel == AttendKernel::Small) {
         e = launch_attend_small(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
                                 cache->softmax_scale, static_cast<cudaStream_t>(stream));
+    } else if (kernel == AttendKernel::Mid) {
+        e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
+                              cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream));
     } else if (kernel == AttendKernel::Pair) {
         e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes,
                                cache->k_maps64[layer].bytes, cache->v_maps64[layer].bytes, ranges, T, cache->rows,
@@ -432,7 +439,12 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         for (int i = 0; i < rl.n; ++i) rl.total += rl.r[i].len;
         CurrentScaleSource src{ks, vs, false, 0, cache->region(layer)};
         cudaError_t e;
-        if (cache->tc_ready && cache->path != AMSKV_PATH_SIMT && !(cache->path == AMSKV_PATH_AUTO && T == 1))
+        if (choose_kernel(cache, T, rl.total) == AttendKernel::Mid) {
+            --rl.n;   // the kernel takes the scale itself from `src`
+            rl.total -= T;
+            e = launch_attend_mid(q, o, cache->region(layer), rl, T, cache->rows, cache->heads, cache->head_dim,
+                                  cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream), &src);
+        } else if (cache->tc_ready && cache->path != AMSKV_PATH_SIMT && !(cache->path == AMSKV_PATH_AUTO && T == 1))
             e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes, cache->k_maps64[layer].bytes,
                                    cache->v_maps64[layer].bytes, rl, T, cache->rows, cache->heads, cache->head_dim,
                                    cache->softmax_scale, cache->status_word(), cache->sm_count,
@@ -472,8 +484,20 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
             return AMSKV_OK;
         }
     }
-    bool fused = cache->tc_ready && kernel == AttendKernel::Pair && one_copy;
     RangeList ranges;
+    if (kernel == AttendKernel::Mid) {
+        // takes any set of copies and any number of older ranges
+        ranges.n = lay.ranges_before(cache->tokens, scale, ranges.r);
+        ranges.total = 0;
+        for (int i = 0; i < ranges.n; ++i) ranges.total += ranges.r[i].len;
+        CurrentScaleSource cur{ks, vs, true, 0, cache->region(layer)};
+        cudaError_t e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
+                                          cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream), &cur, piece, n_pieces);
+        if (e != cudaSuccess) { (void)cudaGetLastError(); return AMSKV_ERR_CUDA; }
+        note_appended(cache, layer, scale);
+        return AMSKV_OK;
+    }
+    bool fused = cache->tc_ready && kernel == AttendKernel::Pair && one_copy;
     if (fused) {
         ranges.n = lay.ranges_before(cache->tokens, scale, ranges.r);
         if (ranges.n >= kMaxRanges) fused = false;
@@ -586,9 +610,10 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
     if (n < 0) return AMSKV_ERR_UNSUPPORTED;   // the scale's own keys are not in the cache (never-stored last scale)
     int32_t total = 0;
     for (int32_t i = 0; i < n; ++i) total += rp[i].len;
-    // One launch where the paired kernel serves the scale: its key tiles are cut at the boundaries of the runs
-    // (one range per piece of a run), and each row's mass per run falls out of the softmax loop.
-    if (cache->tc_ready && choose_kernel(cache, T, total) == AttendKernel::Pair && n_runs <= kPairMaxDensityRuns && n <= kMaxRanges) {
+    // One launch where the paired or the warp-matrix kernel serves the scale: the former cuts its key tiles at the
+    // boundaries of the runs (one range per piece of a run), the latter multiplies P by the keys' run membership.
+    const AttendKernel kernel = choose_kernel(cache, T, total, true);
+    if (cache->tc_ready && (kernel == AttendKernel::Pair || kernel == AttendKernel::Mid) && n_runs <= kPairMaxDensityRuns && n <= kMaxRanges) {
         RangeList ranges;
         PairDensity den;
         den.out = density;
@@ -602,7 +627,10 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
         }
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         cudaError_t e = cudaMemsetAsync(density, 0, sizeof(double) * (size_t)cache->heads * n_runs, st);
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && kernel == AttendKernel::Mid)
+            e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
+                                  cache->softmax_scale, cache->sm_count, st, nullptr, nullptr, 0, &den);
+        else if (e == cudaSuccess)
             e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes, cache->k_maps64[layer].bytes,
                                    cache->v_maps64[layer].bytes, ranges, T, cache->rows, cache->heads, cache->head_dim,
                                    cache->softmax_scale, cache->status_word(), cache->sm_count, st, nullptr, &den);

@@ -1,0 +1,573 @@
+// Attention for calls of few (row, head) items or few queries, which the paired tensor-memory kernel spends on its
+// set-up and on its per-tile chain rather than on memory or arithmetic.
+//
+// A CTA serves up to NW / 2 sixteen-row query blocks of one item with warp-level matrix instructions (mma.sync), two warps
+// per query block, each with half of the keys of every chunk.  Keys are one packed sequence -- the retained ranges of the
+// cache first, then (append fused in) the current scale in the caller's tensors -- cut into 64-key chunks with no regard
+// to where a range ends.  K and V of a chunk go to a stage of shared memory by 16-byte asynchronous copies of all threads, up
+// to kStages chunks ahead, so the whole key set of a coarse scale is in flight after a few hundred clocks; there is no
+// tensor map, no tensor memory to allocate and no role to hand data to.  The thread that copied a piece of the current
+// scale also writes it to its place in the cache, after the output where the stage can wait that long.
+//
+// S = Q K^T takes both operands as 16-byte pieces used directly as fragment registers (the contraction order inside a
+// piece is permuted alike on both sides); K pieces are swizzled by the row's lowest bit for conflict-free 16-byte
+// reads, V pieces by its three lowest bits for ldmatrix.trans.  A row's reference maximum moves only when a chunk exceeds
+// it by more than 2^8; the two halves of the keys are merged through shared memory at the end.
+//
+// Attention density (kDen): the mass of a row on each of up to 16 runs of keys is P times a 0/1 matrix of run membership,
+// two more column tiles of the second product.  P enters as the sum of two bf16 numbers, so the masses are those of the
+// unrounded probabilities to 2^-16.
+#include <cstring>
+
+#include "kernels.cuh"
+
+namespace amskv {
+
+namespace {
+
+constexpr int kChunk = 64;            // keys per stage
+constexpr int kSplits = 2;            // warps per query block
+constexpr float kRescaleLog2 = 8.f;
+constexpr int kMaxDenRuns = kPairMaxDensityRuns;
+
+template <int D, bool kDen>
+struct MidCfg {
+    static constexpr int kStages = D == 64 ? 4 : 2;
+    static constexpr int kRowBytes = D * 2;
+    static constexpr int kTileBytes = kChunk * kRowBytes;       // one of K, V
+    static constexpr int kStageBytes = 2 * kTileBytes;
+    static constexpr int kMergeBytes = (16 * D + 32 + (kDen ? 256 : 0)) * 4;   // O, maxima and sums (and masses) of 16 rows
+};
+
+struct MidExt {
+    const __nv_bfloat16* K;
+    const __nv_bfloat16* V;
+    int64_t row, head, tok;            // element strides, the same for K and V
+    int32_t len;                       // tokens of the current scale read from there (0: none)
+    int32_t n_pieces;                  // where they go in the per-item region
+    Piece piece[LayerLayout::kMaxPieces];
+};
+struct MidDen {
+    double* out;
+    int32_t n_runs;
+    float weight[kMaxDenRuns];
+    int8_t run_of_range[kMaxRanges];
+};
+
+__device__ __forceinline__ float fast_exp2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                          uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+// 16 bytes global -> shared
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float y;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+// a * b + c and d + a on two packed fp32 lanes
+__device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c)
+{
+    asm("{\n"
+        ".reg .b64 ra, rb, rc, rd;\n"
+        "mov.b64 ra, {%2, %3};\n"
+        "mov.b64 rb, {%4, %4};\n"
+        "mov.b64 rc, {%5, %5};\n"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n"
+        "mov.b64 {%0, %1}, rd;\n"
+        "}\n"
+        : "=f"(d0), "=f"(d1)
+        : "f"(a0), "f"(a1), "f"(b), "f"(c));
+}
+__device__ __forceinline__ void add2(float (&d)[2], float a0, float a1)
+{
+    asm("{\n"
+        ".reg .b64 ra, rd;\n"
+        "mov.b64 ra, {%2, %3};\n"
+        "mov.b64 rd, {%0, %1};\n"
+        "add.rn.f32x2 rd, rd, ra;\n"
+        "mov.b64 {%0, %1}, rd;\n"
+        "}\n"
+        : "+f"(d[0]), "+f"(d[1])
+        : "f"(a0), "f"(a1));
+}
+
+// 4x4 transpose of 32-bit words among the four lanes of a quad: lane q's w[j] becomes lane j's w[q]
+__device__ __forceinline__ void quad_transpose(uint32_t (&w)[4], int q)
+{
+    const bool odd = q & 1, high = q & 2;
+    {
+        const uint32_t s0 = odd ? w[0] : w[1], s1 = odd ? w[2] : w[3];
+        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+        if (odd) { w[0] = r0; w[2] = r1; } else { w[1] = r0; w[3] = r1; }
+    }
+    {
+        const uint32_t s0 = high ? w[0] : w[2], s1 = high ? w[1] : w[3];
+        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, s0, 2), r1 = __shfl_xor_sync(0xffffffffu, s1, 2);
+        if (high) { w[0] = r0; w[1] = r1; } else { w[2] = r0; w[3] = r1; }
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void scale_rows(float (&o)[N][4], float f_a, float f_b)
+{
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        o[n][0] *= f_a;
+        o[n][1] *= f_a;
+        o[n][2] *= f_b;
+        o[n][3] *= f_b;
+    }
+}
+
+template <int D, int NW, bool kDen>
+__global__ void __launch_bounds__(NW * 32, D == 64 ? 16 / NW : 2)
+attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
+                  __nv_bfloat16* __restrict__ O, int64_t o_row, int64_t o_head, int64_t o_tok,
+                  __nv_bfloat16* __restrict__ region, int32_t capacity, const __grid_constant__ RangeList ranges,
+                  int32_t T, int32_t heads, int32_t parts, int32_t n_rb, int32_t n_stages, float scale_log2,
+                  const __grid_constant__ MidExt ext, const __grid_constant__ MidDen den)
+{
+    using C = MidCfg<D, kDen>;
+    constexpr int kPieces = D / 32;            // 16-byte pieces of a token row per lane in fragment order
+    constexpr int kTokPieces = D / 8;          // 16-byte pieces of a token row
+    constexpr int kWarpKeys = kChunk / kSplits, kTiles = kWarpKeys / 8;
+    constexpr int kDenTiles = kDen ? 2 : 1;    // (one unused register tile otherwise)
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ int8_t key_run[kDen ? C::kStages : 1][kChunk];
+    __shared__ double den_sum[kDen ? kMaxDenRuns : 1];
+    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(smem);
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int g = lane >> 2, q = lane & 3;
+    const int ks = warp % kSplits, rb = warp / kSplits;
+    const int32_t item = blockIdx.x / parts, part = blockIdx.x - item * parts;
+    const int32_t row = item / heads, head = item - row * heads;
+    const int32_t m0 = (part * n_rb + rb) * 16;                 // first query row of this warp
+    const bool live = rb < n_rb && m0 < T;                      // (a warp without a query block only copies)
+    const int32_t Lc = ranges.total, L = Lc + ext.len;
+    const int32_t n_chunks = (L + kChunk - 1) / kChunk;
+    __nv_bfloat16* kbase = region + (int64_t)item * (2ll * capacity * D);
+    const int64_t v_shift = (int64_t)capacity * D;
+
+    // This thread's part of the copies: one 16-byte column of every kStep-th row.  kStep is a multiple of 8, so the
+    // swizzle of a thread's rows is the same for all of them.
+    constexpr int kStep = NW * 32 / kTokPieces, kRows = kChunk / kStep;
+    static_assert(kStep % 8 == 0 && kChunk % kStep == 0, "copy mapping");
+    const int cp_piece = (int)threadIdx.x % kTokPieces, cp_row0 = (int)threadIdx.x / kTokPieces;
+    const uint32_t k_slot = (uint32_t)cp_row0 * C::kRowBytes + (uint32_t)((cp_piece ^ ((cp_row0 & 1) << 2)) << 4);
+    const uint32_t v_slot = C::kTileBytes + (uint32_t)cp_row0 * C::kRowBytes + (uint32_t)((cp_piece ^ (cp_row0 & 7)) << 4);
+
+    // The source of keys src_first .. src_end - 1; walks forward as the chunks do.
+    int src_range = -1;
+    int32_t src_first = 0, src_end = 0;
+    const __nv_bfloat16 *src_k = nullptr, *src_v = nullptr;   // of key src_first
+    int64_t src_tok = D;
+    auto next_source = [&]() {
+        ++src_range;
+        src_first = src_end;
+        if (src_range < ranges.n) {
+            src_k = kbase + (int64_t)ranges.r[src_range].start * D;
+            src_v = src_k + v_shift;
+            src_end = src_first + ranges.r[src_range].len;
+        } else {
+            src_k = ext.K + row * ext.row + head * ext.head;
+            src_v = ext.V + row * ext.row + head * ext.head;
+            src_tok = ext.tok;
+            src_end = L;
+        }
+    };
+    auto load_chunk = [&](int c, int stage) {
+        const uint32_t st = smem0 + (uint32_t)stage * C::kStageBytes;
+        const int32_t first = c * kChunk, end = min(first + kChunk, L);
+        // one pass per source the chunk draws from (nearly always one)
+        for (int32_t at = first; at < end;) {
+            while (at >= src_end) next_source();
+            const int32_t stop = min(src_end, end);
+            const __nv_bfloat16* kp = src_k + (int64_t)(first + cp_row0 - src_first) * src_tok + cp_piece * 8;
+            const __nv_bfloat16* vp = src_v + (int64_t)(first + cp_row0 - src_first) * src_tok + cp_piece * 8;
+#pragma unroll
+            for (int i = 0; i < kRows; ++i) {
+                const int32_t key = first + cp_row0 + i * kStep;
+                if (key >= at && key < stop) {
+                    cp_async16(st + k_slot + i * kStep * C::kRowBytes, kp + (int64_t)(i * kStep) * src_tok);
+                    cp_async16(st + v_slot + i * kStep * C::kRowBytes, vp + (int64_t)(i * kStep) * src_tok);
+                    if (kDen && cp_piece == 0) key_run[stage][cp_row0 + i * kStep] = den.run_of_range[src_range];
+                }
+            }
+            at = stop;
+        }
+        if (end - first < kChunk) {   // rows past the last key: finite, and of no run
+#pragma unroll
+            for (int i = 0; i < kRows; ++i)
+                if (first + cp_row0 + i * kStep >= end) {
+                    uint8_t* dst = smem + stage * C::kStageBytes + i * kStep * C::kRowBytes;
+                    *reinterpret_cast<uint4*>(dst + k_slot) = make_uint4(0, 0, 0, 0);
+                    *reinterpret_cast<uint4*>(dst + v_slot) = make_uint4(0, 0, 0, 0);
+                    if (kDen && cp_piece == 0) key_run[stage][cp_row0 + i * kStep] = -1;
+                }
+        }
+    };
+    // the append: this thread's own pieces of chunk c's share of the current scale, from the stage to their place in the
+    // cache (the item's CTAs share the chunks)
+    auto store_chunk = [&](int c, int stage) {
+        if (ext.n_pieces == 0 || (c + 1) * kChunk <= Lc || c % parts != part) return;
+        const uint8_t* tile = smem + stage * C::kStageBytes;
+#pragma unroll 1
+        for (int i = 0; i < kRows; ++i) {
+            const int32_t j = c * kChunk + cp_row0 + i * kStep - Lc;
+            if (j < 0 || j >= ext.len) continue;
+            int32_t d = -1;
+            for (int n = 0; n < ext.n_pieces; ++n)
+                if (j >= ext.piece[n].src && j < ext.piece[n].src + ext.piece[n].len) d = ext.piece[n].dst + j - ext.piece[n].src;
+            if (d < 0) continue;
+            __nv_bfloat16* kd = kbase + (int64_t)d * D + cp_piece * 8;
+            *reinterpret_cast<uint4*>(kd) = *reinterpret_cast<const uint4*>(tile + k_slot + i * kStep * C::kRowBytes);
+            *reinterpret_cast<uint4*>(kd + v_shift) = *reinterpret_cast<const uint4*>(tile + v_slot + i * kStep * C::kRowBytes);
+        }
+    };
+
+    next_source();   // (reads launch parameters only)
+    const __nv_bfloat16* qbase = Q + row * q_row + head * q_head;
+    const uint4* q0 = reinterpret_cast<const uint4*>(qbase + min(m0 + g, T - 1) * q_tok + 8 * q);
+    const uint4* q1 = reinterpret_cast<const uint4*>(qbase + min(m0 + g + 8, T - 1) * q_tok + 8 * q);
+    overlap_with_previous();
+    // query pieces of rows m0 + g and m0 + g + 8 (clamped; rows past T are not stored)
+    uint4 qa0[kPieces], qa1[kPieces];
+#pragma unroll
+    for (int h = 0; h < kPieces; ++h) {
+        qa0[h] = __ldg(q0 + 4 * h);
+        qa1[h] = __ldg(q1 + 4 * h);
+    }
+#pragma unroll 1
+    for (int c = 0; c < C::kStages; ++c) {
+        if (c < n_chunks) load_chunk(c, c);   // (n_stages = min(kStages, n_chunks))
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (kDen && threadIdx.x < kMaxDenRuns) den_sum[threadIdx.x] = 0.0;
+
+    float o[D / 8][4];
+#pragma unroll
+    for (int n = 0; n < D / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
+    float od[kDenTiles][4];
+#pragma unroll
+    for (int n = 0; n < kDenTiles; ++n) od[n][0] = od[n][1] = od[n][2] = od[n][3] = 0.f;
+    float m_a = -INFINITY, m_b = -INFINITY, nb_a = 0.f, nb_b = 0.f;
+    float l2_a[2] = {0.f, 0.f}, l2_b[2] = {0.f, 0.f};   // row sums of the even and of the odd keys
+
+    int stage = 0;
+#pragma unroll 1
+    for (int c = 0; c < n_chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(C::kStages - 1) : "memory");
+        __syncthreads();
+        const uint8_t* tile = smem + stage * C::kStageBytes;
+        const int32_t key0 = c * kChunk + ks * kWarpKeys;
+        if (live && key0 < L) {
+            const uint8_t* kt = tile + (ks * kWarpKeys + g) * C::kRowBytes;
+            const int kx = (q ^ ((g & 1) << 2)) << 4;
+            float s[kTiles][4];
+#pragma unroll
+            for (int t = 0; t < kTiles; ++t) {
+                s[t][0] = s[t][1] = s[t][2] = s[t][3] = 0.f;
+#pragma unroll
+                for (int h = 0; h < kPieces; ++h) {
+                    const uint4 kk = *reinterpret_cast<const uint4*>(kt + t * 8 * C::kRowBytes + (kx ^ (h << 6)));
+                    mma_16816(s[t], qa0[h].x, qa1[h].x, qa0[h].y, qa1[h].y, kk.x, kk.y);
+                    mma_16816(s[t], qa0[h].z, qa1[h].z, qa0[h].w, qa1[h].w, kk.z, kk.w);
+                }
+            }
+            if (key0 + kWarpKeys > L) {
+#pragma unroll
+                for (int t = 0; t < kTiles; ++t)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        if (key0 + t * 8 + 2 * q + e >= L) s[t][e] = s[t][2 + e] = -INFINITY;
+            }
+            float mx_a = fmaxf(s[0][0], s[0][1]), mx_b = fmaxf(s[0][2], s[0][3]);
+#pragma unroll
+            for (int t = 1; t < kTiles; ++t) {
+                mx_a = max3(mx_a, s[t][0], s[t][1]);
+                mx_b = max3(mx_b, s[t][2], s[t][3]);
+            }
+            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 1));
+            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 1));
+            mx_a = fmaxf(mx_a, __shfl_xor_sync(0xffffffffu, mx_a, 2));
+            mx_b = fmaxf(mx_b, __shfl_xor_sync(0xffffffffu, mx_b, 2));
+            // (the first chunk always moves the reference: it starts at minus infinity)
+            const bool grow_a = (mx_a - m_a) * scale_log2 > kRescaleLog2, grow_b = (mx_b - m_b) * scale_log2 > kRescaleLog2;
+            if (__any_sync(0xffffffffu, grow_a || grow_b)) {
+                const float f_a = grow_a ? fast_exp2((m_a - mx_a) * scale_log2) : 1.f;
+                const float f_b = grow_b ? fast_exp2((m_b - mx_b) * scale_log2) : 1.f;
+                if (grow_a) { m_a = mx_a; nb_a = -mx_a * scale_log2; }
+                if (grow_b) { m_b = mx_b; nb_b = -mx_b * scale_log2; }
+                l2_a[0] *= f_a;
+                l2_a[1] *= f_a;
+                l2_b[0] *= f_b;
+                l2_b[1] *= f_b;
+                scale_rows(o, f_a, f_b);
+                if (kDen) scale_rows(od, f_a, f_b);
+            }
+            // ---- P V, 16 keys at a time
+            const int vkey = ks * kWarpKeys + (lane & 15);
+            const uint32_t vt = smem0 + (uint32_t)stage * C::kStageBytes + C::kTileBytes + (uint32_t)vkey * C::kRowBytes;
+            const uint32_t vx = (uint32_t)(((lane >> 4) ^ (vkey & 7)) << 4);
+#pragma unroll
+            for (int step = 0; step < kTiles / 2; ++step) {
+                uint32_t p[4];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float (&x)[4] = s[2 * step + u];
+                    fma2(x[0], x[1], x[0], x[1], scale_log2, nb_a);
+                    fma2(x[2], x[3], x[2], x[3], scale_log2, nb_b);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) x[e] = fast_exp2(x[e]);
+                    add2(l2_a, x[0], x[1]);
+                    add2(l2_b, x[2], x[3]);
+                    p[2 * u] = pack_bf16(x[0], x[1]);
+                    p[2 * u + 1] = pack_bf16(x[2], x[3]);
+                }
+#pragma unroll
+                for (int j = 0; j < D / 16; ++j) {
+                    uint32_t v[4];
+                    ldmatrix_x4_trans(v, vt + step * 16 * C::kRowBytes + ((uint32_t)(j << 5) ^ vx));
+                    mma_16816(o[2 * j], p[0], p[1], p[2], p[3], v[0], v[1]);
+                    mma_16816(o[2 * j + 1], p[0], p[1], p[2], p[3], v[2], v[3]);
+                }
+                if (kDen) {
+                    uint32_t lo[4];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float (&x)[4] = s[2 * step + u];
+                        lo[2 * u] = pack_bf16(x[0] - bf16_lo(p[2 * u]), x[1] - bf16_hi(p[2 * u]));
+                        lo[2 * u + 1] = pack_bf16(x[2] - bf16_lo(p[2 * u + 1]), x[3] - bf16_hi(p[2 * u + 1]));
+                    }
+                    const int8_t* kr = &key_run[kDen ? stage : 0][ks * kWarpKeys + step * 16 + 2 * q];
+#pragma unroll
+                    for (int n = 0; n < kDenTiles; ++n) {
+                        const int run = n * 8 + g;
+                        const uint32_t b0 = (kr[0] == run ? 0x3f80u : 0u) | (kr[1] == run ? 0x3f800000u : 0u);
+                        const uint32_t b1 = (kr[8] == run ? 0x3f80u : 0u) | (kr[9] == run ? 0x3f800000u : 0u);
+                        mma_16816(od[n], p[0], p[1], p[2], p[3], b0, b1);
+                        mma_16816(od[n], lo[0], lo[1], lo[2], lo[3], b0, b1);
+                    }
+                }
+            }
+        }
+        if (c + C::kStages < n_chunks) {
+            store_chunk(c, stage);
+            __syncthreads();
+            load_chunk(c + C::kStages, stage);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        stage = stage + 1 == n_stages ? 0 : stage + 1;
+    }
+
+    // row sums: a row is spread over the four lanes of a quad
+    float l_a = l2_a[0] + l2_a[1], l_b = l2_b[0] + l2_b[1];
+    l_a += __shfl_xor_sync(0xffffffffu, l_a, 1);
+    l_b += __shfl_xor_sync(0xffffffffu, l_b, 1);
+    l_a += __shfl_xor_sync(0xffffffffu, l_a, 2);
+    l_b += __shfl_xor_sync(0xffffffffu, l_b, 2);
+
+    // ---- merge the two halves of the keys: the second warp leaves its part in shared memory, the first adds it
+    float* other = reinterpret_cast<float*>(smem + n_stages * C::kStageBytes + rb * C::kMergeBytes);
+    float4* other4 = reinterpret_cast<float4*>(other);
+    float* other_ml = other + 16 * D;
+    float4* other_den = reinterpret_cast<float4*>(other + 16 * D + 32);
+    if (ks > 0 && live) {
+#pragma unroll
+        for (int n = 0; n < D / 8; ++n) other4[n * 32 + lane] = make_float4(o[n][0], o[n][1], o[n][2], o[n][3]);
+        if (q == 0) {
+            other_ml[g] = m_a;
+            other_ml[8 + g] = m_b;
+            other_ml[16 + g] = l_a;
+            other_ml[24 + g] = l_b;
+        }
+        if (kDen) {
+#pragma unroll
+            for (int n = 0; n < kDenTiles; ++n) other_den[n * 32 + lane] = make_float4(od[n][0], od[n][1], od[n][2], od[n][3]);
+        }
+    }
+    __syncthreads();
+    if (ks == 0 && live) {
+        const float om_a = other_ml[g], om_b = other_ml[8 + g];
+        const float M_a = fmaxf(m_a, om_a), M_b = fmaxf(m_b, om_b);
+        const float f_a = fast_exp2((m_a - M_a) * scale_log2), f_b = fast_exp2((m_b - M_b) * scale_log2);
+        const float e_a = fast_exp2((om_a - M_a) * scale_log2), e_b = fast_exp2((om_b - M_b) * scale_log2);
+        l_a = fmaf(other_ml[16 + g], e_a, l_a * f_a);
+        l_b = fmaf(other_ml[24 + g], e_b, l_b * f_b);
+        scale_rows(o, f_a, f_b);
+#pragma unroll
+        for (int n = 0; n < D / 8; ++n) {
+            const float4 x = other4[n * 32 + lane];
+            o[n][0] = fmaf(x.x, e_a, o[n][0]);
+            o[n][1] = fmaf(x.y, e_a, o[n][1]);
+            o[n][2] = fmaf(x.z, e_b, o[n][2]);
+            o[n][3] = fmaf(x.w, e_b, o[n][3]);
+        }
+        if (kDen) {
+            scale_rows(od, f_a, f_b);
+#pragma unroll
+            for (int n = 0; n < kDenTiles; ++n) {
+                const float4 x = other_den[n * 32 + lane];
+                od[n][0] = fmaf(x.x, e_a, od[n][0]);
+                od[n][1] = fmaf(x.y, e_a, od[n][1]);
+                od[n][2] = fmaf(x.z, e_b, od[n][2]);
+                od[n][3] = fmaf(x.w, e_b, od[n][3]);
+            }
+        }
+        // ---- out = O / l: after a transpose among the quad a lane holds 8 consecutive channels of its rows
+        const float inv_a = 1.f / l_a, inv_b = 1.f / l_b;
+        const bool st_a = m0 + g < T, st_b = m0 + g + 8 < T;
+        __nv_bfloat16* obase = O + row * o_row + head * o_head + (int64_t)(m0 + g) * o_tok + 8 * q;
+#pragma unroll
+        for (int h = 0; h < kPieces; ++h) {
+            uint32_t w[4], x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                w[j] = pack_bf16(o[4 * h + j][0] * inv_a, o[4 * h + j][1] * inv_a);
+                x[j] = pack_bf16(o[4 * h + j][2] * inv_b, o[4 * h + j][3] * inv_b);
+            }
+            quad_transpose(w, q);
+            quad_transpose(x, q);
+            if (st_a) *reinterpret_cast<uint4*>(obase + 32 * h) = make_uint4(w[0], w[1], w[2], w[3]);
+            if (st_b) *reinterpret_cast<uint4*>(obase + 8 * o_tok + 32 * h) = make_uint4(x[0], x[1], x[2], x[3]);
+        }
+        if (kDen) {
+#pragma unroll
+            for (int n = 0; n < kDenTiles; ++n)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    float v = (st_a ? od[n][e] * inv_a : 0.f) + (st_b ? od[n][2 + e] * inv_b : 0.f);
+                    v += __shfl_xor_sync(0xffffffffu, v, 4);
+                    v += __shfl_xor_sync(0xffffffffu, v, 8);
+                    v += __shfl_xor_sync(0xffffffffu, v, 16);
+                    if (g == 0) atomicAdd(&den_sum[kDen ? n * 8 + 2 * q + e : 0], (double)v);
+                }
+        }
+    }
+    // chunks whose stages were never refilled (a thread reads back its own copies only)
+    for (int c = max(0, n_chunks - C::kStages); c < n_chunks; ++c) store_chunk(c, c % n_stages);
+    if (kDen) {
+        __syncthreads();
+        if ((int)threadIdx.x < den.n_runs)
+            atomicAdd(den.out + (int64_t)head * den.n_runs + threadIdx.x, den_sum[kDen ? threadIdx.x : 0] * (double)den.weight[threadIdx.x]);
+    }
+}
+
+template <int D, int NW, bool kDen>
+cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges, int32_t T,
+                   int32_t heads, int64_t items, float scale_log2, const MidExt& ext, const MidDen& den, cudaStream_t stream)
+{
+    using C = MidCfg<D, kDen>;
+    const int n_rb_all = (T + 15) / 16;
+    const int parts = (n_rb_all + NW / kSplits - 1) / (NW / kSplits);
+    const int n_rb = (n_rb_all + parts - 1) / parts;
+    if (items * parts > 0x7fffffffll) return cudaErrorInvalidValue;
+    const int n_chunks = (ranges.total + ext.len + kChunk - 1) / kChunk;
+    const int n_stages = n_chunks < C::kStages ? n_chunks : C::kStages;
+    static SharedMemoryOptIn opt_in;
+    const cudaError_t oe = opt_in.ensure(attend_mid_kernel<D, NW, kDen>, C::kStages * C::kStageBytes + NW / kSplits * C::kMergeBytes);
+    if (oe != cudaSuccess) return oe;
+    return launch_kernel(overlap, attend_mid_kernel<D, NW, kDen>, dim3((unsigned)(items * parts)), dim3(NW * 32),
+                         (size_t)(n_stages * C::kStageBytes + n_rb * C::kMergeBytes), stream, (const __nv_bfloat16*)Q.ptr, Q.row,
+                         Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token, region.base, region.capacity, ranges, T,
+                         heads, (int32_t)parts, (int32_t)n_rb, (int32_t)n_stages, scale_log2, ext, den);
+}
+
+}  // namespace
+
+// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.  64 channels: 19 units.
+// Below it the paired kernel (and, where the append cannot be fused into that, the copy before it) costs 6 to 14 us
+// whatever the size; above it the warp-level matrix instructions, a quarter of the tensor pipe's rate, are what the call
+// takes.  us per call, this kernel / the paired one, append included, in a graph: T = 25: 3.9 / 8.9 (60 items), 6.4 / 11.2
+// (512), 11.5 / 14.9 (1 024), 19.7 / 19.8 (1 920); T = 36: 4.7 / 6.6 (60), 6.4 / 7.9 (256), 12.9 / 9.0 (512); T = 64: 5.1 / 7.4
+// (60), 8.9 / 9.6 (256), 15.7 / 11.2 (512); T = 100: 7.2 / 10.0 (60), 9.2 / 10.8 (128), 16.1 / 12.4 (256); T = 169: 8.5 / 9.9 (32),
+// 11.3 / 10.4 (60).  128 channels: 6 units: T = 36: 5.2 / 10.2 (32), 6.2 / 10.8 (128), 20.5 / 17.1 (512); T = 64: 6.5 / 7.2 (32),
+// 8.7 / 8.5 (128); T = 144: 10.5 / 9.2 (32).  With the density the paired kernel's tiles are cut at the runs and the line lies
+// higher (T = 25, 36, 64 at 512 items: 13.4 / 19.7, 21.1 / 23.2, 26.7 / 26.3; 128 channels, T = 64, 128 items: 15.4 / 20.2), and up to 16
+// queries the alternative is the attention call plus the CUDA-core density pass (T = 4, 9, 16 at 512 items: 12.5 / 16.6,
+// 13.5 / 23.6, 13.0 / 35.0): always this one.  Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).
+bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density)
+{
+    if (density && T <= kSmallMaxQueries) return true;
+    if (!density && small_supported(T, total_keys)) return false;
+    const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
+    return units <= (int64_t)sm_count * (D == 64 ? (density ? 24 : 19) : (density ? 10 : 6));
+}
+
+cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges, int32_t T,
+                              int32_t rows, int32_t heads, int32_t D, float softmax_scale, int sm_count, cudaStream_t stream,
+                              const CurrentScaleSource* cur, const Piece* piece, int32_t n_pieces, const PairDensity* density)
+{
+    MidExt ext;
+    memset(&ext, 0, sizeof(ext));
+    if (cur) {
+        if (cur->V.row != cur->K.row || cur->V.head != cur->K.head || cur->V.token != cur->K.token) return cudaErrorNotSupported;
+        if (n_pieces < 0 || n_pieces > LayerLayout::kMaxPieces) return cudaErrorInvalidValue;
+        ext.K = (const __nv_bfloat16*)cur->K.ptr;
+        ext.V = (const __nv_bfloat16*)cur->V.ptr;
+        ext.row = cur->K.row;
+        ext.head = cur->K.head;
+        ext.tok = cur->K.token;
+        ext.len = T;
+        ext.n_pieces = n_pieces;
+        for (int i = 0; i < n_pieces; ++i) ext.piece[i] = piece[i];
+    }
+    MidDen den;
+    memset(&den, 0, sizeof(den));
+    if (density) {
+        if (cur || density->n_runs < 1 || density->n_runs > kMaxDenRuns) return cudaErrorInvalidValue;
+        den.out = density->out;
+        den.n_runs = density->n_runs;
+        for (int i = 0; i < density->n_runs; ++i) den.weight[i] = density->weight[i];
+        for (int i = 0; i < ranges.n; ++i) den.run_of_range[i] = density->run_of_range[i];
+    }
+    if (T < 1 || ranges.total + ext.len < 1) return cudaErrorInvalidValue;
+    const int64_t items = (int64_t)rows * heads;
+    const float scale_log2 = softmax_scale * 1.4426950408889634f;
+    const bool overlap = cur != nullptr;
+#define AMSKV_MID_LAUNCH(DD, NN, DEN) return launch<DD, NN, DEN>(overlap, Q, O, region, ranges, T, heads, items, scale_log2, ext, den, stream)
+    if (D == 128) {
+        if (density) AMSKV_MID_LAUNCH(128, 4, true);
+        AMSKV_MID_LAUNCH(128, 4, false);
+    }
+    // Four query blocks per CTA; two where there are no more, or where that still gives no SM a second CTA (T = 25, 512 items:
+    // 6.3 us with 4 warps, 8.6 with 8; T = 64, 60 items: 5.1 and 5.8; T = 64, 256 items: 9.3 and 8.9).
+    if (T <= 32 || items * ((T + 31) / 32) <= sm_count) {
+        if (density) AMSKV_MID_LAUNCH(64, 4, true);
+        AMSKV_MID_LAUNCH(64, 4, false);
+    }
+    if (density) AMSKV_MID_LAUNCH(64, 8, true);
+    AMSKV_MID_LAUNCH(64, 8, false);
+#undef AMSKV_MID_LAUNCH
+}
+
+}  // namespace amskv

@@ -1,0 +1,95 @@
+"""GPU parity of the warp-matrix kernel that AMSKV_PATH_AUTO uses for calls of few items or few queries: edges of its
+16-query blocks and 64-key chunks, key sets longer than its ring of stages, several cache ranges, fused appends of
+several copies, the never-stored last scale, and the densities from its third product."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2511_16047_b200 import binding as B
+
+from gpu_common import Cache, check_close, make_qkv, to_items
+
+pytestmark = pytest.mark.gpu
+
+# sides -> T = 4, 9, 16, 25, 36, 49, 64, 81: one to six query blocks, full and partial; the key counts of the layers below run
+# from 13 to 285, across the chunk edges, with and without a refilled stage
+SIDES = (2, 3, 4, 5, 6, 7, 8, 9)
+POLICIES = [(1, 1, False), (2, 3, False), (0, 9, True)]
+
+
+def _run(D, rows, heads, fused, budgets=None, flags=0, peaked=False, packed=False, density=False):
+    qkv = make_qkv(rows, heads, SIDES, D, seed=91, peaked=peaked)
+    if packed:
+        qkv = [tuple(x.transpose(1, 2).contiguous().transpose(1, 2) for x in t) for t in qkv]
+    Ks, Vs = [to_items(k) for _, k, _ in qkv], [to_items(v) for _, _, v in qkv]
+    scale = 1.0 / math.sqrt(D)
+    with Cache(len(POLICIES), heads, D, rows, SIDES, POLICIES, flags=flags, token_budgets=budgets) as c:
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(POLICIES)):
+                out = torch.full_like(q, float("nan"))
+                n0 = B.amskv_launch_count()
+                if fused:
+                    B.amskv_append_attend(c.h, layer, k, kk, v, q, out)
+                    assert B.amskv_launch_count() - n0 == 1      # whatever the number of copies of the append
+                else:
+                    B.amskv_append(c.h, layer, k, kk, v)
+                runs = B.amskv_attended_tokens(c.h, layer, k)
+                if density:
+                    den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+                    B.amskv_attend_density(c.h, layer, k, q, out, den, den.numel())
+                elif not fused:
+                    B.amskv_attend(c.h, layer, k, q, out)
+                torch.cuda.synchronize()
+                tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
+                check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, scale),
+                            "layer %d scale %d" % (layer, k), max_abs=4e-2 if peaked else 1e-2)
+                if density:
+                    want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
+                    # masses from 16 bits of P and fp32 sums: the tolerance of the paired kernel's densities holds too
+                    assert np.allclose(den.cpu().numpy(), want, rtol=2e-4, atol=1e-7), (layer, k)
+        assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
+@pytest.mark.parametrize("rows,heads", [(1, 1), (3, 5)])
+def test_blocks_chunks_and_ranges(D, fused, rows, heads):
+    _run(D, rows, heads, fused, peaked=True, packed=(rows == 3))
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_appends_of_several_copies_are_one_launch(D):
+    """Token budgets whose ring wraps inside a scale, a scale cut by its own roll, one larger than the budget."""
+    _run(D, 2, 3, True, budgets=[(70, 5), (40, 0), (130, 20)])
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_never_stored_last_scale(D):
+    _run(D, 2, 3, True, flags=B.FLAG_TRANSIENT_LAST_SCALE)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("budgets", [None, [(70, 5), (40, 0), (130, 20)]], ids=["scales", "tokens"])
+def test_densities(D, budgets):
+    _run(D, 2, 3, False, budgets=budgets, density=True, peaked=True)
+
+
+def test_item_counts_on_both_sides_of_the_line():
+    """The same scale served by this kernel and, with more items, by the paired one."""
+    sides, D, heads = (4, 5, 6), 64, 30
+    for rows in (2, 13, 17, 60):
+        qkv = make_qkv(rows, heads, sides, D, seed=92)
+        with Cache(1, heads, D, rows, sides, [(1, 2, False)]) as c:
+            for k, (q, kk, v) in enumerate(qkv):
+                out = torch.full_like(q, float("nan"))
+                B.amskv_append_attend(c.h, 0, k, kk, v, q, out)
+                pick = [0, rows * heads // 2, rows * heads - 1]
+                got = out.reshape(rows * heads, -1, D)[pick].cpu().double().numpy()
+                items = [x.reshape(rows * heads, -1, D)[pick].cpu().double().numpy() for t in qkv[: k + 1] for x in t]
+                keep = oracle.keep_set(k, 1, 2, False)
+                want = oracle.attend_selected(items[3 * k], items[1::3], items[2::3], keep, 0.125)
+                check_close(torch.from_numpy(got), want, "rows %d scale %d" % (rows, k))
+            assert B.amskv_status(c.h) == 0

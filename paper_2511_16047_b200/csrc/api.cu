@@ -192,11 +192,12 @@ void note_appended(amskv_cache* cache, int layer, int scale)
 
 // which kernel amskv_attend uses for T query tokens over `total` keys
 enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
-AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false)
+// (copies: the call includes an append of several copies, which only the warp-matrix kernel takes in)
+AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool copies = false)
 {
     // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained)
     if (cache->path == AMSKV_PATH_AUTO && T > 1 && cache->tc_ready &&
-        mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density))
+        mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density, copies))
         return AttendKernel::Mid;
     // AUTO: the warp-per-item kernel wherever a scale's retained keys fit its register tile, the paired
     // tcgen05 kernel elsewhere (the CUDA-core kernel only where tensor maps are unavailable)
@@ -466,7 +467,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
     Piece piece[LayerLayout::kMaxPieces];
     const int32_t n_pieces = lay.pieces(cache->tokens, scale, piece);
     const bool one_copy = n_pieces == 1 && piece[0].src == 0 && piece[0].len == T;
-    AttendKernel kernel = choose_kernel(cache, T, after.total);
+    AttendKernel kernel = choose_kernel(cache, T, after.total, false, !one_copy);
     // a single-token scale that is its own only key (the first scale): out = V, one copy kernel does both calls
     if (cache->path == AMSKV_PATH_AUTO && T == 1 && after.total == 1) kernel = AttendKernel::Small;
     if (kernel == AttendKernel::Small && one_copy) {
@@ -526,13 +527,14 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
     if (fused && cache->path == AMSKV_PATH_AUTO) {
         // Taking the scale from the caller's tensors splits it off the range it would be part of in the
         // cache; where that adds a tile, attention loses more than the saved copy is worth (measured), so
-        // such scales run as the two calls (AMSKV_PATH_TENSOR_PAIR fuses wherever it can).
+        // such scales run as the two calls (AMSKV_PATH_TENSOR_PAIR fuses wherever it can).  Not where the kernel has an SM
+        // for every query tile: there another key tile is 0.8 us, the copy 2.
         auto tiles = [](const RangeList& rl) {
             int32_t n = 0;
             for (int i = 0; i < rl.n; ++i) n += (rl.r[i].len + 63) / 64;
             return n;
         };
-        if (tiles(ranges) + (T + 63) / 64 > tiles(after)) fused = false;
+        if (tiles(ranges) + (T + 63) / 64 > tiles(after) && !pair_one_tile_per_sm(cache->items(), T, cache->sm_count)) fused = false;
         // Well below a full key tile per scale the units are so short that the kernel is bound by the latency of
         // its loads; holding a stage until it has been written out costs as much there as the copy (measured:
         // equal at T = 36, where fusing at least saves the launch and the second read; a loss at T = 25).

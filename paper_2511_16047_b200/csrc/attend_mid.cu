@@ -504,23 +504,30 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 
 }  // namespace
 
-// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.  64 channels: 19 units.
-// Below it the paired kernel (and, where the append cannot be fused into that, the copy before it) costs 6 to 14 us
-// whatever the size; above it the warp-level matrix instructions, a quarter of the tensor pipe's rate, are what the call
-// takes.  us per call, this kernel / the paired one, append included, in a graph: T = 25: 3.9 / 8.9 (60 items), 6.4 / 11.2
-// (512), 11.5 / 14.9 (1 024), 19.7 / 19.8 (1 920); T = 36: 4.7 / 6.6 (60), 6.4 / 7.9 (256), 12.9 / 9.0 (512); T = 64: 5.1 / 7.4
-// (60), 8.9 / 9.6 (256), 15.7 / 11.2 (512); T = 100: 7.2 / 10.0 (60), 9.2 / 10.8 (128), 16.1 / 12.4 (256); T = 169: 8.5 / 9.9 (32),
-// 11.3 / 10.4 (60).  128 channels: 6 units: T = 36: 5.2 / 10.2 (32), 6.2 / 10.8 (128), 20.5 / 17.1 (512); T = 64: 6.5 / 7.2 (32),
-// 8.7 / 8.5 (128); T = 144: 10.5 / 9.2 (32).  With the density the paired kernel's tiles are cut at the runs and the line lies
-// higher (T = 25, 36, 64 at 512 items: 13.4 / 19.7, 21.1 / 23.2, 26.7 / 26.3; 128 channels, T = 64, 128 items: 15.4 / 20.2), and up to 16
-// queries the alternative is the attention call plus the CUDA-core density pass (T = 4, 9, 16 at 512 items: 12.5 / 16.6,
-// 13.5 / 23.6, 13.0 / 35.0): always this one.  Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).
-bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density)
+// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.
+// 64 channels: 19 units.  Below it the paired kernel (and, where the append cannot be fused into that, the copy before it)
+// costs 6 to 14 us whatever the size; above it the warp-level matrix instructions, a quarter of the tensor pipe's rate, are
+// what the call takes.  us per call, this kernel / the paired one, append included, in a graph: T = 25: 3.9 / 8.9 (60 items),
+// 6.4 / 11.2 (512), 11.5 / 14.9 (1 024), 19.7 / 19.8 (1 920); T = 36: 4.7 / 6.6 (60), 6.4 / 7.9 (256), 12.9 / 9.0 (512); T = 64: 8.9 /
+// 9.6 (256), 15.7 / 11.2 (512); T = 100: 16.1 / 12.4 (256).  7 units where the paired kernel has an SM for every query tile:
+// T = 64: 5.4 / 5.6 (48), 6.5 / 6.7 (96), 7.4 / 6.9 (120); T = 81: 6.1 / 6.4 (32), 7.6 / 6.7 (60); T = 100: 6.4 / 7.4 (16), 7.4 / 7.5 (32),
+// 8.8 / 7.7 (60); T = 144: 8.2 / 8.5 (16), 10.3 / 8.7 (32).
+// 128 channels: 6 units: T = 36: 5.2 / 10.2 (32), 6.2 / 10.8 (128), 20.5 / 17.1 (512); T = 64: 6.8 / 8.0 (32), 7.0 / 8.9 (64), 10.4 / 10.4
+// (128); none above 64 queries where the paired kernel has an SM for every tile: T = 81: 8.0 / 7.2 (16), 7.9 / 7.5 (32), 9.8 / 8.2 (64).
+// With the density the paired kernel's tiles are cut at the runs and the line lies higher (T = 25, 36, 64 at 512 items: 13.4 /
+// 19.7, 21.1 / 23.2, 26.7 / 26.3; 128 channels, T = 64, 128 items: 15.4 / 20.2), and up to 16 queries the alternative is the
+// attention call plus the CUDA-core density pass (T = 4, 9, 16 at 512 items: 12.5 / 16.6, 13.5 / 23.6, 13.0 / 35.0): always this
+// one.  Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).  An append of several copies (`copies`),
+// 2 us each beside the paired kernel, keeps the first lines.
+bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies)
 {
     if (density && T <= kSmallMaxQueries) return true;
     if (!density && small_supported(T, total_keys)) return false;
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
-    return units <= (int64_t)sm_count * (D == 64 ? (density ? 24 : 19) : (density ? 10 : 6));
+    int line = D == 64 ? 19 : 6;
+    if (density) line = D == 64 ? 24 : 10;
+    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? 7 : (T > 64 ? 0 : 6);
+    return units <= (int64_t)sm_count * line;
 }
 
 cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges, int32_t T,

@@ -25,6 +25,8 @@
 // next query tile as soon as the last S of the current one has landed.
 // Every wait is bounded: a wait that gives up records a status code, all roles wind down,
 // copies in flight are awaited and the tensor memory is freed.
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "sm100_ptx.cuh"
 
@@ -47,8 +49,8 @@ constexpr float kLazySumLimit = 1.8446744e19f;   // 2^64: see the kLazy form of 
 constexpr int kPolyEvery = 6;     // every 6th pair of exponentials goes to the FMA pipe (0: none); swept 2, 3, 4, 6, 8
 
 // kWide: one CTA per SM with two S buffers per stream and an issuing warp per stream (below): the form
-// 128 channels use.  64 channels use the two-CTA form (the wide form is instantiable for them, but lost
-// wherever it was measured).
+// 128 channels use, and 64 channels in launches of at most one unit per SM; with more units 64 channels use the
+// two-CTA form.
 // kDen: the launch also accumulates the attention density (below): two CTAs per SM then run with three
 // key/value stages, the fourth stage's 16 KB holding the per-row sums.
 template <int D, bool kWide, bool kDen = false>
@@ -119,7 +121,8 @@ struct PairPlan {
     int32_t n_items;
     int32_t n_shared;     // = n_items * npi
     int32_t n_pairs;      // n_shared + ceil(n_items * (nqt & 1) / 2)
-    int32_t kind;         // 0: no pair is shared, 1: every pair is, 2: both kinds (so that the common cases test a launch constant)
+    int32_t kind;         // 0: no pair is shared, 1: every pair is, 2: both kinds (so that the common cases test a launch constant),
+                          // 3: a pair is one query tile, stream B absent
 };
 
 // The current scale read from the caller's K/V tensors instead of the cache: the last entry of the
@@ -157,6 +160,8 @@ __device__ __forceinline__ bool pair_is_shared(const PairPlan& pp, int32_t pair)
     return pp.kind == 2 ? pair < pp.n_shared : pp.kind == 1;
 }
 
+// (kSolo: the kernel form knows pairs of one query tile, kind 3)
+template <bool kSolo>
 __device__ __forceinline__ Stream stream_of(const PairPlan& pp, int32_t pair, int g)
 {
     Stream s;
@@ -164,6 +169,10 @@ __device__ __forceinline__ Stream stream_of(const PairPlan& pp, int32_t pair, in
         s.item = pp.npi == 1 ? pair : pair / pp.npi;
         s.qt = 2 * (pair - s.item * pp.npi) + g;
         s.valid = true;
+    } else if (kSolo && pp.kind == 3) {
+        s.item = pp.nqt == 1 ? pair : pair / pp.nqt;
+        s.qt = pair - s.item * pp.nqt;
+        s.valid = g == 0;
     } else {
         s.item = 2 * (pair - pp.n_shared) + g;
         s.qt = pp.nqt - 1;
@@ -350,11 +359,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         };
         for (uint32_t n = 0; ok && n < my_pairs; ++n) {
             const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
-            const Stream sa = stream_of(pp, pair, 0), sb = stream_of(pp, pair, 1);
+            const Stream sa = stream_of<kWide>(pp, pair, 0), sb = stream_of<kWide>(pp, pair, 1);
             const bool shared = pair_is_shared(pp, pair);
             const int per_tile = (!shared && sb.valid) ? 2 : 1;
             // one unit per item writes the item's tiles: the unit of its first query tiles
-            const bool unit_stores = storing && (shared ? sa.qt == 0 : pp.nqt == 1);
+            const bool unit_stores = storing && (shared || (kWide && pp.kind == 3) ? sa.qt == 0 : pp.nqt == 1);
             for (int j = 0; ok && j < n_tiles; ++j) {
                 int32_t t0, valid;
                 tile_of(j, t0, valid);
@@ -552,7 +561,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 
             for (uint32_t n = 0; ok && n < my_pairs; ++n) {
                 const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
-                const int ng = stream_of(pp, pair, 1).valid ? 2 : 1;
+                const int ng = stream_of<kWide>(pp, pair, 1).valid ? 2 : 1;
                 const bool shared = pair_is_shared(pp, pair);
                 for (int j = 0; ok && j < n_tiles; ++j) {
                     int32_t t0, valid;
@@ -592,7 +601,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         // overwrites its P.  Two buffers: this S goes first and runs on the tensor pipe while
                         // the softmax of the previous tile finishes (streams with tiles of their own keep the
                         // first order: they need their key/value stages back sooner).
-                        const bool s_first = C::kSBufs == 2 && shared;
+                        const bool s_first = C::kSBufs == 2 && (shared || pp.kind == 3);
                         if (!s_first && pv_live[g] && !issue_pv(g)) { ok = false; continue; }
                         tc_fence_after();
                         const uint32_t t_now = tcount[g];
@@ -651,7 +660,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         auto load_next_q = [&]() {
             for (; q_next_n < my_pairs; ++q_next_n) {
                 const int32_t pair = (int32_t)(blockIdx.x + q_next_n * gridDim.x);
-                const Stream s = stream_of(pp, pair, g);
+                const Stream s = stream_of<kWide>(pp, pair, g);
                 if (!s.valid) continue;
                 const int32_t row = s.item / heads, head = s.item - row * heads;
                 const int32_t valid_rows = min(kQRows, T - s.qt * kQRows);
@@ -684,7 +693,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         bool ok = true;
         for (uint32_t n = 0; ok && n < my_pairs; ++n) {
             const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
-            const Stream st = stream_of(pp, pair, g);
+            const Stream st = stream_of<kWide>(pp, pair, g);
             if (!st.valid) continue;
             const int32_t valid_rows = min(kQRows, T - st.qt * kQRows);
             const bool warp_live = wq * 32 < valid_rows;
@@ -790,11 +799,15 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                     // P V is issued for as many 16-token steps): the columns behind them keep stale bits.
                     int groups = kKT / 16;
                     if (valid < kKT) groups = ((valid + 15) >> 4) + ((kExt && ext.rider_valid > 0 && j == n_tiles - 1) ? 1 : 0);
-                    auto exp_tile = [&]() -> float {
+                    // (`whole`: all four groups as one straight piece of code, whose instructions overlap from group to group; 64
+                    // channels in the wide form only, where a warp has its scheduler nearly to itself: 1 000 -> 860 clocks a
+                    // tile; 3 to 12 % slower elsewhere)
+                    constexpr bool kStraight = kWide && D == 64;
+                    auto exp_tile = [&](auto whole) -> float {
                         float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
                         for (int grp = 0; grp < kKT / 16; ++grp) {
-                            if (grp < groups) {   // (the same for the whole warp)
+                            if (decltype(whole)::value || grp < groups) {   // (the same for the whole warp)
                                 uint32_t pk[8];
 #pragma unroll
                                 for (int ii = 0; ii < 8; ++ii) {
@@ -819,7 +832,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         }
                         return sum0 + sum1;
                     };
-                    float tile_sum = exp_tile();
+                    float tile_sum = kStraight && groups == kKT / 16 ? exp_tile(std::bool_constant<kStraight>{}) : exp_tile(std::false_type{});
                     if (kLazy && j > 0) {
                         // No maximum was taken for this tile: its exponentials were formed against the row's reference
                         // as it stood (the maximum of the unit's first tile, or of the last tile that was redone).
@@ -836,7 +849,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                 ok = false;
                                 break;
                             }
-                            tile_sum = exp_tile();
+                            tile_sum = exp_tile(std::false_type{});
                         }
                     }
                     l += tile_sum;
@@ -1004,12 +1017,23 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     pp.n_shared = (int32_t)n_shared;
     pp.n_pairs = (int32_t)n_pairs;
     pp.kind = pp.npi == 0 ? 0 : ((pp.nqt & 1) ? 2 : 1);
+    // When every query tile of the launch can have an SM of its own, it gets one: what such a call takes is a stream's serial
+    // chain, and two streams on the same SM sub-partitions lengthen it (64 channels 2 090 -> 1 500 clocks a key tile with
+    // the form below; the second fetch of K and V comes from L2).  us per call, before / after: 64 channels, 60 items: T = 100
+    // 10.1 / 7.7, T = 169 11.1 / 9.6, T = 256 14.2 / 11.7; 32 items, T = 256 13.2 / 10.9; 128 channels, 32 items: T = 144 12.9 /
+    // 10.3, T = 256 14.5 / 12.3, T = 400 23.6 / 20.7; 16 items, T = 576 35.3 / 22.6.  With more tiles than SMs the pairs win (128
+    // channels, 32 items, T = 576, 160 tiles: 38.3 / 40.9).
+    if (!density && pair_one_tile_per_sm(pp.n_items, T, sm_count)) {
+        pp.kind = 3;
+        pp.n_shared = 0;
+        pp.n_pairs = pp.n_items * pp.nqt;
+    }
     int32_t n_tiles = 0;
     for (int i = 0; i < ranges.n; ++i) n_tiles += (ranges.r[i].len + kKT - 1) / kKT;
     const int3 qpos = make_int3(pos[0], pos[1], pos[2]);
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
-    // 64 channels always take the two-CTA form: the wide form was measured on the tensor-bound launches of a
-    // 2 240-token schedule (T = 576 and 1 024, 36 heads) and lost there too (26.3 vs 20.8 and 64.2 vs 53.9 ms):
+    // 64 channels take the two-CTA form once there are units for it: the wide form was measured on the tensor-bound launches
+    // of a 2 240-token schedule (T = 576 and 1 024, 36 heads, 64 rows) and lost there too (26.3 vs 20.8 and 64.2 vs 53.9 ms):
     // two streams per SM do not keep the tensor pipe as busy as four, even with the chain broken.
 #define AMSKV_PAIR_LAUNCH(DD, EXT, WIDE, DEN, LAZY, SHORT)                                                          \
     return launch<DD, EXT, WIDE, DEN, LAZY, SHORT>(qm, km, vm, km64, vm64, ext, O, ranges, T, heads, pp, n_tiles, qpos,  \
@@ -1031,6 +1055,14 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
         AMSKV_PAIR_LAUNCH(128, false, true, false, false, false);
     }
     if (density) AMSKV_PAIR_LAUNCH(64, false, false, true, false, false);
+    // A launch of at most one unit per SM takes the wide form: nobody shares the SM, so the second S buffer, which takes S of
+    // the next tile off the chain, costs no parallelism (T = 256, 60 items 13.8 -> 12.8 us, 128 items 15.2 -> 14.6; T = 1 024, 36
+    // items, 144 units 37.9 -> 33.4; with 256 units 21.0 -> 24.3).  Not for launches of both kinds of pairs (T = 576, 36 items:
+    // 23.6 -> 24.7).
+    if (pp.n_pairs <= sm_count && pp.kind != 2) {
+        if (cur) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true);
+        AMSKV_PAIR_LAUNCH(64, false, true, false, true, true);
+    }
     if (n_tiles > short_max) {
         if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, true, false);
         AMSKV_PAIR_LAUNCH(64, false, false, false, true, false);

@@ -10,7 +10,7 @@ import torch
 import oracle
 from paper_2511_16047_b200 import binding as B
 
-from gpu_common import Cache, check_close, make_qkv, to_items
+from gpu_common import Cache, check_close, make_qkv, oracle_outputs, run_pass, to_items
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +93,24 @@ def test_item_counts_on_both_sides_of_the_line():
                 want = oracle.attend_selected(items[3 * k], items[1::3], items[2::3], keep, 0.125)
                 check_close(torch.from_numpy(got), want, "rows %d scale %d" % (rows, k))
             assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("path", [B.PATH_AUTO, B.PATH_TENSOR_PAIR], ids=["auto", "pair"])
+@pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
+def test_one_query_tile_per_sm(D, path, fused):
+    """The paired kernel with a query tile per CTA (as many tiles as SMs, 148, at the most): one to three tiles per item with
+    full and ragged last ones, up to nine key tiles, fused writes from the CTA of an item's first tile; and the launches
+    with one tile too many for it, which take pairs again."""
+    sides = (4, 8, 11, 13, 17)                                 # T = 16, 64, 121, 169 (two tiles), 289 (three)
+    pols = [(1, 2, False), (0, 9, True)]
+    for rows, heads in ((1, 3), (7, 7), (1, 74), (3, 25)):     # 49 x 3 = 147, 74 x 2 = 148, 75 x 2 = 150 tiles
+        qkv = make_qkv(rows, heads, sides, D, seed=93, peaked=(rows == 7))
+        with Cache(len(pols), heads, D, rows, sides, pols) as c:
+            outs = run_pass(c, qkv, path, fused=fused)
+            for layer, pol in enumerate(pols):
+                items = sorted({0, rows * heads // 2, rows * heads - 1})
+                want = oracle_outputs(qkv, pol, 1.0 / math.sqrt(D), items=items)
+                for k in range(len(sides)):
+                    got = outs[layer][k].reshape(rows * heads, -1, D)[items].cpu().double()
+                    check_close(got, want[k], "%d items layer %d scale %d" % (rows * heads, layer, k), max_abs=4e-2 if rows == 7 else 1e-2)

@@ -498,7 +498,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         note_appended(cache, layer, scale);
         return AMSKV_OK;
     }
-    bool fused = cache->tc_ready && kernel == AttendKernel::Pair && one_copy;
+    bool fused = cache->tc_ready && kernel == AttendKernel::Pair;
     if (fused) {
         ranges.n = lay.ranges_before(cache->tokens, scale, ranges.r);
         if (ranges.n >= kMaxRanges) fused = false;
@@ -528,13 +528,15 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         // Taking the scale from the caller's tensors splits it off the range it would be part of in the
         // cache; where that adds a tile, attention loses more than the saved copy is worth (measured), so
         // such scales run as the two calls (AMSKV_PATH_TENSOR_PAIR fuses wherever it can).  Not where the kernel has an SM
-        // for every query tile: there another key tile is 0.8 us, the copy 2.
+        // for every query tile: there another key tile is 0.8 us, the copy 2.  Above 128 queries one more tile is less than
+        // the several copies of an append whose ring wraps (1 920 items, three such layers of ten: T = 256 1 046 -> 1 028 us; T =
+        // 100, seven of ten: 487 -> 554).
         auto tiles = [](const RangeList& rl) {
             int32_t n = 0;
             for (int i = 0; i < rl.n; ++i) n += (rl.r[i].len + 63) / 64;
             return n;
         };
-        if (tiles(ranges) + (T + 63) / 64 > tiles(after) && !pair_one_tile_per_sm(cache->items(), T, cache->sm_count)) fused = false;
+        if (tiles(ranges) + (T + 63) / 64 > tiles(after) + (!one_copy && T > 128 ? 1 : 0) && !pair_one_tile_per_sm(cache->items(), T, cache->sm_count)) fused = false;
         // Well below a full key tile per scale the units are so short that the kernel is bound by the latency of
         // its loads; holding a stage until it has been written out costs as much there as the copy (measured:
         // equal at T = 36, where fusing at least saves the launch and the second read; a loss at T = 25).
@@ -549,6 +551,10 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
     ranges.total = 0;
     for (int i = 0; i < ranges.n; ++i) ranges.total += ranges.r[i].len;
     CurrentScaleSource cur{ks, vs, true, piece[0].dst, cache->region(layer)};
+    if (!one_copy) {
+        cur.piece = piece;
+        cur.n_pieces = n_pieces;
+    }
     cur.rider_tok = rider_tok;
     cur.rider_valid = rider_valid;
     cudaError_t e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes,

@@ -136,6 +136,10 @@ struct ExtArgs {
     int32_t store;
     int32_t dst;                      // first position of the scale in the per-item region
     int3 pos;                         // coordinate slots of token, head and row in the rank-4 maps
+    __nv_bfloat16* region;            // the layer's region, for rows written one by one
+    int32_t capacity;
+    int32_t n_pieces, last_piece;     // kPieces form: the scale's place is several pieces (a ring that wraps inside it, say);
+    Piece piece[LayerLayout::kMaxPieces];   // last_piece holds its last token, and the store maps end where that piece does
     int32_t rider_tok, rider_valid;   // older cache tokens that ride in the spare box of the scale's last tile
 };
 
@@ -202,7 +206,7 @@ __device__ __forceinline__ void tile_at(const RangeList& rl, int j, int32_t& t0,
 }
 
 // ---------------------------------------------------------------- kernel
-template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort>
+template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces>
 __global__ void __launch_bounds__(Cfg<D, kWide, kDen>::kThreads, Cfg<D, kWide, kDen>::kCtasPerSm)
 attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                    const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap k_map64,
@@ -343,8 +347,37 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         auto store_front = [&]() -> bool {
             const uint32_t stage = st_sq[0] % C::kStages, use = st_sq[0] / C::kStages;
             if (!warp_wait(kv_full0 + 8 * stage, use & 1u, abort_flag)) return false;
-            if (lane == 0) {
-                const uint32_t k_src = kv_smem + stage * C::kStageBytes, v_src = k_src + C::kKVBytes;
+            const uint32_t k_src = kv_smem + stage * C::kStageBytes, v_src = k_src + C::kKVBytes;
+            if constexpr (kPieces) {
+                // Of every piece the tile's share: with one bulk store where it is the whole tile (up to the end of the scale,
+                // where the map clips the box), else row by row (a box that starts or ends inside the tile cannot be told
+                // to the copy engine: the swizzle wants it to start on eight rows, and a clipped start is not allowed).
+                const int32_t first = st_tok[0], end = min(first + kKT, T);
+                for (int i = 0; i < ext.n_pieces; ++i) {
+                    const int32_t lo = max(first, ext.piece[i].src), hi = min(end, ext.piece[i].src + ext.piece[i].len);
+                    if (lo >= hi) continue;
+                    const int32_t dst = ext.piece[i].dst + lo - ext.piece[i].src;
+                    if (lo == first && (hi - lo == kKT || (hi == T && i == ext.last_piece))) {
+                        if (lane == 0) {
+#pragma unroll
+                            for (int h = 0; h < C::kHalves; ++h) {
+                                tma_store_3d(hi - lo < kKT ? &ext.k_store : &k_map64, k_src + h * C::kKVHalfBytes, h * 64, dst, st_item[0]);
+                                tma_store_3d(hi - lo < kKT ? &ext.v_store : &v_map64, v_src + h * C::kKVHalfBytes, h * 64, dst, st_item[0]);
+                            }
+                        }
+                    } else {
+                        const uint8_t* tile = smem_raw + (k_src - raw);
+                        uint4* kd = reinterpret_cast<uint4*>(ext.region + ((int64_t)st_item[0] * 2 * ext.capacity + dst) * D);
+                        for (int32_t c = lane; c < (hi - lo) * (D / 8); c += 32) {
+                            const int32_t r = c / (D / 8), p = c % (D / 8), row = lo - first + r;
+                            const uint32_t off = (uint32_t)((p >> 3) * C::kKVHalfBytes + row * 128 + (((p & 7) ^ (row & 7)) << 4));
+                            kd[(int64_t)r * (D / 8) + p] = *reinterpret_cast<const uint4*>(tile + off);
+                            kd[((int64_t)r + ext.capacity) * (D / 8) + p] = *reinterpret_cast<const uint4*>(tile + C::kKVBytes + off);
+                        }
+                    }
+                }
+                __syncwarp();
+            } else if (lane == 0) {
 #pragma unroll
                 for (int h = 0; h < C::kHalves; ++h) {
                     tma_store_3d(&ext.k_store, k_src + h * C::kKVHalfBytes, h * 64, ext.dst + st_tok[0], st_item[0]);
@@ -933,7 +966,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 }
 
 // ---------------------------------------------------------------- host side
-template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort>
+template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces>
 cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorMap& vm, const CUtensorMap& km64,
                    const CUtensorMap& vm64, const ExtArgs& ext, const Strided& O,
                    const RangeList& ranges, int32_t T, int32_t heads, const PairPlan& pp, int32_t n_tiles, int3 qpos,
@@ -941,11 +974,11 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
 {
     using C = Cfg<D, kWide, kDen>;
     static SharedMemoryOptIn opt_in;
-    const cudaError_t oe = opt_in.ensure(attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort>, (int)C::kSmemBytes);
+    const cudaError_t oe = opt_in.ensure(attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces>, (int)C::kSmemBytes);
     if (oe != cudaSuccess) return oe;
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
     if (grid > pp.n_pairs) grid = pp.n_pairs;
-    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort>, dim3((unsigned)grid), dim3(C::kThreads),
+    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces>, dim3((unsigned)grid), dim3(C::kThreads),
                          C::kSmemBytes, stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
                          ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);
 }
@@ -994,8 +1027,24 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
             ext.rider_tok = cur->rider_tok;
             ext.rider_valid = cur->rider_valid;
         }
+        int32_t place_end = cur->dst + T;
+        if (cur->n_pieces > 0) {
+            if (cur->n_pieces > LayerLayout::kMaxPieces || !cur->store) return cudaErrorInvalidValue;
+            ext.region = cur->region.base;
+            ext.capacity = cur->region.capacity;
+            ext.n_pieces = cur->n_pieces;
+            ext.last_piece = -1;
+            for (int i = 0; i < cur->n_pieces; ++i) {
+                ext.piece[i] = cur->piece[i];
+                if (cur->piece[i].src + cur->piece[i].len == T) {
+                    ext.last_piece = i;   // (the last of them, should there be two)
+                    place_end = cur->piece[i].dst + cur->piece[i].len;
+                }
+            }
+            if (ext.last_piece < 0) place_end = cur->region.capacity;   // (no piece ends the scale: the maps are not used)
+        }
         if (cur->store &&
-            !tc_encode_kv_store_maps(cur->region, (int64_t)rows * heads, D, kKT, cur->dst + T, &ext.k_store, &ext.v_store))
+            !tc_encode_kv_store_maps(cur->region, (int64_t)rows * heads, D, kKT, place_end, &ext.k_store, &ext.v_store))
             return cudaErrorNotSupported;
     }
     CUtensorMap qm;
@@ -1035,8 +1084,8 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // 64 channels take the two-CTA form once there are units for it: the wide form was measured on the tensor-bound launches
     // of a 2 240-token schedule (T = 576 and 1 024, 36 heads, 64 rows) and lost there too (26.3 vs 20.8 and 64.2 vs 53.9 ms):
     // two streams per SM do not keep the tensor pipe as busy as four, even with the chain broken.
-#define AMSKV_PAIR_LAUNCH(DD, EXT, WIDE, DEN, LAZY, SHORT)                                                          \
-    return launch<DD, EXT, WIDE, DEN, LAZY, SHORT>(qm, km, vm, km64, vm64, ext, O, ranges, T, heads, pp, n_tiles, qpos,  \
+#define AMSKV_PAIR_LAUNCH(DD, EXT, WIDE, DEN, LAZY, SHORT, ...)                                                     \
+    return launch<DD, EXT, WIDE, DEN, LAZY, SHORT, __VA_ARGS__>(qm, km, vm, km64, vm64, ext, O, ranges, T, heads, pp, n_tiles, qpos,  \
                                                    scale_log2, status, sm_count, stream, den)
     // Launches of three key tiles or more take the row maximum of a unit's first tile only (the kLazy form of the
     // softmax loop: 1.7 % of a 256x256-shaped pass, 6 % of a 1024x1024-shaped one); with fewer tiles there is next
@@ -1044,35 +1093,40 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // channels) have a producer that issues a tile's bulk copies from several lanes at once and fetches a partly
     // filled tile of the caller's tensors as one box; the long launches keep the one-lane producer (its smaller code
     // measured 2 % faster there).
+    // Writes in several pieces are instantiated for the lazy form only.
     constexpr int lazy_min = 3, lazy128_min = 3, short_max = 4;
     if (D == 128) {
-        if (density) AMSKV_PAIR_LAUNCH(128, false, true, true, false, false);
-        if (n_tiles >= lazy128_min) {
-            if (cur) AMSKV_PAIR_LAUNCH(128, true, true, false, true, false);
-            AMSKV_PAIR_LAUNCH(128, false, true, false, true, false);
+        if (density) AMSKV_PAIR_LAUNCH(128, false, true, true, false, false, false);
+        if (n_tiles >= lazy128_min || ext.n_pieces > 0) {
+            if (ext.n_pieces > 0) AMSKV_PAIR_LAUNCH(128, true, true, false, true, false, true);
+            if (cur) AMSKV_PAIR_LAUNCH(128, true, true, false, true, false, false);
+            AMSKV_PAIR_LAUNCH(128, false, true, false, true, false, false);
         }
-        if (cur) AMSKV_PAIR_LAUNCH(128, true, true, false, false, false);
-        AMSKV_PAIR_LAUNCH(128, false, true, false, false, false);
+        if (cur) AMSKV_PAIR_LAUNCH(128, true, true, false, false, false, false);
+        AMSKV_PAIR_LAUNCH(128, false, true, false, false, false, false);
     }
-    if (density) AMSKV_PAIR_LAUNCH(64, false, false, true, false, false);
+    if (density) AMSKV_PAIR_LAUNCH(64, false, false, true, false, false, false);
     // A launch of at most one unit per SM takes the wide form: nobody shares the SM, so the second S buffer, which takes S of
     // the next tile off the chain, costs no parallelism (T = 256, 60 items 13.8 -> 12.8 us, 128 items 15.2 -> 14.6; T = 1 024, 36
     // items, 144 units 37.9 -> 33.4; with 256 units 21.0 -> 24.3).  Not for launches of both kinds of pairs (T = 576, 36 items:
     // 23.6 -> 24.7).
     if (pp.n_pairs <= sm_count && pp.kind != 2) {
-        if (cur) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true);
-        AMSKV_PAIR_LAUNCH(64, false, true, false, true, true);
+        if (ext.n_pieces > 0) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true, true);
+        if (cur) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true, false);
+        AMSKV_PAIR_LAUNCH(64, false, true, false, true, true, false);
     }
     if (n_tiles > short_max) {
-        if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, true, false);
-        AMSKV_PAIR_LAUNCH(64, false, false, false, true, false);
+        if (ext.n_pieces > 0) AMSKV_PAIR_LAUNCH(64, true, false, false, true, false, true);
+        if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, true, false, false);
+        AMSKV_PAIR_LAUNCH(64, false, false, false, true, false, false);
     }
-    if (n_tiles >= lazy_min) {
-        if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, true, true);
-        AMSKV_PAIR_LAUNCH(64, false, false, false, true, true);
+    if (n_tiles >= lazy_min || ext.n_pieces > 0) {
+        if (ext.n_pieces > 0) AMSKV_PAIR_LAUNCH(64, true, false, false, true, true, true);
+        if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, true, true, false);
+        AMSKV_PAIR_LAUNCH(64, false, false, false, true, true, false);
     }
-    if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, false, true);
-    AMSKV_PAIR_LAUNCH(64, false, false, false, false, true);
+    if (cur) AMSKV_PAIR_LAUNCH(64, true, false, false, false, true, false);
+    AMSKV_PAIR_LAUNCH(64, false, false, false, false, true, false);
 #undef AMSKV_PAIR_LAUNCH
 }
 

@@ -58,6 +58,8 @@ struct CurrentScaleSource {
     int32_t dst;
     LayerRegion region;
     int32_t rider_tok = 0, rider_valid = 0;
+    const Piece* piece = nullptr;   // the place is `n_pieces` pieces instead of T tokens from `dst` (the paired kernel)
+    int32_t n_pieces = 0;
 };
 
 // (the CUDA-core kernel takes a current-scale source without `store` only)

@@ -114,3 +114,30 @@ def test_one_query_tile_per_sm(D, path, fused):
                 for k in range(len(sides)):
                     got = outs[layer][k].reshape(rows * heads, -1, D)[items].cpu().double()
                     check_close(got, want[k], "%d items layer %d scale %d" % (rows * heads, layer, k), max_abs=4e-2 if rows == 7 else 1e-2)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_paired_kernel_writes_an_append_in_pieces(D):
+    """Token budgets under the paired kernel: rings that wrap inside a key tile, a head and a ring filled by the same scale,
+    scales cut by their own roll, pieces that end inside the last tile.  One launch each; every output of every later scale
+    depends on what was written."""
+    sides = (2, 8, 8, 9, 11, 8, 13, 12)
+    budgets = [(133, 5), (128, 64), (200, 70), (150, 0), (64, 64)]
+    pols = [(1, 1, False)] * len(budgets)
+    rows, heads = 2, 3
+    qkv = make_qkv(rows, heads, sides, D, seed=94)
+    Ks, Vs = [to_items(k) for _, k, _ in qkv], [to_items(v) for _, _, v in qkv]
+    copies = set()
+    with Cache(len(pols), heads, D, rows, sides, pols, token_budgets=budgets) as c:
+        B.amskv_set_attend_path(c.h, B.PATH_TENSOR_PAIR)
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(pols)):
+                out = torch.full_like(q, float("nan"))
+                n0 = B.amskv_launch_count()
+                B.amskv_append_attend(c.h, layer, k, kk, v, q, out)
+                assert B.amskv_launch_count() - n0 == 1
+                copies.add(len(B.amskv_append_copies(c.h, layer, k)))
+                tokens = [(s, t) for s, first, count in B.amskv_attended_tokens(c.h, layer, k) for t in range(first, first + count)]
+                check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, 1.0 / math.sqrt(D)), "layer %d scale %d" % (layer, k))
+        assert B.amskv_status(c.h) == 0
+    assert copies == {1, 2, 3}

@@ -12,6 +12,8 @@
 //   warp 8       TMA producer of the key/value tiles (ring of stages, 16 tokens per bulk copy so a
 //                range's tail tile reads only the 16-token groups it needs)
 //   warp 9       issues tcgen05.mma for both streams, alternating between them
+// In the split form two CTAs (a cluster) share the key tiles of each pair of a launch's last round and merge O, references and
+// sums through distributed shared memory.
 // Per stream and tile: S = Q K^T (128 x 64 fp32 in TMEM) -> the group reads S with tcgen05.ld,
 // exponentiates in exp2 form against a reference maximum, packs P to bf16 and writes it back
 // over S with tcgen05.st -> O += P V with P read from TMEM.  S and P share their columns, so
@@ -121,6 +123,7 @@ struct PairPlan {
     int32_t n_items;
     int32_t n_shared;     // = n_items * npi
     int32_t n_pairs;      // n_shared + ceil(n_items * (nqt & 1) / 2)
+    int32_t full;         // kSplit form: whole pairs per CTA; the pairs left over are shared by clusters of two CTAs
     int32_t kind;         // 0: no pair is shared, 1: every pair is, 2: both kinds (so that the common cases test a launch constant),
                           // 3: a pair is one query tile, stream B absent
 };
@@ -206,7 +209,7 @@ __device__ __forceinline__ void tile_at(const RangeList& rl, int j, int32_t& t0,
 }
 
 // ---------------------------------------------------------------- kernel
-template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces>
+template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces, bool kSplit>
 __global__ void __launch_bounds__(Cfg<D, kWide, kDen>::kThreads, Cfg<D, kWide, kDen>::kCtasPerSm)
 attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                    const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap k_map64,
@@ -311,8 +314,19 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     const uint32_t o_full0 = smem_u32(&bars->o_full[0]);
     const uint32_t kv_full0 = smem_u32(&bars->kv_full[0]), kv_empty0 = smem_u32(&bars->kv_empty[0]);
 
-    // pairs of this CTA: p = blockIdx.x + n * gridDim.x, n = 0 .. my_pairs-1
-    const uint32_t my_pairs = (int32_t)blockIdx.x < pp.n_pairs ? ((uint32_t)pp.n_pairs - 1u - blockIdx.x) / gridDim.x + 1u : 0u;
+    // pairs of this CTA: p = blockIdx.x + n * gridDim.x, n = 0 .. my_pairs-1.  In the split form that gives every CTA pp.full
+    // pairs, and of the pairs left over each cluster of two CTAs takes one, its CTAs one half of the key tiles each.
+    const uint32_t rank = kSplit ? cluster_rank() : 0u;
+    const int32_t split_pair = kSplit ? pp.full * (int32_t)gridDim.x + (int32_t)(blockIdx.x >> 1) : 0;
+    const bool has_split = kSplit && split_pair < pp.n_pairs;
+    const uint32_t my_pairs = kSplit ? (uint32_t)pp.full + (has_split ? 1u : 0u)
+                                     : ((int32_t)blockIdx.x < pp.n_pairs ? ((uint32_t)pp.n_pairs - 1u - blockIdx.x) / gridDim.x + 1u : 0u);
+    auto pair_at = [&](uint32_t n) -> int32_t {
+        return kSplit && n == (uint32_t)pp.full ? split_pair : (int32_t)(blockIdx.x + n * gridDim.x);
+    };
+    auto tiles_begin = [&](uint32_t n) -> int { return kSplit && n == (uint32_t)pp.full && rank == 1u ? n_tiles / 2 : 0; };
+    auto tiles_end = [&](uint32_t n) -> int { return kSplit && n == (uint32_t)pp.full && rank == 0u ? n_tiles / 2 : n_tiles; };
+    float m_ref = 0.f, l = 0.f;   // softmax warps: a row's reference maximum and sum
 
     // The producer and the MMA issuer run their loops with the whole warp converged and let one
     // elected lane issue: addresses, descriptors and coordinates then stay warp-uniform values,
@@ -391,13 +405,14 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             return true;
         };
         for (uint32_t n = 0; ok && n < my_pairs; ++n) {
-            const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
+            const int32_t pair = pair_at(n);
+            const int j_begin = tiles_begin(n), j_end = tiles_end(n);
             const Stream sa = stream_of<kWide>(pp, pair, 0), sb = stream_of<kWide>(pp, pair, 1);
             const bool shared = pair_is_shared(pp, pair);
             const int per_tile = (!shared && sb.valid) ? 2 : 1;
             // one unit per item writes the item's tiles: the unit of its first query tiles
             const bool unit_stores = storing && (shared || (kWide && pp.kind == 3) ? sa.qt == 0 : pp.nqt == 1);
-            for (int j = 0; ok && j < n_tiles; ++j) {
+            for (int j = j_begin; ok && j < j_end; ++j) {
                 int32_t t0, valid;
                 tile_of(j, t0, valid);
                 (void)tile_run(valid);
@@ -593,10 +608,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             };
 
             for (uint32_t n = 0; ok && n < my_pairs; ++n) {
-                const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
+                const int32_t pair = pair_at(n);
+                const int j_begin = tiles_begin(n), j_end = tiles_end(n);
                 const int ng = stream_of<kWide>(pp, pair, 1).valid ? 2 : 1;
                 const bool shared = pair_is_shared(pp, pair);
-                for (int j = 0; ok && j < n_tiles; ++j) {
+                for (int j = j_begin; ok && j < j_end; ++j) {
                     int32_t t0, valid;
                     tile_of(j, t0, valid);
                     (void)tile_run(valid);
@@ -620,7 +636,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         // almost always landed, and this keeps the two waits out of the P -> P V -> S chain.
                         const uint32_t seq = shared ? sq : sq + g;
                         const uint32_t stage = seq % C::kStages, use = seq / C::kStages;
-                        if (j == 0) {
+                        if (j == j_begin) {
                             const uint32_t u = ucount[g];
                             q_half[g] = q_split ? (u & 1u) : 0u;
                             const uint32_t parity = q_split ? ((u >> 1) & 1u) : (u & 1u);
@@ -657,8 +673,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         pv_stage[g] = stage;
                         pv_nch[g] = nch;
                         pv_t[g] = t_now;
-                        pv_first[g] = (j == 0);
-                        pv_last[g] = (j == n_tiles - 1);
+                        pv_first[g] = (j == j_begin);
+                        pv_last[g] = (j == j_end - 1);
                         pv_release[g] = (shared && my_g < 0) ? (g == ng - 1) : true;
                         pv_twice[g] = !shared;
                         ++tcount[g];
@@ -692,7 +708,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         if (kShort && q_loader) prefetch_tensormap(&q_map);
         auto load_next_q = [&]() {
             for (; q_next_n < my_pairs; ++q_next_n) {
-                const int32_t pair = (int32_t)(blockIdx.x + q_next_n * gridDim.x);
+                const int32_t pair = pair_at(q_next_n);
                 const Stream s = stream_of<kWide>(pp, pair, g);
                 if (!s.valid) continue;
                 const int32_t row = s.item / heads, head = s.item - row * heads;
@@ -725,15 +741,18 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         uint32_t un = 0;  // units done by this stream
         bool ok = true;
         for (uint32_t n = 0; ok && n < my_pairs; ++n) {
-            const int32_t pair = (int32_t)(blockIdx.x + n * gridDim.x);
+            const int32_t pair = pair_at(n);
+            const int j_begin = tiles_begin(n), j_end = tiles_end(n);
             const Stream st = stream_of<kWide>(pp, pair, g);
             if (!st.valid) continue;
             const int32_t valid_rows = min(kQRows, T - st.qt * kQRows);
             const bool warp_live = wq * 32 < valid_rows;
-            float m_ref = 0.f, nb = 0.f, l = 0.f;
+            m_ref = 0.f;
+            l = 0.f;
+            float nb = 0.f;
             float run_mass = 0.f;   // density: this row's un-normalised mass on the run the tiles are in
             int cur_run = -1;
-            for (int j = 0; j < n_tiles; ++j, ++t) {
+            for (int j = j_begin; j < j_end; ++j, ++t) {
                 int32_t t0, valid;
                 tile_of(j, t0, valid);
                 const int run = tile_run(valid);
@@ -752,7 +771,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 }
                 tc_fence_after();
                 // the last S of this unit has landed, so its query tile is no longer read
-                if (j == n_tiles - 1 && q_loader) load_next_q();
+                if (j == j_end - 1 && q_loader) load_next_q();
                 if (warp_live) {
                     uint32_t sr[kKT];
                     tmem_ld64(s_tmem, sr);
@@ -815,7 +834,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         }
                         return true;
                     };
-                    if (j == 0) {
+                    if (j == j_begin) {
                         const float mt = row_max();
                         m_ref = mt;
                         nb = -mt * scale_log2;
@@ -866,7 +885,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         return sum0 + sum1;
                     };
                     float tile_sum = kStraight && groups == kKT / 16 ? exp_tile(std::bool_constant<kStraight>{}) : exp_tile(std::false_type{});
-                    if (kLazy && j > 0) {
+                    if (kLazy && j > j_begin) {
                         // No maximum was taken for this tile: its exponentials were formed against the row's reference
                         // as it stood (the maximum of the unit's first tile, or of the last tile that was redone).
                         // That is exact as long as nothing overflows.  A row whose tile sum is beyond the limit (or
@@ -901,6 +920,10 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 break;
             }
             tc_fence_after();
+            if (kSplit && n == (uint32_t)pp.full) {   // (always the last pair) the two CTAs merge their halves below
+                ++un;
+                break;
+            }
             if (warp_live) {
                 const float inv = 1.f / l;
                 const int32_t row = st.item / heads, head = st.item - row * heads;
@@ -956,6 +979,74 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
     }
 
+    if constexpr (kSplit) {
+        if (has_split) {   // (the same for both CTAs of a cluster)
+            // -------------------------------------------------------- merge of the two halves of the pair's keys
+            // Each CTA holds O of both query tiles against its own references and sums, and finishes one half of the
+            // channels: it sends the other CTA its columns of the other half (fp32) with its references and sums, into that
+            // CTA's key/value ring, which nobody reads any more once every role of both CTAs is done (first barrier).  Columns
+            // in groups of four, one row per lane: 16-byte accesses without bank conflicts.
+            constexpr uint32_t W = D / 2, kMl = 2u * W * kQRows * 4u;   // references and sums behind the columns
+            static_assert(kMl + 2u * kQRows * 8u <= C::kStages * C::kStageBytes, "exchange fits the ring");
+            const int g = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
+            const Stream st = g < 2 ? stream_of<kWide>(pp, split_pair, g) : Stream{0, 0, false};
+            const int32_t valid_rows = st.valid ? min(kQRows, T - st.qt * kQRows) : 0;
+            const bool warp_live = wq * 32 < valid_rows;
+            const uint32_t o_tmem = tmem + C::kOCol + g * D + (((uint32_t)(wq * 32)) << 16);
+            auto col_off = [&](uint32_t c4) -> uint32_t { return ((g * (W / 4u) + c4) * kQRows + r) * 16u; };
+            __syncwarp();
+            cluster_sync();
+            if (warp_live) {
+                tc_fence_after();
+                const uint32_t to = map_to_rank(kv_smem, rank ^ 1u);
+#pragma unroll
+                for (uint32_t cb = 0; cb < W; cb += 16) {
+                    uint32_t o[16];
+                    tmem_ld16(o_tmem + (rank ^ 1u) * W + cb, o);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) st_cluster_16B(to + col_off(cb / 4u + i), o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                }
+                st_cluster_8B(to + kMl + (g * kQRows + r) * 8u, m_ref, l);
+            }
+            cluster_sync();
+            if (warp_live) {
+                const uint8_t* ring = smem_raw + (kv_smem - raw);
+                const float2 other = reinterpret_cast<const float2*>(ring + kMl)[g * kQRows + r];
+                const float M = fmaxf(m_ref, other.x);
+                float f_own = fast_exp2((m_ref - M) * scale_log2), f_other = fast_exp2((other.x - M) * scale_log2);
+                const float inv = 1.f / fmaf(l, f_own, other.y * f_other);
+                f_own *= inv;
+                f_other *= inv;
+                const bool o_sectors = ((reinterpret_cast<uintptr_t>(O) | (uintptr_t)(2 * o_row) | (uintptr_t)(2 * o_head) | (uintptr_t)(2 * o_tok)) & 31u) == 0;
+                const int32_t row = st.item / heads, head = st.item - row * heads;
+                __nv_bfloat16* dst = O + row * o_row + head * o_head + (int64_t)(st.qt * kQRows + r) * o_tok + rank * W;
+#pragma unroll
+                for (uint32_t cb = 0; cb < W; cb += 16) {
+                    uint32_t o[16], w[8];
+                    tmem_ld16(o_tmem + rank * W + cb, o);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 x = *reinterpret_cast<const float4*>(ring + col_off(cb / 4u + i));
+                        const __nv_bfloat162 a = __floats2bfloat162_rn(fmaf(x.x, f_other, __uint_as_float(o[4 * i]) * f_own),
+                                                                       fmaf(x.y, f_other, __uint_as_float(o[4 * i + 1]) * f_own));
+                        const __nv_bfloat162 b = __floats2bfloat162_rn(fmaf(x.z, f_other, __uint_as_float(o[4 * i + 2]) * f_own),
+                                                                       fmaf(x.w, f_other, __uint_as_float(o[4 * i + 3]) * f_own));
+                        w[2 * i] = *reinterpret_cast<const uint32_t*>(&a);
+                        w[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&b);
+                    }
+                    if (r < valid_rows) {
+                        if (o_sectors) {
+                            st_global_32B(dst + cb, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+                        } else {
+                            reinterpret_cast<uint4*>(dst + cb)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                            reinterpret_cast<uint4*>(dst + cb)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                        }
+                    }
+                }
+            }
+        }
+    }
+
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
@@ -966,7 +1057,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 }
 
 // ---------------------------------------------------------------- host side
-template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces>
+template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool kPieces, bool kSplit = false>
 cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorMap& vm, const CUtensorMap& km64,
                    const CUtensorMap& vm64, const ExtArgs& ext, const Strided& O,
                    const RangeList& ranges, int32_t T, int32_t heads, const PairPlan& pp, int32_t n_tiles, int3 qpos,
@@ -974,12 +1065,13 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
 {
     using C = Cfg<D, kWide, kDen>;
     static SharedMemoryOptIn opt_in;
-    const cudaError_t oe = opt_in.ensure(attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces>, (int)C::kSmemBytes);
+    const cudaError_t oe = opt_in.ensure(attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, (int)C::kSmemBytes);
     if (oe != cudaSuccess) return oe;
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
-    if (grid > pp.n_pairs) grid = pp.n_pairs;
-    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces>, dim3((unsigned)grid), dim3(C::kThreads),
-                         C::kSmemBytes, stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
+    if (kSplit) grid = pp.full > 0 ? ((int64_t)sm_count * C::kCtasPerSm) & ~1ll : 2ll * pp.n_pairs;
+    else if (grid > pp.n_pairs) grid = pp.n_pairs;
+    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
+                         KernelMemory(C::kSmemBytes, kSplit ? 2u : 1u), stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
                          ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);
 }
 
@@ -1056,6 +1148,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     memcpy(&km64, k_map64, sizeof(km64));
     memcpy(&vm64, v_map64, sizeof(vm64));
     PairPlan pp;
+    pp.full = 0;
     pp.nqt = (T + kQRows - 1) / kQRows;
     pp.npi = pp.nqt / 2;
     if ((int64_t)rows * heads > 0x3fffffffll) return cudaErrorInvalidValue;
@@ -1094,7 +1187,20 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // filled tile of the caller's tensors as one box; the long launches keep the one-lane producer (its smaller code
     // measured 2 % faster there).
     // Writes in several pieces are instantiated for the lazy form only.
-    constexpr int lazy_min = 3, lazy128_min = 3, short_max = 4;
+    constexpr int lazy_min = 3, lazy128_min = 3, short_max = 4, split_min = 12;
+    if (D == 128 && !density && ext.n_pieces == 0 && pp.kind != 3) {
+        // The last round of units often leaves most SMs idle.  Where at most half of them have a unit in it (and there is
+        // something to halve: a merge costs about five key tiles), two CTAs share each of its units.  us per call, before /
+        // after: 32 items, T = 1 600 (208 units on 148 SMs) 139 / 105, T = 4 096 (512) 535 / 491; 48 items, T = 1 024 (192) 82 / 68;
+        // 64 items, T = 576 (160) 61 / 50; 128 items, T = 576 (320) 88 / 77; 256 items, T = 400 (512, 11 to 15 tiles) 89 / 86.
+        // (64 channels have two CTAs per SM, and the one that is left alone in the last round runs a third faster.)
+        const int32_t slots = sm_count & ~1, rest = pp.n_pairs % slots;
+        if (rest > 0 && 2 * rest <= slots && n_tiles >= split_min) {
+            pp.full = pp.n_pairs / slots;
+            if (cur) AMSKV_PAIR_LAUNCH(128, true, true, false, true, false, false, true);
+            AMSKV_PAIR_LAUNCH(128, false, true, false, true, false, false, true);
+        }
+    }
     if (D == 128) {
         if (density) AMSKV_PAIR_LAUNCH(128, false, true, true, false, false, false);
         if (n_tiles >= lazy128_min || ext.n_pieces > 0) {

@@ -161,19 +161,33 @@ void count_launch(int n = 1);
 // its scale's append.  Copies that start on SMs still configured for the attention kernel's shared memory keep their small
 // L1, which is where their loads in flight are held, and attention CTAs placed beside the last blocks of a copy find an SM
 // with its shared-memory split, which only an idle SM can change (T = 256, 1 920 items, a copy before each: +4 to +9 %).
+struct KernelMemory {     // dynamic shared memory, and the CTAs of a cluster (1: no clusters)
+    size_t bytes;
+    unsigned cluster;
+    KernelMemory(size_t n, unsigned c = 1) : bytes(n), cluster(c) {}
+};
 template <typename... P, typename... A>
-cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args)
+cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 block, KernelMemory smem, cudaStream_t stream, const A&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = smem.bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    unsigned n = 0;
+    if (overlap) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (smem.cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = smem.cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 1 : 0;
+    cfg.numAttrs = n;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
     if (e == cudaSuccess) count_launch();
     return e;

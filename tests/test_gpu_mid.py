@@ -141,3 +141,27 @@ def test_paired_kernel_writes_an_append_in_pieces(D):
                 check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, 1.0 / math.sqrt(D)), "layer %d scale %d" % (layer, k))
         assert B.amskv_status(c.h) == 0
     assert copies == {1, 2, 3}
+
+
+@pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
+@pytest.mark.parametrize("rows,heads,sides", [
+    (5, 31, (3, 28)),          # 155 items, seven query tiles: 620 units, 28 left over after four rounds of 148
+    (2, 16, (16, 17, 25)),     # 32 items, five query tiles at the end, pairs of both kinds: 80 units, none whole
+    (1, 150, (5, 27)),         # 150 items, six query tiles (the last ragged): 450 units, six left over
+])
+def test_last_round_shared_by_two_ctas(rows, heads, sides, fused):
+    """128 channels, launches whose last round of units is split over clusters of two CTAs: odd and even numbers of key tiles,
+    a ragged last query tile, streams with tiles of their own, fused writes from both halves, moving references."""
+    D = 128
+    pols = [(0, 9, True)]
+    qkv = make_qkv(rows, heads, sides, D, seed=95, peaked=True)
+    n = rows * heads
+    items = sorted({0, 1, n // 2, n - 28, n - 13, n - 2, n - 1})
+    with Cache(1, heads, D, rows, sides, pols) as c:
+        outs = run_pass(c, qkv, B.PATH_TENSOR_PAIR, fused=fused)
+        want = oracle_outputs(qkv, pols[0], 1.0 / math.sqrt(D), items=items)
+        for k in range(len(sides)):
+            got = outs[0][k].reshape(n, -1, D)[items].cpu().double()
+            check_close(got, want[k], "scale %d" % k, max_abs=4e-2)
+        again = run_pass(c, qkv, B.PATH_TENSOR_PAIR, fused=fused)
+        assert all(torch.equal(x, y) for x, y in zip(outs[0], again[0]))

@@ -97,6 +97,11 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+try:
+    from . import _steps
+except ImportError as e:
+    raise ImportError("the binding's _steps module is not built for this interpreter: run "
+                      "`python paper_2511_16047_b200/build.py`") from e
 EXPORTS = ("amskv_cache_required_bytes amskv_cache_create amskv_cache_destroy amskv_cache_reset amskv_append "
            "amskv_attend amskv_append_attend amskv_attention_density amskv_attend_density amskv_first_overflow_scale amskv_promote_layer amskv_set_attend_path amskv_step_host amskv_step_staging_bytes amskv_layer_similarity "
            "amskv_similarity_workspace_bytes amskv_layer_similarity_static amskv_classify_by_threshold amskv_classify_lowest "
@@ -114,72 +119,35 @@ def _check(code: int, where: str) -> None:
         raise AmskvError(code, where)
 
 
-# The calls of a generation step are made thousands of times a second from Python, so their marshalling is kept short: their
-# own function objects take every pointer as a plain address, and the ctypes array of a stride triple is made once per triple
-# (a memo of values; nothing is kept by a tensor's address or identity).  The Python side of a call with four strided
-# tensors: 8.5 -> 3.3 us, with contiguous ones 2.9 -> 2.1 us.
-def _plain(name: str, args):
-    fn = lib[name]   # (indexing makes a function object of its own; lib.<name> keeps its argument types)
-    fn.argtypes = args
-    fn.restype = ctypes.c_int
-    return fn
-
-
-_VP, _I = ctypes.c_void_p, ctypes.c_int
-_call_append = _plain("amskv_append", [_VP, _I, _I, _VP, _VP, _VP, _VP])
-_call_attend = _plain("amskv_attend", [_VP, _I, _I, _VP, _VP, _VP, _VP, _VP])
-_call_append_attend = _plain("amskv_append_attend", [_VP, _I, _I, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP])
-
-_call_density = _plain("amskv_attention_density", [_VP, _I, _I, _VP, _VP, _VP, ctypes.c_size_t, _VP])
-_call_attend_density = _plain("amskv_attend_density", [_VP, _I, _I, _VP, _VP, _VP, _VP, _VP, ctypes.c_size_t, _VP])
-
-_MAX_TRIPLES = 1024
-_triples_memo = {}
+# The calls of a generation step go through the _steps module, which takes addresses and strides out of the tensors natively.
+_steps.bind(*(ctypes.cast(fn, ctypes.c_void_p).value for fn in (lib.amskv_append, lib.amskv_attend, lib.amskv_append_attend)))
 
 
 def _addr(x) -> Optional[int]:
     if x is None:
         return None
-    try:
-        return x.data_ptr()
-    except AttributeError:
-        return int(x)
+    if hasattr(x, "data_ptr"):
+        return int(x.data_ptr())
+    return int(x)
 
 
-def _strides(x) -> Optional[int]:
-    """Address of the element strides (row, head, token) of a [rows, heads, T, D] tensor, or None if contiguous/raw."""
-    try:
-        if x.is_contiguous():
-            return None
-        s = x.stride()
-    except AttributeError:
+def _strides(x) -> Optional[ctypes.Array]:
+    """Element strides (row, head, token) of a [rows, heads, T, D] tensor, or None if contiguous/raw."""
+    if x is None or not hasattr(x, "stride"):
         return None
-    entry = _triples_memo.get(s)
-    if entry is None:
-        assert len(s) == 4 and s[3] == 1, "expected [rows, heads, T, D] with contiguous channels"
-        arr = (ctypes.c_int64 * 3)(s[0], s[1], s[2])
-        # (an array that is no longer in the memo must outlive the call that uses its address: beyond the bound nothing is
-        # taken out, the caller's frame keeps the array instead)
-        if len(_triples_memo) >= _MAX_TRIPLES:
-            return arr
-        entry = _triples_memo.setdefault(s, (ctypes.addressof(arr), arr))   # one array per triple whichever thread comes first
-    return entry[0]
-
-
-def _kv_strides(K, V):
-    ks, vs = _strides(K), _strides(V)
-    if ks is not vs and (ks is None or vs is None or K.stride()[:3] != V.stride()[:3]):
-        raise ValueError("K and V must share one stride triple")
-    return ks
+    if x.is_contiguous():
+        return None
+    s = x.stride()
+    assert x.dim() == 4 and s[3] == 1, "expected [rows, heads, T, D] with contiguous channels"
+    return (ctypes.c_int64 * 3)(s[0], s[1], s[2])
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
         return None
-    try:
-        return stream.cuda_stream
-    except AttributeError:
-        return int(stream)
+    if hasattr(stream, "cuda_stream"):
+        return int(stream.cuda_stream)
+    return int(stream)
 
 
 def make_desc(layers: int, heads: int, head_dim: int, rows: int, sides: Sequence[int],
@@ -234,34 +202,33 @@ def amskv_cache_reset(cache: int) -> None:
 
 
 def amskv_append(cache: int, layer: int, scale: int, K, V, stream=None) -> None:
-    rc = _call_append(cache, layer, scale, _addr(K), _addr(V), _kv_strides(K, V), _stream(stream))
-    if rc != OK:
+    rc = _steps.append(cache, layer, scale, K, V, stream)
+    if rc:
         raise AmskvError(rc, "amskv_append")
 
 
 def amskv_attend(cache: int, layer: int, scale: int, Q, out, stream=None) -> None:
-    rc = _call_attend(cache, layer, scale, _addr(Q), _addr(out), _strides(Q), _strides(out), _stream(stream))
-    if rc != OK:
+    rc = _steps.attend(cache, layer, scale, Q, out, stream)
+    if rc:
         raise AmskvError(rc, "amskv_attend")
 
 
 def amskv_append_attend(cache: int, layer: int, scale: int, K, V, Q, out, stream=None) -> None:
     """append(layer, scale, K, V) then attend(layer, scale, Q, out), as one launch where possible."""
-    rc = _call_append_attend(cache, layer, scale, _addr(K), _addr(V), _kv_strides(K, V), _addr(Q), _addr(out), _strides(Q),
-                             _strides(out), _stream(stream))
-    if rc != OK:
+    rc = _steps.append_attend(cache, layer, scale, K, V, Q, out, stream)
+    if rc:
         raise AmskvError(rc, "amskv_append_attend")
 
 
 def amskv_attention_density(cache: int, layer: int, scale: int, Q, out, out_entries: int, stream=None) -> None:
     """Attention density per (head, run of amskv_attended_tokens) into `out` (device doubles)."""
-    _check(_call_density(cache, layer, scale, _addr(Q), _strides(Q), _addr(out), int(out_entries), _stream(stream)),
+    _check(lib.amskv_attention_density(cache, layer, scale, _addr(Q), _strides(Q), _addr(out), int(out_entries), _stream(stream)),
            "amskv_attention_density")
 
 
 def amskv_attend_density(cache: int, layer: int, scale: int, Q, out, density, density_entries: int, stream=None) -> None:
     """amskv_attend plus the attention density of the same queries, from one launch where the paired kernel serves."""
-    _check(_call_attend_density(cache, layer, scale, _addr(Q), _addr(out), _strides(Q), _strides(out), _addr(density),
+    _check(lib.amskv_attend_density(cache, layer, scale, _addr(Q), _addr(out), _strides(Q), _strides(out), _addr(density),
                                 int(density_entries), _stream(stream)), "amskv_attend_density")
 
 

@@ -1,13 +1,17 @@
-"""Builds libamskv.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds libamskv.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension), and the small CPython module
+(_steps) through which the binding calls it."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libamskv.so")
+STEPS = os.path.join(HERE, "_steps" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+STEPS_SOURCE = os.path.join(CSRC, "steps.c")
 SOURCES = ["api.cu", "append.cu", "attend_simt.cu", "attend_tc.cu", "attend_pair.cu", "attend_small.cu", "attend_mid.cu", "similarity.cu", "density.cu", "selftest.cu"]
 HEADERS = ["kernels.cuh", "policy.hpp", "sm100_ptx.cuh", os.path.join("..", "..", "include", "amskv.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,8 +33,20 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_steps(force: bool = False) -> str:
+    """Compile the binding's CPython module for the running interpreter."""
+    if not force and os.path.exists(STEPS) and os.path.getmtime(STEPS) >= os.path.getmtime(STEPS_SOURCE):
+        return STEPS
+    tmp = STEPS + ".tmp.%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-I" + sysconfig.get_paths()["include"], STEPS_SOURCE, "-o", tmp])
+    os.replace(tmp, STEPS)
+    return STEPS
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu for sm_100a into one shared library next to this file."""
+    build_steps(force)
     if not force and not _stale():
         return LIB
     objs = []

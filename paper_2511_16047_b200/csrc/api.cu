@@ -196,7 +196,7 @@ enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
 AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool copies = false)
 {
     // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained)
-    if (cache->path == AMSKV_PATH_AUTO && T > 1 && cache->tc_ready &&
+    if (cache->path == AMSKV_PATH_AUTO && (T > 1 || density) && cache->tc_ready &&
         mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density, copies))
         return AttendKernel::Mid;
     // AUTO: the warp-per-item kernel wherever a scale's retained keys fit its register tile, the paired
@@ -634,7 +634,7 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
             den.run_of_range[i] = (int8_t)rp[i].run;
         }
         cudaStream_t st = static_cast<cudaStream_t>(stream);
-        cudaError_t e = cudaMemsetAsync(density, 0, sizeof(double) * (size_t)cache->heads * n_runs, st);
+        cudaError_t e = launch_zero(density, (size_t)cache->heads * n_runs, st);
         if (e == cudaSuccess && kernel == AttendKernel::Mid)
             e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
                                   cache->softmax_scale, cache->sm_count, st, nullptr, nullptr, 0, &den);

@@ -1070,7 +1070,7 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
     if (kSplit) grid = pp.full > 0 ? ((int64_t)sm_count * C::kCtasPerSm) & ~1ll : 2ll * pp.n_pairs;
     else if (grid > pp.n_pairs) grid = pp.n_pairs;
-    return launch_kernel(kExt, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
+    return launch_kernel(kExt || kDen, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
                          KernelMemory(C::kSmemBytes, kSplit ? 2u : 1u), stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
                          ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);
 }

@@ -93,7 +93,21 @@ density_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_hea
         atomicAdd(out + (int64_t)head * pieces.n_runs + pieces.run[i], acc[i] * inv_rows * pieces.weight[i]);
 }
 
+// Zeroes the result ahead of a launch that adds to it.  A kernel rather than a memset: the launch behind it can then overlap
+// it (append, zero, attention at T = 25, 512 items: 14.2 -> 11.3 us; a whole pass of 4 layers 1 104 -> 1 071 us).
+__global__ void __launch_bounds__(256) zero_kernel(double* __restrict__ p, int64_t n)
+{
+    overlap_with_previous();
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) p[i] = 0.0;
+}
+
 }  // namespace
+
+cudaError_t launch_zero(double* p, size_t n, cudaStream_t stream)
+{
+    const unsigned blocks = n > 256 * 64 ? 64u : (unsigned)((n + 255) / 256);
+    return launch_kernel(false, zero_kernel, dim3(blocks > 0 ? blocks : 1u), dim3(256), 0, stream, p, (int64_t)n);
+}
 
 cudaError_t launch_density(const Strided& Q, const LayerRegion& region, const DensityPieces& pieces, int32_t T,
                            int32_t rows, int32_t heads, int32_t D, float softmax_scale, double* out, cudaStream_t stream)

@@ -141,6 +141,7 @@ struct DensityPieces {
     int32_t start[kMaxDensityPieces], len[kMaxDensityPieces], run[kMaxDensityPieces];
     double weight[kMaxDensityPieces];
 };
+cudaError_t launch_zero(double* p, size_t n, cudaStream_t stream);
 cudaError_t launch_density(const Strided& Q, const LayerRegion& region, const DensityPieces& pieces, int32_t T,
                            int32_t rows, int32_t heads, int32_t D, float softmax_scale, double* out, cudaStream_t stream);
 

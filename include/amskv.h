@@ -218,9 +218,8 @@ AMSKV_API int amskv_attend(amskv_cache* cache, int layer, int scale, const void*
  * from the caller's tensors and stores the registers that feed its products), and a single-token scale
  * that is its own only key is one copy kernel (out = V).  Scales served by the CUDA-core or the single-stream
  * kernel and, under AMSKV_PATH_AUTO, paired-kernel scales of fewer than 32 tokens and scales where
- * splitting the current scale off its cache range would add a 64-token key tile, run as the two calls
- * (appends of several copies -- a token budget whose ring wraps inside the scale -- may add one above 128
- * tokens, launches of at most one query tile per SM may add any).
+ * splitting the current scale off its cache range would add more 64-token key tiles than the copy is
+ * worth, run as the two calls.
  *   K, V: as for amskv_append (one stride triple kv_strides for both); Q, out: as for
  *   amskv_attend.  out must not overlap Q, K or V.
  * Stream ordering: as for the two calls -- this call must come after attend(layer, scale - 1)

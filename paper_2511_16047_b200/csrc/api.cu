@@ -525,18 +525,23 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         }
     }
     if (fused && cache->path == AMSKV_PATH_AUTO) {
-        // Taking the scale from the caller's tensors splits it off the range it would be part of in the
-        // cache; where that adds a tile, attention loses more than the saved copy is worth (measured), so
-        // such scales run as the two calls (AMSKV_PATH_TENSOR_PAIR fuses wherever it can).  Not where the kernel has an SM
-        // for every query tile: there another key tile is 0.8 us, the copy 2.  Above 128 queries one more tile is less than
-        // the several copies of an append whose ring wraps (1 920 items, three such layers of ten: T = 256 1 046 -> 1 028 us; T =
-        // 100, seven of ten: 487 -> 554).
+        // Taking the scale from the caller's tensors splits it off the range it would be part of in the cache, which may add a
+        // 64-token key tile.  One more tile costs less than the copy kernel, its launch and the second read of K and V (us per
+        // call, two calls / fused, 64 channels: T = 81 43.8 / 39.9, T = 169 101 / 83 and T = 324 246 / 223 with 2 304 items, T = 121
+        // 29.4 / 24.5 with 512, T = 169 228 / 208 with 5 120; T = 100 with 255 keys is even: 1 920 items 50 / 52, 15 360 items 283 /
+        // 279), except where 128 channels have few tiles (T = 49, two to three tiles, 1 024 items: 35.5 / 38.1; T = 144, four to
+        // five, 256 items: 26.7 / 23.6).  Appends of several copies, which the producer writes partly row by row, take it above
+        // 128 queries only (1 920 items, ten layers: T = 256 1 046 / 1 028, T = 100 487 / 554).  A launch of at most one unit per
+        // SM fuses anyway: another key tile is 0.8 us there, the copy 2 (T = 100, 256 items: 16.9 / 13.6).
+        // (AMSKV_PATH_TENSOR_PAIR fuses wherever it can.)
         auto tiles = [](const RangeList& rl) {
             int32_t n = 0;
             for (int i = 0; i < rl.n; ++i) n += (rl.r[i].len + 63) / 64;
             return n;
         };
-        if (tiles(ranges) + (T + 63) / 64 > tiles(after) + (!one_copy && T > 128 ? 1 : 0) && !pair_one_tile_per_sm(cache->items(), T, cache->sm_count)) fused = false;
+        const int32_t more = tiles(ranges) + (T + 63) / 64 - tiles(after);
+        const bool worth = one_copy ? more <= 1 && (cache->head_dim == 64 || tiles(after) > 3) : more <= (T > 128 ? 1 : 0);
+        if (more > 0 && !worth && pair_units(cache->items(), T) > cache->sm_count) fused = false;
         // Well below a full key tile per scale the units are so short that the kernel is bound by the latency of
         // its loads; holding a stage until it has been written out costs as much there as the copy (measured:
         // equal at T = 36, where fusing at least saves the launch and the second read; a loss at T = 25).

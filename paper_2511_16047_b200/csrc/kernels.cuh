@@ -105,6 +105,12 @@ struct PairDensity {
 
 // Whether the paired kernel gives every 128-query tile of a launch a CTA and an SM of its own.
 inline bool pair_one_tile_per_sm(int64_t items, int32_t T, int sm_count) { return items * ((T + 127) / 128) <= sm_count; }
+// Units of a launch that pairs query tiles: two of one item, or the left-over ones of two items.
+inline int64_t pair_units(int64_t items, int32_t T)
+{
+    const int64_t nqt = (T + 127) / 128;
+    return items * (nqt / 2) + ((nqt & 1) ? (items + 1) / 2 : 0);
+}
 
 // Paired tensor-core kernel: two softmax groups per CTA, probabilities kept in tensor memory.
 cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k_map16, const void* v_map16,

@@ -87,7 +87,8 @@ extern "C" {
 /* amskv_set_attend_path */
 #define AMSKV_PATH_AUTO 0   /* warp-per-item kernel for the coarse scales (at most 16 queries and 32
                                retained keys; CUDA-core kernel for a single query token with several
-                               keys), paired tcgen05 kernel otherwise                               */
+                               keys), warp-matrix kernel for calls that would leave most of the chip
+                               idle in the paired tcgen05 kernel, that kernel otherwise             */
 #define AMSKV_PATH_SIMT 1   /* always the CUDA-core kernel                                     */
 #define AMSKV_PATH_TENSOR 2 /* always the single-stream tcgen05 kernel                         */
 #define AMSKV_PATH_TENSOR_PAIR 3 /* always the paired tcgen05 kernel (two query tiles per CTA)  */
@@ -257,8 +258,10 @@ AMSKV_API int amskv_attention_density(amskv_cache* cache, int layer, int scale, 
  * second pass over the keys; the cut tiles make the launch somewhat longer than a plain amskv_attend (more,
  * partly filled key tiles).  `out` is the same as amskv_attend's.  `density`, `density_entries` and the
  * meaning of the numbers are those of amskv_attention_density (probabilities after their rounding to bf16,
- * where that call uses them unrounded: they agree to about 1e-4 relative).  Scales the other kernels serve,
- * and layers with more than 16 runs, run as amskv_attend followed by amskv_attention_density.
+ * where that call uses them unrounded: they agree to about 1e-4 relative).  The warp-matrix kernel serves
+ * scales of at most 16 queries and calls of few items the same way in one launch (the masses are products of
+ * the probabilities with a 0/1 matrix of run membership).  The kernels of the other paths, and layers with
+ * more than 16 runs, run as amskv_attend followed by amskv_attention_density.
  * Errors: as for the two calls.
  */
 AMSKV_API int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q, void* out,

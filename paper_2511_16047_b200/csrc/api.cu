@@ -389,7 +389,7 @@ int amskv_attend(amskv_cache* cache, int layer, int scale, const void* Q, void* 
     cudaError_t e;
     if (kernel == AttendKernel::Small) {
         e = launch_attend_small(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
-                                cache->softmax_scale, static_cast<cudaStream_t>(stream));
+                                cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream));
     } else if (kernel == AttendKernel::Mid) {
         e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
                               cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream));
@@ -479,7 +479,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         if (before.total + T == after.total) {
             CurrentScaleSource cur{ks, vs, true, piece[0].dst, cache->region(layer)};
             cudaError_t e = launch_attend_small(q, o, cache->region(layer), before, T, cache->rows, cache->heads, cache->head_dim,
-                                                cache->softmax_scale, static_cast<cudaStream_t>(stream), &cur);
+                                                cache->softmax_scale, cache->sm_count, static_cast<cudaStream_t>(stream), &cur);
             if (e != cudaSuccess) { (void)cudaGetLastError(); return AMSKV_ERR_CUDA; }
             note_appended(cache, layer, scale);
             return AMSKV_OK;

@@ -31,7 +31,7 @@ namespace amskv {
 
 namespace {
 
-constexpr int kWarpsPerCta = 4;
+constexpr int kWarpsPerCta = 2;     // (4: the same above 3 000 items, up to 10 % slower where the items leave SMs idle)
 static_assert(kSmallMaxKeys == 32, "the register tile is instantiated for 1, 2 and 4 eight-key tiles");
 
 __device__ __forceinline__ float fast_exp2(float x)
@@ -88,8 +88,14 @@ struct SmallExt {
 // kTiles: 8-key tiles a row can have (1, 2 or 4): the register tile is sized for it, so the coarsest scales,
 // whose rows are a handful of keys, run with more warps per SM -- their launches are bound by how many
 // independent items are in flight, not by arithmetic.
-template <int D, bool kExt, int kTiles>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? (kTiles == 1 ? 6 : 4) : (kTiles == 1 ? 3 : 2))
+// kEarlyV: V is fetched together with K instead of when the second product starts.  With the largest tile that
+// costs registers.  With 64 channels that means 12 resident warps per SM instead of 16, which a large batch is
+// bound by (3 840 items, T = 16: 15.8 us per call late, 18.1 early), while a launch whose items are all resident
+// at once is bound by its round trips to memory, one instead of three (60 items 3.5 -> 3.2 us, 960 items 7.4 ->
+// 7.1).  With 128 channels both forms have 8 warps per SM and the early one is always ahead (30 items 4.1 -> 3.3
+// us, 480 items 6.8 -> 5.8, 2 880 items 21.4 -> 18.5).
+template <int D, bool kExt, int kTiles, bool kEarlyV>
+__global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? (kTiles == 1 ? 6 : kTiles == 4 && kEarlyV ? 6 : 8) : (kTiles == 1 ? 6 : 4))
 attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
                     __nv_bfloat16* __restrict__ O, int64_t o_row, int64_t o_head, int64_t o_tok,
                     __nv_bfloat16* __restrict__ region, int32_t capacity, const RangeList ranges, int32_t T,
@@ -154,10 +160,7 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
                 for (int h = 0; h < kPieces; ++h) kk[t][h] = __ldg(kp[t] + 4 * h);
             }
         }
-        // ---- V pieces likewise (nothing the softmax computes is needed to fetch them), except with the
-        // largest register tile, where holding them through the softmax costs more in resident warps than the
-        // earlier fetch gains (measured): there they are fetched when the second product starts
-        constexpr bool kEarlyV = kTiles < 4;
+        // ---- V pieces likewise (nothing the softmax computes is needed to fetch them)
         uint4 vv[kTiles][kPieces];
 #pragma unroll
         for (int t = 0; t < kTiles; ++t) {
@@ -306,7 +309,7 @@ bool small_supported(int32_t T, int32_t total_keys) { return T <= kSmallMaxQueri
 
 cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges,
                                 int32_t T, int32_t rows, int32_t heads, int32_t D, float softmax_scale,
-                                cudaStream_t stream, const CurrentScaleSource* cur)
+                                int sm_count, cudaStream_t stream, const CurrentScaleSource* cur)
 {
     const int32_t total = ranges.total + (cur ? T : 0);
     if (!small_supported(T, total)) return cudaErrorInvalidValue;
@@ -335,15 +338,17 @@ cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerR
     }
     const int64_t blocks = (items + kWarpsPerCta - 1) / kWarpsPerCta;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
-#define AMSKV_SMALL_LAUNCH(DD, EXT, TILES)                                                                            \
-    return launch_kernel(EXT, attend_small_kernel<DD, EXT, TILES>, dim3((unsigned)blocks), dim3(kWarpsPerCta * 32), 0, stream, \
-                         (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head, \
+    const bool early = D == 128 || items <= (int64_t)sm_count * 12;   // (all items resident at once; see the kernel)
+#define AMSKV_SMALL_LAUNCH(DD, EXT, TILES, EARLY)                                                                             \
+    return launch_kernel(EXT, attend_small_kernel<DD, EXT, TILES, EARLY>, dim3((unsigned)blocks), dim3(kWarpsPerCta * 32), 0, stream,\
+                         (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head,           \
                          O.token, region.base, region.capacity, ranges, T, heads, (int32_t)items, scale_log2, ext)
-#define AMSKV_SMALL_TILES(DD, EXT)                                                                                    \
-    do {                                                                                                              \
-        if (total <= 8) AMSKV_SMALL_LAUNCH(DD, EXT, 1);                                                               \
-        else if (total <= 16) AMSKV_SMALL_LAUNCH(DD, EXT, 2);                                                         \
-        else AMSKV_SMALL_LAUNCH(DD, EXT, 4);                                                                          \
+#define AMSKV_SMALL_TILES(DD, EXT)                                                                                            \
+    do {                                                                                                                      \
+        if (total <= 8) AMSKV_SMALL_LAUNCH(DD, EXT, 1, true);                                                                 \
+        else if (total <= 16) AMSKV_SMALL_LAUNCH(DD, EXT, 2, true);                                                           \
+        else if (early) AMSKV_SMALL_LAUNCH(DD, EXT, 4, true);                                                                 \
+        else AMSKV_SMALL_LAUNCH(DD, EXT, 4, DD == 128);                                                                       \
     } while (0)
     if (D == 64) {
         if (cur) AMSKV_SMALL_TILES(64, true);

@@ -127,7 +127,7 @@ bool small_supported(int32_t T, int32_t total_keys);
 // keys must fit the limits.  A single-token scale that is its own only key is served by a copy kernel.
 cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges,
                                 int32_t T, int32_t rows, int32_t heads, int32_t D, float softmax_scale,
-                                cudaStream_t stream, const CurrentScaleSource* cur = nullptr);
+                                int sm_count, cudaStream_t stream, const CurrentScaleSource* cur = nullptr);
 
 // Kernel for calls of few items or few queries (attend_mid.cu): a CTA per item and group of query blocks, warp-level matrix
 // instructions.  With `cur`, `ranges` lists the cached keys only and the current scale's tokens come from the caller's

@@ -154,3 +154,19 @@ def test_order_contract():
                                          None, None, None) == B.ERR_ORDER
         torch.cuda.synchronize()
         assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_coarse_scale_on_both_sides_of_one_round_of_items(D):
+    """The largest register tile of the warp-per-item kernel fetches V with K where all items are resident at once
+    (64 channels: 148 x 12 = 1776 items) and late beyond; an odd number of items leaves a CTA half empty."""
+    sides, heads = (3, 4), 37
+    for rows in (1, 48, 49):                                   # 37, 1776 and 1813 items
+        qkv = make_qkv(rows, heads, sides, D, seed=96)
+        with Cache(1, heads, D, rows, sides, [(1, 2, False)]) as c:
+            outs = run_pass(c, qkv, B.PATH_AUTO, fused=True)
+            pick = [0, rows * heads // 2, rows * heads - 1]
+            for k in range(len(sides)):
+                items = [x.reshape(rows * heads, -1, D)[pick].cpu().double().numpy() for t in qkv[: k + 1] for x in t]
+                want = oracle.attend_selected(items[3 * k], items[1::3], items[2::3], oracle.keep_set(k, 1, 2, False), 1 / D ** 0.5)
+                check_close(outs[0][k].reshape(rows * heads, -1, D)[pick], want, "rows %d scale %d" % (rows, k))

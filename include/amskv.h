@@ -252,11 +252,11 @@ AMSKV_API int amskv_attention_density(amskv_cache* cache, int layer, int scale, 
 /*
  * amskv_attend(layer, scale, Q, out) that also returns the attention density of the same queries (Sec. 4.1,
  * the definition of d), as a by-product of the attention launch: where the paired tensor-core kernel serves
- * the scale, its key tiles are cut at the boundaries of the runs of attended tokens, and the un-normalised
- * probability mass of a query row on a run is a running sum of the per-tile sums the softmax computes anyway;
+ * the scale, every 16-token box of its key tiles belongs to one run of attended tokens, and the un-normalised
+ * probability mass of a query row on a run is a running sum of the box sums the softmax computes anyway;
  * the rows are normalised by their row sums in the epilogue and added up per (head, run).  One launch, no
- * second pass over the keys; the cut tiles make the launch somewhat longer than a plain amskv_attend (more,
- * partly filled key tiles).  `out` is the same as amskv_attend's.  `density`, `density_entries` and the
+ * second pass over the keys; the launch is somewhat longer than a plain amskv_attend (a few more, partly
+ * filled key tiles, and the sums).  `out` is the same as amskv_attend's.  `density`, `density_entries` and the
  * meaning of the numbers are those of amskv_attention_density (probabilities after their rounding to bf16,
  * where that call uses them unrounded: they agree to about 1e-4 relative).  The warp-matrix kernel serves
  * scales of at most 16 queries and calls of few items the same way in one launch (the masses are products of

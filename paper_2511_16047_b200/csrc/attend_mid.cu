@@ -514,8 +514,9 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // 8.8 / 7.7 (60); T = 144: 8.2 / 8.5 (16), 10.3 / 8.7 (32).
 // 128 channels: 6 units: T = 36: 5.2 / 10.2 (32), 6.2 / 10.8 (128), 20.5 / 17.1 (512); T = 64: 6.8 / 8.0 (32), 7.0 / 8.9 (64), 10.4 / 10.4
 // (128); none above 64 queries where the paired kernel has an SM for every tile: T = 81: 8.0 / 7.2 (16), 7.9 / 7.5 (32), 9.8 / 8.2 (64).
-// With the density the paired kernel's tiles are cut at the runs and the line lies higher (T = 25, 36, 64 at 512 items: 13.4 /
-// 19.7, 21.1 / 23.2, 26.7 / 26.3; 128 channels, T = 64, 128 items: 15.4 / 20.2), and up to 16 queries the alternative is the
+// With the density (20 and 7 units; times with the append and the zeroed result): T = 36: 10.2 / 13.0 (120 items), 12.0 / 14.5
+// (256), 18.2 / 16.4 (384), 19.4 / 16.9 (512); T = 64: 15.3 / 18.2 (256), 21.7 / 19.8 (384); T = 100: 15.8 / 18.4 (120), 26.4 / 21.8
+// (256); T = 25: 18.9 / 21.0 (1 024); 128 channels, T = 64: 13.9 / 17.0 (120), 22.5 / 19.3 (256); and up to 16 queries the alternative is the
 // attention call plus the CUDA-core density pass (T = 4, 9, 16 at 512 items: 12.5 / 16.6, 13.5 / 23.6, 13.0 / 35.0): always this
 // one.  Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).  An append of several copies (`copies`),
 // 2 us each beside the paired kernel, keeps the first lines.
@@ -525,7 +526,7 @@ bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int 
     if (!density && small_supported(T, total_keys)) return false;
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
     int line = D == 64 ? 19 : 6;
-    if (density) line = D == 64 ? 24 : 10;
+    if (density) line = D == 64 ? 20 : 7;
     else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? 7 : (T > 64 ? 0 : 6);
     return units <= (int64_t)sm_count * line;
 }

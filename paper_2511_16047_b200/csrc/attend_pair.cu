@@ -27,6 +27,7 @@
 // next query tile as soon as the last S of the current one has landed.
 // Every wait is bounded: a wait that gives up records a status code, all roles wind down,
 // copies in flight are awaited and the tensor memory is freed.
+#include <algorithm>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -147,14 +148,28 @@ struct ExtArgs {
 };
 
 // Attention density as a by-product (Sec. 4.1): the range list of such a launch has one entry per piece of a
-// run of attended tokens (never merged across runs), so every key tile belongs to one run and a row's
-// un-normalised probability mass per run is a running sum of the tile sums the softmax computes anyway.
+// run of attended tokens (never merged across runs), and every 16-token box of a key tile belongs to one run, so
+// a row's un-normalised probability mass per run is a running sum of the box sums the softmax computes anyway.
+// The whole 64-token tiles of the ranges come first; what is left of each range, up to four boxes with the last
+// partly filled, is packed four boxes to a mixed tile, whatever the runs.  (With every tile cut at the runs, T = 100 of a
+// cache-demanding layer of the 680-token schedule was nine tiles; it is five.  With the epilogue below: 512 items, T = 64, 100,
+// 169, 256: 22.9 / 31.1 / 48.6 / 64.8 -> 19.9 / 27.9 / 44.2 / 62.3 us per call, copy of the append included.)
+struct MixedTile {
+    uint64_t keep;                     // a bit per column that holds a key
+    int32_t tok[4];                    // first token of each box
+    uint32_t runs;                     // run of each box, a byte each
+    int32_t boxes;
+};
+template <bool kDen>   // (without the tables for the launches that do not need them)
 struct DenArgs {
     double* out;                       // [heads][n_runs], accumulated with atomic adds
     int32_t n_runs;
-    float weight[kMaxDenRuns];         // 1 / (rows * tokens of the run)
-    int8_t run_of_range[kMaxRanges];
+    int32_t n_whole;                   // whole tiles; the mixed ones are the tiles behind them
+    float weight[kDen ? kMaxDenRuns : 1];         // 1 / (rows * tokens of the run)
+    int8_t run_of_range[kDen ? kMaxRanges : 1];
+    MixedTile mixed[kDen ? kMaxRanges : 1];       // (a range leaves at most four boxes)
 };
+constexpr int32_t kMixedFlag = 1 << 16;   // in a tile's second word; its first is then the index of the mixed tile
 
 struct Stream {
     int32_t item;
@@ -193,8 +208,7 @@ using namespace ptx;
 
 // Tile j of the resident ranges: first token and number of valid tokens (<= 64).
 // A tile of range `ext_range` (the current scale in the caller's tensors) carries kExtFlag in t0.
-__device__ __forceinline__ void tile_at(const RangeList& rl, int j, int32_t& t0, int32_t& valid, int ext_range = -1,
-                                        int* range_index = nullptr)
+__device__ __forceinline__ void tile_at(const RangeList& rl, int j, int32_t& t0, int32_t& valid, int ext_range = -1)
 {
     int r = 0;
     for (; r < rl.n - 1; ++r) {
@@ -205,7 +219,24 @@ __device__ __forceinline__ void tile_at(const RangeList& rl, int j, int32_t& t0,
     t0 = rl.r[r].start + j * kKT;
     valid = min(kKT, rl.r[r].start + rl.r[r].len - t0);
     if (r == ext_range) t0 |= kExtFlag;
-    if (range_index) *range_index = r;
+}
+
+// The same for a density launch: (first token, 64 | run << 8) of a whole tile, (index, 16 * boxes | kMixedFlag) of a mixed one.
+__device__ __forceinline__ void density_tile_at(const RangeList& rl, const DenArgs<true>& den, int j, int32_t& t0, int32_t& word)
+{
+    if (j >= den.n_whole) {
+        t0 = j - den.n_whole;
+        word = den.mixed[t0].boxes * kKVBoxRows | kMixedFlag;
+        return;
+    }
+    int r = 0;
+    for (; r < rl.n - 1; ++r) {
+        const int nt = rl.r[r].len / kKT;
+        if (j < nt) break;
+        j -= nt;
+    }
+    t0 = rl.r[r].start + j * kKT;
+    word = kKT | ((int32_t)den.run_of_range[r] << 8);
 }
 
 // ---------------------------------------------------------------- kernel
@@ -217,7 +248,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                    __nv_bfloat16* __restrict__ O, int64_t o_row,
                    int64_t o_head, int64_t o_tok, const RangeList ranges, int32_t T, int32_t heads,
                    const PairPlan pp, int32_t n_tiles, int3 qpos, float scale_log2, int* __restrict__ status,
-                   const __grid_constant__ DenArgs den)
+                   const __grid_constant__ DenArgs<kDen> den)
 {
     static_assert(!(kDen && kExt), "the density form serves the plain attend call");
     const int ext_range = kExt ? ext.range : -1;
@@ -255,9 +286,9 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
     for (int j = threadIdx.x; j < n_tiles && j < kTileTab; j += C::kThreads) {
         int32_t t0, valid;
-        int ri = 0;
-        tile_at(ranges, j, t0, valid, ext_range, &ri);
-        bars->tile_tab[j] = make_int2(t0, kDen ? (valid | ((int32_t)den.run_of_range[ri] << 8)) : valid);
+        if constexpr (kDen) density_tile_at(ranges, den, j, t0, valid);
+        else tile_at(ranges, j, t0, valid, ext_range);
+        bars->tile_tab[j] = make_int2(t0, valid);
     }
     if (layout_ok) {
         // query rows a tile does not cover keep whatever the slot held before; start them at zero
@@ -281,20 +312,19 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
-    // (in a density launch `valid` carries the tile's run in its bits 8..15; tile_run() strips it)
+    // (in a density launch `valid` also carries the tile's run, or that the tile is a mixed one; tile_run() strips that)
     auto tile_of = [&](int j, int32_t& t0, int32_t& valid) {
         if (j < kTileTab) {
             const int2 e = bars->tile_tab[j];
             t0 = e.x;
             valid = e.y;
         } else {
-            int ri = 0;
-            tile_at(ranges, j, t0, valid, ext_range, &ri);
-            if (kDen) valid |= (int32_t)den.run_of_range[ri] << 8;
+            if constexpr (kDen) density_tile_at(ranges, den, j, t0, valid);
+            else tile_at(ranges, j, t0, valid, ext_range);
         }
     };
-    auto tile_run = [](int32_t& valid) -> int {
-        const int run = kDen ? (valid >> 8) : 0;
+    auto tile_run = [](int32_t& valid) -> int {   // run of a whole tile, -1 for a mixed one
+        const int run = !kDen ? 0 : (valid & kMixedFlag) ? -1 : (valid >> 8);
         if (kDen) valid &= 0xff;
         return run;
     };
@@ -415,7 +445,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             for (int j = j_begin; ok && j < j_end; ++j) {
                 int32_t t0, valid;
                 tile_of(j, t0, valid);
-                (void)tile_run(valid);
+                const bool mixed = tile_run(valid) < 0;
                 const bool from_ext = kExt && (t0 & kExtFlag) != 0;
                 t0 &= ~kExtFlag;
                 const int nch = (valid + 15) >> 4;
@@ -443,7 +473,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                     // A tile of the caller's tensors that no rider shares its stage with is one 64-token box whatever
                     // its length: the tokens past the end of the scale are outside the tensor, cost no traffic and
                     // arrive as zeros (the products never read their rows, the fused write is clipped at the scale's end).
-                    const bool whole_box = nch == kKT / kKVBoxRows || (kShort && from_ext && !rider);
+                    const bool whole_box = !mixed && (nch == kKT / kKVBoxRows || (kShort && from_ext && !rider));
                     if (whole_box) {
                         if (elect_one()) {
                             mbar_expect_tx(full, (uint32_t)kKT * D * 2 * 2);
@@ -466,7 +496,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                 }
                             }
                         }
-                    } else if (!kShort) {
+                    } else if (!kShort && !kDen) {
                         // 16-token boxes (and the rider's box), issued by one lane
                         if (elect_one()) {
                             mbar_expect_tx(full, (uint32_t)(nch + (rider ? 1 : 0)) * kKVBoxRows * D * 2 * 2);
@@ -507,7 +537,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                             }
                         }
                     } else {
-                        // Short units (at most four key tiles): one lane per bulk copy, all issued by one instruction.  A
+                        // Short units (at most four key tiles) and mixed tiles: one lane per bulk copy, all issued by one instruction.  A
                         // lane issuing six or eight copies one after the other is what such units wait for (the issuing
                         // warp of a 36-token scale spent half its time waiting for tiles).
                         if (lane == 0) mbar_expect_tx(full, (uint32_t)(nch + (rider ? 1 : 0)) * kKVBoxRows * D * 2 * 2);
@@ -526,7 +556,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                 c[ext.pos.x] = t0 + bx * kKVBoxRows;
                                 tma_load_4d(dst, kv ? &ext.v16 : &ext.k16, full, h * 64, c[1], c[2], c[3]);
                             } else {
-                                tma_load_3d(dst, kv ? &v_map : &k_map, full, h * 64, is_rider ? ext.rider_tok : t0 + bx * kKVBoxRows, item);
+                                const int32_t tok = is_rider ? ext.rider_tok : kDen && mixed ? den.mixed[t0].tok[bx] : t0 + bx * kKVBoxRows;
+                                tma_load_3d(dst, kv ? &v_map : &k_map, full, h * 64, tok, item);
                             }
                         }
                     }
@@ -756,12 +787,6 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 int32_t t0, valid;
                 tile_of(j, t0, valid);
                 const int run = tile_run(valid);
-                if (kDen && run != cur_run) {
-                    // (the same for every thread: tiles and their runs are launch constants)
-                    if (cur_run >= 0 && warp_live) den_rows[cur_run * kQRows + r] += run_mass;
-                    run_mass = 0.f;
-                    cur_run = run;
-                }
                 const uint32_t s_tmem = s_tmem0 + buf_of(t) * kKT;
                 const uint32_t s_full = s_full0 + 16 * g + 8 * buf_of(t), p_full = p_full0 + 16 * g + 8 * buf_of(t);
                 if (!__all_sync(0xffffffffu, mbar_wait(s_full, par_of(t), abort_flag))) {
@@ -775,10 +800,12 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 if (warp_live) {
                     uint32_t sr[kKT];
                     tmem_ld64(s_tmem, sr);
-                    if (valid < kKT) {
+                    if (valid < kKT || (kDen && run < 0)) {
                         // (a rider occupies the box behind the tile's own: its tokens stay, the gap before them goes)
                         // as a bit per column, so that each column costs one test of a constant bit
-                        uint64_t keep = (1ull << valid) - 1ull;
+                        uint64_t keep;
+                        if (kDen) keep = den.mixed[t0].keep;   // (every other tile of a density launch is whole)
+                        else keep = (1ull << valid) - 1ull;
                         if (kExt && ext.rider_valid > 0 && j == n_tiles - 1)
                             keep |= ((1ull << ext.rider_valid) - 1ull) << ((valid + 15) & ~15);
                         const uint32_t keep_lo = (uint32_t)keep, keep_hi = (uint32_t)(keep >> 32);
@@ -855,10 +882,12 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                     // channels in the wide form only, where a warp has its scheduler nearly to itself: 1 000 -> 860 clocks a
                     // tile; 3 to 12 % slower elsewhere)
                     constexpr bool kStraight = kWide && D == 64;
+                    float box_sum[4] = {0.f, 0.f, 0.f, 0.f};   // kDen form only
                     auto exp_tile = [&](auto whole) -> float {
                         float sum0 = 0.f, sum1 = 0.f;
 #pragma unroll
                         for (int grp = 0; grp < kKT / 16; ++grp) {
+                            if (kDen) sum0 = sum1 = 0.f;
                             if (decltype(whole)::value || grp < groups) {   // (the same for the whole warp)
                                 uint32_t pk[8];
 #pragma unroll
@@ -881,7 +910,9 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                 }
                                 tmem_st8_nowait(s_tmem + grp * 8, pk);
                             }
+                            if (kDen) box_sum[grp] = sum0 + sum1;
                         }
+                        if (kDen) return (box_sum[0] + box_sum[1]) + (box_sum[2] + box_sum[3]);
                         return sum0 + sum1;
                     };
                     float tile_sum = kStraight && groups == kKT / 16 ? exp_tile(std::bool_constant<kStraight>{}) : exp_tile(std::false_type{});
@@ -905,7 +936,25 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         }
                     }
                     l += tile_sum;
-                    if (kDen) run_mass += tile_sum;
+                    if constexpr (kDen) {
+                        // (runs are the same for every thread: tiles and their boxes are launch constants)
+                        auto add_mass = [&](const int to, const float mass) {
+                            if (to != cur_run) {
+                                if (cur_run >= 0) den_rows[cur_run * kQRows + r] += run_mass;
+                                run_mass = 0.f;
+                                cur_run = to;
+                            }
+                            run_mass += mass;
+                        };
+                        if (run >= 0) {
+                            add_mass(run, tile_sum);
+                        } else {
+                            const uint32_t runs = den.mixed[t0].runs;
+#pragma unroll
+                            for (int b = 0; b < kKT / kKVBoxRows; ++b)
+                                if (b < groups) add_mass((int)((runs >> (8 * b)) & 0xffu), box_sum[b]);
+                        }
+                    }
                     tmem_wait_st();
                 }
                 tc_fence_before();
@@ -952,18 +1001,29 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 }
             }
             if (kDen && warp_live) {
-                // the row's share of every run, normalised by its row sum, added up over the warp's rows and
-                // then, weighted by 1 / (rows * tokens of the run), into the head's entry of the result
+                // The row's share of every run, normalised by its row sum, added up over the warp's rows and then,
+                // weighted by 1 / (rows * tokens of the run), into the head's entry of the result.  Lane (half, run) adds
+                // up 16 of the 32 rows, each lane starting at another row, so that no two read the same bank; the
+                // warp's runs then go out as one request, neighbouring lanes to neighbouring addresses.  (A run at a
+                // time, with a reduction by shuffles and an atomic of its own: 512 items, L = 274 and 424, 48.2 against
+                // 45.3 us per call.)
                 if (cur_run >= 0) den_rows[cur_run * kQRows + r] += run_mass;
+                __syncwarp();
                 const float inv = (r < valid_rows) ? 1.f / l : 0.f;
-                const int32_t head = st.item % heads;
-                for (int rn = 0; rn < den.n_runs; ++rn) {
-                    float v = den_rows[rn * kQRows + r] * inv;
-                    den_rows[rn * kQRows + r] = 0.f;   // the next unit starts from zero
+                static_assert(kMaxDenRuns == 16, "a lane per run and half of the rows");
+                const int rn = lane & 15;
+                float v = 0.f;
 #pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                    if (lane == 0) atomicAdd(den.out + (int64_t)head * den.n_runs + rn, (double)v * (double)den.weight[rn]);
+                for (int i = 0; i < 16; ++i) {
+                    const int row = (lane & 16) + ((i + rn) & 15);
+                    float* e = den_rows + rn * kQRows + wq * 32 + row;
+                    v = fmaf(*e, __shfl_sync(0xffffffffu, inv, row), v);
+                    *e = 0.f;   // the next unit starts from zero
                 }
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                if (lane < den.n_runs)
+                    atomicAdd(den.out + (int64_t)(st.item % heads) * den.n_runs + lane, (double)v * (double)den.weight[lane]);
+                __syncwarp();
             }
             tc_fence_before();   // orders the reads of O before the arrival on p_full for the next unit's first tile
             ++un;
@@ -1061,9 +1121,12 @@ template <int D, bool kExt, bool kWide, bool kDen, bool kLazy, bool kShort, bool
 cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorMap& vm, const CUtensorMap& km64,
                    const CUtensorMap& vm64, const ExtArgs& ext, const Strided& O,
                    const RangeList& ranges, int32_t T, int32_t heads, const PairPlan& pp, int32_t n_tiles, int3 qpos,
-                   float scale_log2, int* status, int sm_count, cudaStream_t stream, const DenArgs& den)
+                   float scale_log2, int* status, int sm_count, cudaStream_t stream, const DenArgs<true>& den_tables)
 {
     using C = Cfg<D, kWide, kDen>;
+    DenArgs<kDen> den;
+    if constexpr (kDen) den = den_tables;
+    else memset(&den, 0, sizeof(den));
     static SharedMemoryOptIn opt_in;
     const cudaError_t oe = opt_in.ensure(attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, (int)C::kSmemBytes);
     if (oe != cudaSuccess) return oe;
@@ -1083,7 +1146,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
                                const CurrentScaleSource* cur, const PairDensity* density)
 {
     if (ranges.n < 1 || ranges.total < 1 || T < 1) return cudaErrorInvalidValue;
-    DenArgs den;
+    DenArgs<true> den;
     memset(&den, 0, sizeof(den));
     if (density) {
         static_assert(kPairMaxDensityRuns == kMaxDenRuns, "interface and kernel disagree");
@@ -1171,7 +1234,22 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
         pp.n_pairs = pp.n_items * pp.nqt;
     }
     int32_t n_tiles = 0;
-    for (int i = 0; i < ranges.n; ++i) n_tiles += (ranges.r[i].len + kKT - 1) / kKT;
+    for (int i = 0; i < ranges.n; ++i) n_tiles += density ? ranges.r[i].len / kKT : (ranges.r[i].len + kKT - 1) / kKT;
+    if (density) {
+        den.n_whole = n_tiles;
+        int boxes = 0;
+        for (int i = 0; i < ranges.n; ++i) {
+            for (int32_t at = ranges.r[i].len / kKT * kKT; at < ranges.r[i].len; at += kKVBoxRows, ++boxes) {
+                MixedTile& m = den.mixed[boxes / 4];
+                const int b = boxes % 4;
+                m.keep |= ((1ull << std::min(kKVBoxRows, ranges.r[i].len - at)) - 1ull) << (b * kKVBoxRows);
+                m.tok[b] = ranges.r[i].start + at;
+                m.runs |= (uint32_t)den.run_of_range[i] << (8 * b);
+                m.boxes = b + 1;
+            }
+        }
+        n_tiles += (boxes + 3) / 4;
+    }
     const int3 qpos = make_int3(pos[0], pos[1], pos[2]);
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
     // 64 channels take the two-CTA form once there are units for it: the wide form was measured on the tensor-bound launches

@@ -9,7 +9,7 @@ import oracle
 from paper_2511_16047_b200 import binding as B
 from paper_2511_16047_b200 import synth
 
-from gpu_common import Cache, make_qkv, to_items
+from gpu_common import Cache, check_close, make_qkv, to_items
 
 pytestmark = pytest.mark.gpu
 
@@ -94,4 +94,35 @@ def test_density_as_a_by_product_of_the_attention_launch(D, peaked):
                 assert np.allclose(got, want, rtol=2e-4, atol=1e-7), (layer, k, np.abs(got / want - 1).max())
                 counts = np.array([n for _, _, n in runs], dtype=np.float64)
                 assert np.allclose(got @ counts, sides[k] ** 2, rtol=1e-4)
+        assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("rows,budgets", [(1, None), (3, None), (2, [(70, 5), (40, 0), (130, 20)])], ids=["r1", "r3", "tokens"])
+def test_key_tiles_of_several_runs(D, rows, budgets):
+    """The paired kernel packs what whole 64-token tiles leave of each run into tiles of four 16-token boxes: runs of 1, 16,
+    49 (four boxes, one key in the last), 64 (none left), 81 and 121 tokens, and the pieces of rings cut anywhere."""
+    sides, heads, scale = (1, 4, 7, 8, 9, 11), 3, 1.0 / math.sqrt(D)
+    pols = [(1, 1, False), (2, 3, False), (0, 9, True)]
+    qkv = make_qkv(rows, heads, sides, D, seed=95, peaked=True)
+    Ks, Vs = [to_items(k) for _, k, _ in qkv], [to_items(v) for _, _, v in qkv]
+    with Cache(len(pols), heads, D, rows, sides, pols, token_budgets=budgets) as c:
+        B.amskv_set_attend_path(c.h, B.PATH_TENSOR_PAIR)
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(pols)):
+                B.amskv_append(c.h, layer, k, kk, v)
+                runs = B.amskv_attended_tokens(c.h, layer, k)
+                out = torch.full_like(q, float("nan"))
+                den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+                n0 = B.amskv_launch_count()
+                B.amskv_attend_density(c.h, layer, k, q, out, den, den.numel())
+                assert B.amskv_launch_count() - n0 == 2      # the result zeroed, one attention launch
+                torch.cuda.synchronize()
+                tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
+                check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, scale), "layer %d scale %d" % (layer, k), max_abs=4e-2)
+                want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
+                # A run of one key is as exact as that key's exponential, and every sixth pair's comes from the cubic
+                # sum of f^n (ln 2)^n / n!, n <= 3, |f| <= 1/2: at most 7.9e-4 of 2^f too small (f = -1/2).  Longer
+                # runs and more rows average it down to the 2e-4 asked for above.
+                assert np.allclose(den.cpu().numpy(), want, rtol=1e-3, atol=1e-7), (layer, k)
         assert B.amskv_status(c.h) == 0

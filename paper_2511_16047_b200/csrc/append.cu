@@ -9,6 +9,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kUnroll = 4;
+static_assert(kThreads * kUnroll == kAppendBlockChunks, "blocks of a copy, as the launch rules count them");
 
 template <int D>
 __global__ void __launch_bounds__(kThreads)
@@ -16,6 +17,7 @@ append_kernel(const uint4* __restrict__ Ksrc, const uint4* __restrict__ Vsrc, in
               int64_t k_tok, int64_t v_row, int64_t v_head, int64_t v_tok, uint4* __restrict__ dst, int32_t capacity,
               int32_t token_offset, int32_t T, int32_t heads, int64_t total_chunks)
 {
+    overlap_with_previous();
     constexpr int CPT = D / 8;  // 16-byte chunks per token
     const int64_t chunks_per_item = (int64_t)T * CPT;
     const int64_t item_stride = 2ll * capacity * CPT;     // chunks
@@ -188,7 +190,12 @@ cudaError_t launch_append(const Strided& K, const Strided& V, const LayerRegion&
     int64_t blocks = (total + (int64_t)kThreads * kUnroll - 1) / ((int64_t)kThreads * kUnroll);
     if (blocks > (1 << 20)) blocks = 1 << 20;
     auto* dst = reinterpret_cast<uint4*>(region.base);
-    return launch_kernel(false, D == 64 ? append_kernel<64> : append_kernel<128>, dim3((unsigned)blocks), dim3(kThreads), 0, stream,
+    // A copy of a few blocks is mostly launch latency and overlaps the kernel before it: 64 channels, T = 25, 60 items 6.6 -> 6.1
+    // us per append and attend, T = 16, 32 items 6.1 -> 5.9. Not beyond a third of the SMs, where the small L1 that the attention
+    // kernel leaves (launch_kernel) costs more (T = 36, 256 items, 72 blocks: 8.7 -> 10.2), and not with 128 channels (T = 36,
+    // 32 items: 6.9 -> 7.2).
+    const bool overlap = D == 64 && 3 * blocks <= sm_count;
+    return launch_kernel(overlap, D == 64 ? append_kernel<64> : append_kernel<128>, dim3((unsigned)blocks), dim3(kThreads), 0, stream,
                          (const uint4*)K.ptr, (const uint4*)V.ptr, K.row, K.head, K.token, V.row, V.head, V.token, dst,
                          region.capacity, token_offset, T, heads, total);
 }

@@ -561,7 +561,7 @@ cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerReg
     if (T < 1 || ranges.total + ext.len < 1) return cudaErrorInvalidValue;
     const int64_t items = (int64_t)rows * heads;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
-    const bool overlap = cur || density;   // (a density launch follows the kernel that zeroes its result)
+    const bool overlap = cur || density || overlaps_append(items, T, D, sm_count);   // (a density launch follows the kernel that zeroes its result)
 #define AMSKV_MID_LAUNCH(DD, NN, DEN) return launch<DD, NN, DEN>(overlap, Q, O, region, ranges, T, heads, items, scale_log2, ext, den, stream)
     if (D == 128) {
         if (density) AMSKV_MID_LAUNCH(128, 4, true);

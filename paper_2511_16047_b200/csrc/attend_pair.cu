@@ -1133,7 +1133,11 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
     if (kSplit) grid = pp.full > 0 ? ((int64_t)sm_count * C::kCtasPerSm) & ~1ll : 2ll * pp.n_pairs;
     else if (grid > pp.n_pairs) grid = pp.n_pairs;
-    return launch_kernel(kExt || kDen, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
+    // (With a second round for less than half of the CTAs it matters that those with two units do not share SMs: launched onto
+    // an idle chip they do not, but onto SMs that come free one by one they do: T = 361, 256 items 49.9 -> 54.6 us.)
+    const int64_t slots = (int64_t)sm_count * C::kCtasPerSm;
+    const bool overlap = kExt || kDen || (overlaps_append(pp.n_items, T, D, sm_count) && (pp.n_pairs <= slots || 2 * (int64_t)pp.n_pairs > 3 * slots));
+    return launch_kernel(overlap, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
                          KernelMemory(C::kSmemBytes, kSplit ? 2u : 1u), stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
                          ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);
 }

@@ -338,9 +338,10 @@ cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerR
     }
     const int64_t blocks = (items + kWarpsPerCta - 1) / kWarpsPerCta;
     const float scale_log2 = softmax_scale * 1.4426950408889634f;
+    const bool overlap = cur || overlaps_append(items, T, D, sm_count);
     const bool early = D == 128 || items <= (int64_t)sm_count * 12;   // (all items resident at once; see the kernel)
 #define AMSKV_SMALL_LAUNCH(DD, EXT, TILES, EARLY)                                                                             \
-    return launch_kernel(EXT, attend_small_kernel<DD, EXT, TILES, EARLY>, dim3((unsigned)blocks), dim3(kWarpsPerCta * 32), 0, stream,\
+    return launch_kernel(overlap, attend_small_kernel<DD, EXT, TILES, EARLY>, dim3((unsigned)blocks), dim3(kWarpsPerCta * 32), 0, stream,\
                          (const __nv_bfloat16*)Q.ptr, Q.row, Q.head, Q.token, (__nv_bfloat16*)O.ptr, O.row, O.head,           \
                          O.token, region.base, region.capacity, ranges, T, heads, (int32_t)items, scale_log2, ext)
 #define AMSKV_SMALL_TILES(DD, EXT)                                                                                            \

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) zero_kernel(double* __restrict__ p, int64
 cudaError_t launch_zero(double* p, size_t n, cudaStream_t stream)
 {
     const unsigned blocks = n > 256 * 64 ? 64u : (unsigned)((n + 255) / 256);
-    return launch_kernel(false, zero_kernel, dim3(blocks > 0 ? blocks : 1u), dim3(256), 0, stream, p, (int64_t)n);
+    return launch_kernel(true, zero_kernel, dim3(blocks > 0 ? blocks : 1u), dim3(256), 0, stream, p, (int64_t)n);
 }
 
 cudaError_t launch_density(const Strided& Q, const LayerRegion& region, const DensityPieces& pieces, int32_t T,

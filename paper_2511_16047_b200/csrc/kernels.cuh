@@ -164,10 +164,11 @@ void count_launch(int n = 1);
 // several hundred microseconds are unchanged.  It lets the next kernel in only after its own wait: released before it,
 // kernels pile up two and three deep, and the CTAs of the later ones take the free SMs (T = 256, 60 items: 14.6 -> 15.3 us
 // a call; released after it: 13.2).
-// overlap = false launches the ordinary way: the append copies and the attention of amskv_attend, which normally follows
-// its scale's append.  Copies that start on SMs still configured for the attention kernel's shared memory keep their small
-// L1, which is where their loads in flight are held, and attention CTAs placed beside the last blocks of a copy find an SM
-// with its shared-memory split, which only an idle SM can change (T = 256, 1 920 items, a copy before each: +4 to +9 %).
+// overlap = false launches the ordinary way: all but the smallest append copies, and the attention of amskv_attend, which
+// normally follows its scale's append, where that copy is large (overlaps_append).  Copies that start on SMs still
+// configured for the attention kernel's shared memory keep their small L1, which is where their loads in flight are held,
+// and attention CTAs placed beside the last blocks of a copy find an SM with its shared-memory split, which only an idle SM
+// can change (T = 256, 1 920 items, a copy before each: +4 to +9 %).
 struct KernelMemory {     // dynamic shared memory, and the CTAs of a cluster (1: no clusters)
     size_t bytes;
     unsigned cluster;
@@ -206,6 +207,15 @@ __device__ __forceinline__ void overlap_with_previous()
     asm volatile("griddepcontrol.launch_dependents;");
 }
 #endif
+
+// The attention of amskv_attend overlaps the copy of its scale's append where all blocks of that copy are resident at once
+// (eight per SM): us per append and attend, 64 channels: 60 items T = 100 11.5 -> 9.7, 256 items T = 64 12.5 -> 11.7, 512 items
+// T = 169 34.7 -> 33.2, 1 110 items T = 100 32.7 -> 31.3; beyond, 1 920 items T = 256 140 -> 147, 3 840 items T = 361 567 -> 591.
+constexpr int kAppendBlockChunks = 1024;   // 16-byte chunks of K (and of V) a block of the copy moves
+inline bool overlaps_append(int64_t items, int32_t T, int32_t D, int sm_count)
+{
+    return items * T * (D / 8) <= 8ll * kAppendBlockChunks * sm_count;
+}
 
 // A kernel's dynamic shared-memory limit is a per-device setting: raised once per device and kernel,
 // from whichever host thread gets there first (setting it twice is harmless).

@@ -276,3 +276,24 @@ def test_full_size_rows_sampled_against_oracle():
                 check_close(pick(outs[layer][k]), want[k], "full-size layer %d scale %d" % (layer, k))
         # resident KV bytes equal the closed form for these two layers
         assert B.amskv_cache_bytes(cache.h)[1] == oracle.kv_bytes(wl.sides, pols, wl.rows, wl.heads, wl.head_dim)
+
+
+@pytest.mark.parametrize("rows", [1, 16, 64, 65])
+def test_attention_that_starts_while_its_append_ends(rows):
+    """Append and attend of several layers enqueued back to back, twice over the same slots: the copy overlaps the attention
+    before it up to 49 blocks (rows = 1), the attention overlaps the copy up to 8 blocks per SM (64 x 37 items x 64 tokens
+    are 1184) and not beyond.  Every output depends on the copy enqueued just before it."""
+    sides, heads, D = (4, 8), 37, 64
+    qkv = make_qkv(rows, heads, sides, D, seed=97)
+    pols = [(1, 2, False)] * 3
+    pick = [0, rows * heads // 2, rows * heads - 1]
+    take = lambda x: x.reshape(rows * heads, -1, D)[pick]
+    with Cache(len(pols), heads, D, rows, sides, pols) as c:
+        for flip in (False, True):                             # the second pass stores other keys and values where the first did
+            data = [(q, v, kk) if flip else (q, kk, v) for q, kk, v in qkv]
+            outs = run_pass(c, data)
+            items = [take(x).cpu().double().numpy() for t in data for x in t]
+            for k in range(len(sides)):
+                want = oracle.attend_selected(items[3 * k], items[1:3 * k + 3:3], items[2:3 * k + 3:3], oracle.keep_set(k, 1, 2, False), 0.125)
+                for layer in range(len(pols)):
+                    check_close(take(outs[layer][k]), want, "rows %d layer %d scale %d" % (rows, layer, k))

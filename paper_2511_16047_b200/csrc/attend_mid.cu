@@ -567,6 +567,11 @@ cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerReg
         if (density) AMSKV_MID_LAUNCH(128, 4, true);
         AMSKV_MID_LAUNCH(128, 4, false);
     }
+    // Densities of one query block: a CTA of four warps has two idle, which matters once an SM's share of the items is more than the
+    // four such CTAs it holds (T = 4, 9, 16: 1 920 items 17.7 / 20.3 / 22.4 us with four warps, 14.6 / 17.0 / 18.8 with two; 7 680
+    // items 54 / 60 / 68 and 40 / 45 / 51); below, twice the threads fetch the keys sooner (256 items 7.9 / 8.1 / 8.4 and 8.2 / 8.4 /
+    // 8.9).
+    if (density && T <= 16 && items > 4ll * sm_count) AMSKV_MID_LAUNCH(64, 2, true);
     // Four query blocks per CTA; two where there are no more, or where that still gives no SM a second CTA (T = 25, 512 items:
     // 6.3 us with 4 warps, 8.6 with 8; T = 64, 60 items: 5.1 and 5.8; T = 64, 256 items: 9.3 and 8.9).
     if (T <= 32 || items * ((T + 31) / 32) <= sm_count) {

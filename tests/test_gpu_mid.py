@@ -165,3 +165,24 @@ def test_last_round_shared_by_two_ctas(rows, heads, sides, fused):
             check_close(got, want[k], "scale %d" % k, max_abs=4e-2)
         again = run_pass(c, qkv, B.PATH_TENSOR_PAIR, fused=fused)
         assert all(torch.equal(x, y) for x, y in zip(outs[0], again[0]))
+
+
+@pytest.mark.parametrize("rows", [16, 17])
+def test_densities_of_one_query_block_with_two_and_with_four_warps(rows):
+    """One query block per CTA: two warps with more than four items per SM (148 x 4 = 592), four up to there."""
+    sides, heads, D = (1, 3, 4, 4, 4, 4), 37, 64               # 592 and 629 items; one and two key chunks
+    qkv = make_qkv(rows, heads, sides, D, seed=98)
+    Ks, Vs = [to_items(k) for _, k, _ in qkv], [to_items(v) for _, _, v in qkv]
+    with Cache(1, heads, D, rows, sides, [(0, 9, True)]) as c:
+        for k, (q, kk, v) in enumerate(qkv):
+            B.amskv_append(c.h, 0, k, kk, v)
+            runs = B.amskv_attended_tokens(c.h, 0, k)
+            out = torch.full_like(q, float("nan"))
+            den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+            B.amskv_attend_density(c.h, 0, k, q, out, den, den.numel())
+            torch.cuda.synchronize()
+            tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
+            check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, 0.125), "scale %d" % k)
+            want = oracle.attention_density(to_items(q), Ks, runs, 0.125, heads)
+            assert np.allclose(den.cpu().numpy(), want, rtol=2e-4, atol=1e-7), k
+        assert B.amskv_status(c.h) == 0

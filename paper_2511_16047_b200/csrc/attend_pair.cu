@@ -85,7 +85,9 @@ struct Cfg {
     static constexpr int kCtasPerSm = kWide ? 1 : 2;
     // Extents every address in the kernel is derived from, checked at compile time:
     //  - tensor memory: S buffers of both streams, then O of both streams, inside the allocation, and the
-    //    allocations of all CTAs of an SM inside its 512 columns (otherwise tcgen05.alloc would block);
+    //    allocations of all CTAs of an SM inside its 512 columns (otherwise tcgen05.alloc would block; a CTA of
+    //    another form, from the launch before or behind, may make it block until one of the two ends, which both
+    //    do: a launch lets the next one in only when all its CTAs own their columns);
     //  - shared memory: the CTAs of an SM (each with 1 KB reserved by the system) inside 228 KB;
     //  - matrix descriptors: a start address is 14 bits of 16-byte units (256 KB), so adding a stage, half
     //    or K-step offset to the low descriptor word can never carry into the field above it.
@@ -308,8 +310,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     }
     tc_fence_before();
     // everything up to here touches only this CTA's own memory, so it runs while the kernel before this one ends
-    overlap_with_previous();
+    wait_for_previous();
     __syncthreads();
+    // The next kernel comes in only now that this CTA owns its tensor memory.  Let in earlier, a CTA of it could take columns
+    // that this one is still waiting for, and keep them while it waits for this launch to end.
+    let_next_start();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
     // (in a density launch `valid` also carries the tile's run, or that the tile is a mixed one; tile_run() strips that)

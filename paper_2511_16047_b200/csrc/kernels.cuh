@@ -201,10 +201,14 @@ cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), dim3 grid, dim3 bl
     return e;
 }
 #ifdef __CUDACC__
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A kernel that allocates tensor memory calls this behind a barrier that follows the allocation: the CTAs it lets in may
+// allocate at once, and then hold their columns until this launch has ended.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void overlap_with_previous()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    wait_for_previous();
+    let_next_start();
 }
 #endif
 

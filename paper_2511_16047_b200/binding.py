@@ -99,9 +99,8 @@ def _load() -> ctypes.CDLL:
 lib = _load()
 try:
     from . import _steps
-except ImportError as e:
-    raise ImportError("the binding's _steps module is not built for this interpreter: run "
-                      "`python paper_2511_16047_b200/build.py`") from e
+except ImportError:   # not built for this interpreter: every call goes through ctypes
+    _steps = None
 EXPORTS = ("amskv_cache_required_bytes amskv_cache_create amskv_cache_destroy amskv_cache_reset amskv_append "
            "amskv_attend amskv_append_attend amskv_attention_density amskv_attend_density amskv_first_overflow_scale amskv_promote_layer amskv_set_attend_path amskv_step_host amskv_step_staging_bytes amskv_layer_similarity "
            "amskv_similarity_workspace_bytes amskv_layer_similarity_static amskv_classify_by_threshold amskv_classify_lowest "
@@ -119,8 +118,16 @@ def _check(code: int, where: str) -> None:
         raise AmskvError(code, where)
 
 
-# The calls of a generation step go through the _steps module, which takes addresses and strides out of the tensors natively.
-_steps.bind(*(ctypes.cast(fn, ctypes.c_void_p).value for fn in (lib.amskv_append, lib.amskv_attend, lib.amskv_append_attend)))
+# The calls of a generation step go through the _steps module where it is built, which takes addresses and strides out of the
+# tensors natively; it returns None for arguments of other than the usual forms, and the call is made through ctypes.
+if _steps is not None:
+    _steps.bind(*(ctypes.cast(fn, ctypes.c_void_p).value for fn in (lib.amskv_append, lib.amskv_attend, lib.amskv_append_attend)))
+
+
+def _int32(name: str, x) -> None:
+    """ctypes would take the low 32 bits of a longer int."""
+    if type(x) is int and not -2 ** 31 <= x < 2 ** 31:
+        raise OverflowError("%s out of range" % name)
 
 
 def _addr(x) -> Optional[int]:
@@ -201,21 +208,38 @@ def amskv_cache_reset(cache: int) -> None:
     _check(lib.amskv_cache_reset(cache), "amskv_cache_reset")
 
 
+def _kv_strides(K, V):
+    ks, vs = _strides(K), _strides(V)
+    if (ks is None) != (vs is None) or (ks is not None and list(ks) != list(vs)):
+        raise ValueError("K and V must share one stride triple")
+    return ks
+
+
 def amskv_append(cache: int, layer: int, scale: int, K, V, stream=None) -> None:
-    rc = _steps.append(cache, layer, scale, K, V, stream)
+    rc = _steps.append(cache, layer, scale, K, V, stream) if _steps is not None else None
+    if rc is None:
+        _int32("layer", layer), _int32("scale", scale)
+        rc = lib.amskv_append(cache, layer, scale, _addr(K), _addr(V), _kv_strides(K, V), _stream(stream))
     if rc:
         raise AmskvError(rc, "amskv_append")
 
 
 def amskv_attend(cache: int, layer: int, scale: int, Q, out, stream=None) -> None:
-    rc = _steps.attend(cache, layer, scale, Q, out, stream)
+    rc = _steps.attend(cache, layer, scale, Q, out, stream) if _steps is not None else None
+    if rc is None:
+        _int32("layer", layer), _int32("scale", scale)
+        rc = lib.amskv_attend(cache, layer, scale, _addr(Q), _addr(out), _strides(Q), _strides(out), _stream(stream))
     if rc:
         raise AmskvError(rc, "amskv_attend")
 
 
 def amskv_append_attend(cache: int, layer: int, scale: int, K, V, Q, out, stream=None) -> None:
     """append(layer, scale, K, V) then attend(layer, scale, Q, out), as one launch where possible."""
-    rc = _steps.append_attend(cache, layer, scale, K, V, Q, out, stream)
+    rc = _steps.append_attend(cache, layer, scale, K, V, Q, out, stream) if _steps is not None else None
+    if rc is None:
+        _int32("layer", layer), _int32("scale", scale)
+        rc = lib.amskv_append_attend(cache, layer, scale, _addr(K), _addr(V), _kv_strides(K, V), _addr(Q), _addr(out),
+                                     _strides(Q), _strides(out), _stream(stream))
     if rc:
         raise AmskvError(rc, "amskv_append_attend")
 

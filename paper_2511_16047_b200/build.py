@@ -38,8 +38,15 @@ def build_steps(force: bool = False) -> str:
     if not force and os.path.exists(STEPS) and os.path.getmtime(STEPS) >= os.path.getmtime(STEPS_SOURCE):
         return STEPS
     tmp = STEPS + ".tmp.%d" % os.getpid()
-    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
-                           "-I" + sysconfig.get_paths()["include"], STEPS_SOURCE, "-o", tmp])
+    try:
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden",
+                               "-I" + sysconfig.get_paths()["include"], STEPS_SOURCE, "-o", tmp])
+    except (OSError, subprocess.CalledProcessError) as e:
+        # no C compiler or no Python headers here: the binding then goes through ctypes alone
+        sys.stderr.write("_steps not built (%s): the calls of a step go through ctypes\n" % e)
+        if os.path.exists(STEPS):
+            os.remove(STEPS)   # not one of older sources
+        return ""
     os.replace(tmp, STEPS)
     return STEPS
 

@@ -1,10 +1,13 @@
 /* Python side of the calls of a generation step (amskv_append, amskv_attend, amskv_append_attend): takes addresses and strides
- * out of the tensors and calls the library, without the argument conversions of ctypes.  Marshalling only.
+ * out of the tensors and calls the library, without the argument conversions of ctypes.  Marshalling only, and only of the
+ * usual forms: a call with any other argument returns None without having called the library, and the binding makes it
+ * through ctypes, which decides what is accepted and what the error is.
  *
  * These calls are made layers x scales times per image; through ctypes their Python side took 2.1 us with contiguous tensors
  * and 3.3 us with views, about what the launch itself takes; here 0.8 and 1.4.
  *
- * A tensor argument is anything with data_ptr(), is_contiguous() and stride() (a torch tensor), an address (int), or None.
+ * The usual forms: a handle, layer, scale or address that is exactly an int (None as an address), a tensor with data_ptr(),
+ * is_contiguous() and stride() (a torch tensor), a stream that is None, an int or has an int as .cuda_stream.
  * The library's functions are handed over by bind() as addresses, so this module is independent of where it was loaded from.
  */
 #define PY_SSIZE_T_CLEAN
@@ -20,17 +23,17 @@ static attend_fn f_attend;
 static append_attend_fn f_append_attend;
 static PyObject *s_data_ptr, *s_is_contiguous, *s_stride, *s_cuda_stream;
 
-static int as_pointer(PyObject* o, void** out) /* an int (or what __index__ makes one), or None */
+/* The helpers below return 0, or -1 for an argument that is left to ctypes (with or without an error set). */
+
+static int as_pointer(PyObject* o, void** out) /* an int, or None */
 {
     if (o == Py_None) {
         *out = NULL;
         return 0;
     }
-    PyObject* i = PyNumber_Long(o);
-    if (!i) return -1;
-    *out = (void*)(uintptr_t)PyLong_AsUnsignedLongLongMask(i);
-    Py_DECREF(i);
-    return PyErr_Occurred() ? -1 : 0;
+    if (!PyLong_CheckExact(o)) return -1;
+    *out = (void*)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
+    return 0;
 }
 
 /* address of a tensor argument; strides[3] and *strided = 1 when it is a view that is not contiguous */
@@ -39,45 +42,33 @@ static int tensor(PyObject* x, void** addr, int64_t* strides, int* strided)
     *strided = 0;
     if (x == Py_None || PyLong_CheckExact(x)) return as_pointer(x, addr);
     PyObject* r = PyObject_CallMethodNoArgs(x, s_data_ptr);
-    if (!r) {
-        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return -1;
-        PyErr_Clear();
-        return as_pointer(x, addr);
-    }
-    int bad = as_pointer(r, addr);
+    if (!r) return -1;
+    const int bad = as_pointer(r, addr);
     Py_DECREF(r);
     if (bad) return -1;
     r = PyObject_CallMethodNoArgs(x, s_is_contiguous);
-    if (!r) {
-        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return -1;
-        PyErr_Clear();   /* something with an address only */
-        return 0;
-    }
-    const int contiguous = PyObject_IsTrue(r);
+    if (!r) return -1;
+    const int contiguous = r == Py_True ? 1 : r == Py_False ? 0 : -1;
     Py_DECREF(r);
     if (contiguous) return contiguous < 0 ? -1 : 0;
     r = PyObject_CallMethodNoArgs(x, s_stride);
     if (!r) return -1;
-    if (!PyTuple_Check(r) || PyTuple_GET_SIZE(r) != 4 || PyLong_AsLongLong(PyTuple_GET_ITEM(r, 3)) != 1) {
-        if (!PyErr_Occurred()) PyErr_SetString(PyExc_AssertionError, "expected [rows, heads, T, D] with contiguous channels");
-        Py_DECREF(r);
-        return -1;
+    int ok = PyTuple_Check(r) && PyTuple_GET_SIZE(r) == 4;
+    for (int i = 0; ok && i < 4; ++i) {
+        const long long v = PyLong_AsLongLong(PyTuple_GET_ITEM(r, i));
+        if (i < 3) strides[i] = v;
+        ok = i < 3 ? !PyErr_Occurred() : v == 1;
     }
-    for (int i = 0; i < 3; ++i) strides[i] = PyLong_AsLongLong(PyTuple_GET_ITEM(r, i));
     Py_DECREF(r);
     *strided = 1;
-    return PyErr_Occurred() ? -1 : 0;
+    return ok ? 0 : -1;
 }
 
 static int stream_of(PyObject* s, void** out) /* None, an address, or something with .cuda_stream */
 {
     if (s == Py_None || PyLong_CheckExact(s)) return as_pointer(s, out);
     PyObject* a = PyObject_GetAttr(s, s_cuda_stream);
-    if (!a) {
-        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return -1;
-        PyErr_Clear();
-        return as_pointer(s, out);
-    }
+    if (!a) return -1;
     const int bad = as_pointer(a, out);
     Py_DECREF(a);
     return bad;
@@ -85,16 +76,11 @@ static int stream_of(PyObject* s, void** out) /* None, an address, or something 
 
 static int head(PyObject* const* args, void** cache, int* layer, int* scale)
 {
-    if (as_pointer(args[0], cache)) return -1;
+    if (as_pointer(args[0], cache) || !PyLong_CheckExact(args[1]) || !PyLong_CheckExact(args[2])) return -1;
     const long l = PyLong_AsLong(args[1]), s = PyLong_AsLong(args[2]);
-    if (PyErr_Occurred()) return -1;
     *layer = (int)l;
     *scale = (int)s;
-    if (l != *layer || s != *scale) {
-        PyErr_SetString(PyExc_OverflowError, "layer or scale out of range");
-        return -1;
-    }
-    return 0;
+    return PyErr_Occurred() || l != *layer || s != *scale ? -1 : 0;
 }
 
 static int key_value(PyObject* K, PyObject* V, void** k, void** v, int64_t* ks, int* strided)
@@ -102,11 +88,7 @@ static int key_value(PyObject* K, PyObject* V, void** k, void** v, int64_t* ks, 
     int64_t vs[3];
     int v_strided;
     if (tensor(K, k, ks, strided) || tensor(V, v, vs, &v_strided)) return -1;
-    if (*strided != v_strided || (*strided && (ks[0] != vs[0] || ks[1] != vs[1] || ks[2] != vs[2]))) {
-        PyErr_SetString(PyExc_ValueError, "K and V must share one stride triple");
-        return -1;
-    }
-    return 0;
+    return *strided != v_strided || (*strided && (ks[0] != vs[0] || ks[1] != vs[1] || ks[2] != vs[2])) ? -1 : 0;
 }
 
 static int count(Py_ssize_t n, Py_ssize_t want)
@@ -116,44 +98,53 @@ static int count(Py_ssize_t n, Py_ssize_t want)
     return -1;
 }
 
-/* append(cache, layer, scale, K, V, stream) -> return code */
+static PyObject* left_to_ctypes(void)
+{
+    PyErr_Clear();
+    Py_RETURN_NONE;
+}
+
+/* append(cache, layer, scale, K, V, stream) -> return code, or None */
 static PyObject* py_append(PyObject* self, PyObject* const* args, Py_ssize_t n)
 {
     void *cache, *k, *v, *stream;
     int layer, scale, kv, rc;
     int64_t ks[3];
-    if (count(n, 6) || head(args, &cache, &layer, &scale) || key_value(args[3], args[4], &k, &v, ks, &kv) || stream_of(args[5], &stream))
-        return NULL;
+    if (count(n, 6)) return NULL;
+    if (head(args, &cache, &layer, &scale) || key_value(args[3], args[4], &k, &v, ks, &kv) || stream_of(args[5], &stream))
+        return left_to_ctypes();
     Py_BEGIN_ALLOW_THREADS
     rc = f_append(cache, layer, scale, k, v, kv ? ks : NULL, stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
 
-/* attend(cache, layer, scale, Q, out, stream) -> return code */
+/* attend(cache, layer, scale, Q, out, stream) -> return code, or None */
 static PyObject* py_attend(PyObject* self, PyObject* const* args, Py_ssize_t n)
 {
     void *cache, *q, *o, *stream;
     int layer, scale, qv, ov, rc;
     int64_t qs[3], os[3];
-    if (count(n, 6) || head(args, &cache, &layer, &scale) || tensor(args[3], &q, qs, &qv) || tensor(args[4], &o, os, &ov) ||
+    if (count(n, 6)) return NULL;
+    if (head(args, &cache, &layer, &scale) || tensor(args[3], &q, qs, &qv) || tensor(args[4], &o, os, &ov) ||
         stream_of(args[5], &stream))
-        return NULL;
+        return left_to_ctypes();
     Py_BEGIN_ALLOW_THREADS
     rc = f_attend(cache, layer, scale, q, o, qv ? qs : NULL, ov ? os : NULL, stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
 
-/* append_attend(cache, layer, scale, K, V, Q, out, stream) -> return code */
+/* append_attend(cache, layer, scale, K, V, Q, out, stream) -> return code, or None */
 static PyObject* py_append_attend(PyObject* self, PyObject* const* args, Py_ssize_t n)
 {
     void *cache, *k, *v, *q, *o, *stream;
     int layer, scale, kv, qv, ov, rc;
     int64_t ks[3], qs[3], os[3];
-    if (count(n, 8) || head(args, &cache, &layer, &scale) || key_value(args[3], args[4], &k, &v, ks, &kv) ||
-        tensor(args[5], &q, qs, &qv) || tensor(args[6], &o, os, &ov) || stream_of(args[7], &stream))
-        return NULL;
+    if (count(n, 8)) return NULL;
+    if (head(args, &cache, &layer, &scale) || key_value(args[3], args[4], &k, &v, ks, &kv) || tensor(args[5], &q, qs, &qv) ||
+        tensor(args[6], &o, os, &ov) || stream_of(args[7], &stream))
+        return left_to_ctypes();
     Py_BEGIN_ALLOW_THREADS
     rc = f_append_attend(cache, layer, scale, k, v, kv ? ks : NULL, q, o, qv ? qs : NULL, ov ? os : NULL, stream);
     Py_END_ALLOW_THREADS
@@ -169,9 +160,8 @@ static PyObject* py_bind(PyObject* self, PyObject* const* args, Py_ssize_t n)
         return NULL;
     }
     for (int i = 0; i < 3; ++i) {
-        if (as_pointer(args[i], &f[i])) return NULL;
-        if (!f[i]) {
-            PyErr_SetString(PyExc_ValueError, "null function");
+        if (as_pointer(args[i], &f[i]) || !f[i]) {
+            PyErr_SetString(PyExc_ValueError, "bind() wants addresses");
             return NULL;
         }
     }

@@ -54,3 +54,32 @@ def test_mismatched_and_malformed_tensors_are_refused():
     with pytest.raises(OverflowError):
         B.amskv_append(c, 1 << 40, 0, k, v)
     B.amskv_cache_destroy(c)
+
+
+@pytest.mark.parametrize("native", [True, False], ids=["native", "ctypes"])
+def test_what_ctypes_takes_the_step_calls_take(native, monkeypatch):
+    """The native module serves the usual forms of arguments and leaves every other to ctypes: a handle object is accepted,
+    what ctypes refuses is refused, and without the module everything goes through ctypes."""
+    import ctypes
+    if not native:
+        monkeypatch.setattr(B, "_steps", None)
+    c = _plan(layers=2, sides=(1, 2))
+    q, k, v = _views(1)
+    B.amskv_append(ctypes.c_void_p(c), 0, 0, k, v)
+    B.amskv_append_attend(ctypes.c_void_p(c), 1, 0, k, v, q, q)
+    B.amskv_append(c, ctypes.c_int(0), True, k.data_ptr(), ctypes.c_void_p(k.data_ptr()).value)
+    assert B.amskv_kept_segments(c, 0, 1) == [0, 1]
+    for bad in (float(c), torch.tensor(1)):
+        with pytest.raises((TypeError, ctypes.ArgumentError)):
+            B.amskv_append(bad, 1, 1, k, v)
+    for bad in (1.0, "1"):
+        with pytest.raises((TypeError, ctypes.ArgumentError)):
+            B.amskv_append(c, 1, bad, k, v)
+    with pytest.raises(ValueError):
+        B.amskv_append(c, 1, 1, k, v.contiguous())
+    with pytest.raises(AssertionError):
+        B.amskv_attend(c, 1, 0, q.transpose(2, 3), q)
+    with pytest.raises(OverflowError):
+        B.amskv_attend(c, 0, 1 << 31, q, q)
+    B.amskv_append(c, 1, 1, k, v)                                      # none of them went through
+    B.amskv_cache_destroy(c)

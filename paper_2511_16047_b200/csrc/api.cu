@@ -631,7 +631,7 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
         PairDensity den;
         den.out = density;
         den.n_runs = n_runs;
-        for (int32_t r = 0; r < n_runs; ++r) den.weight[r] = (float)(1.0 / ((double)cache->rows * (double)runs[r].count));
+        for (int32_t r = 0; r < n_runs; ++r) den.weight[r] = 1.0 / ((double)cache->rows * (double)runs[r].count);
         ranges.n = n;
         ranges.total = total;
         for (int32_t i = 0; i < n; ++i) {

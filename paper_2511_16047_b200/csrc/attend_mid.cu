@@ -15,8 +15,11 @@
 // it by more than 2^8; the two halves of the keys are merged through shared memory at the end.
 //
 // Attention density (kDen): the mass of a row on each of up to 16 runs of keys is P times a 0/1 matrix of run membership,
-// two more column tiles of the second product.  P enters as the sum of two bf16 numbers, so the masses are those of the
-// unrounded probabilities to 2^-16.
+// two more column tiles of the second product.  P enters as the sum of three bf16 numbers, which hold all 24 bits of the fp32
+// probabilities; a step's products go into accumulators of their own, added up in fp32 with rounding (the tensor pipe
+// truncates), and rows are added up in fp64.  With two terms, one accumulator and fp32 sums and weights the masses were off by
+// 1.4e-7 (480 items, T = 4) and 4.6e-7 (32 items; 1.7e-6 at a single entry); with these by 6e-9 and 1.5e-8, the CUDA-core pass by
+// 6e-9 and 2.4e-8.  512 items, T = 16: 8.9 -> 9.2 us a call.
 #include <cstring>
 
 #include "kernels.cuh"
@@ -50,7 +53,7 @@ struct MidExt {
 struct MidDen {
     double* out;
     int32_t n_runs;
-    float weight[kMaxDenRuns];
+    double weight[kMaxDenRuns];
     int8_t run_of_range[kMaxRanges];
 };
 
@@ -361,12 +364,13 @@ attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_
                     mma_16816(o[2 * j + 1], p[0], p[1], p[2], p[3], v[2], v[3]);
                 }
                 if (kDen) {
-                    uint32_t lo[4];
+                    uint32_t mid[4], lo[4];   // what P leaves, and what that leaves (differences are exact)
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const float (&x)[4] = s[2 * step + u];
-                        lo[2 * u] = pack_bf16(x[0] - bf16_lo(p[2 * u]), x[1] - bf16_hi(p[2 * u]));
-                        lo[2 * u + 1] = pack_bf16(x[2] - bf16_lo(p[2 * u + 1]), x[3] - bf16_hi(p[2 * u + 1]));
+                    for (int u = 0; u < 4; ++u) {
+                        const float (&x)[4] = s[2 * step + u / 2];
+                        const float a = x[2 * (u & 1)] - bf16_lo(p[u]), b = x[2 * (u & 1) + 1] - bf16_hi(p[u]);
+                        mid[u] = pack_bf16(a, b);
+                        lo[u] = pack_bf16(a - bf16_lo(mid[u]), b - bf16_hi(mid[u]));
                     }
                     const int8_t* kr = &key_run[kDen ? stage : 0][ks * kWarpKeys + step * 16 + 2 * q];
 #pragma unroll
@@ -374,8 +378,12 @@ attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_
                         const int run = n * 8 + g;
                         const uint32_t b0 = (kr[0] == run ? 0x3f80u : 0u) | (kr[1] == run ? 0x3f800000u : 0u);
                         const uint32_t b1 = (kr[8] == run ? 0x3f80u : 0u) | (kr[9] == run ? 0x3f800000u : 0u);
-                        mma_16816(od[n], p[0], p[1], p[2], p[3], b0, b1);
-                        mma_16816(od[n], lo[0], lo[1], lo[2], lo[3], b0, b1);
+                        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma_16816(d0, p[0], p[1], p[2], p[3], b0, b1);
+                        mma_16816(d1, mid[0], mid[1], mid[2], mid[3], b0, b1);
+                        mma_16816(d2, lo[0], lo[1], lo[2], lo[3], b0, b1);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) od[n][e] += d0[e] + (d1[e] + d2[e]);
                     }
                 }
             }
@@ -461,15 +469,24 @@ attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_
             if (st_b) *reinterpret_cast<uint4*>(obase + 8 * o_tok + 32 * h) = make_uint4(x[0], x[1], x[2], x[3]);
         }
         if (kDen) {
+            // normalised by the sum of the row's masses, which is l added up in another order: their shares add up to one
+            float d_a = (od[0][0] + od[0][1]) + (od[kDenTiles - 1][0] + od[kDenTiles - 1][1]);
+            float d_b = (od[0][2] + od[0][3]) + (od[kDenTiles - 1][2] + od[kDenTiles - 1][3]);
+            d_a += __shfl_xor_sync(0xffffffffu, d_a, 1);
+            d_b += __shfl_xor_sync(0xffffffffu, d_b, 1);
+            d_a += __shfl_xor_sync(0xffffffffu, d_a, 2);
+            d_b += __shfl_xor_sync(0xffffffffu, d_b, 2);
+            d_a = 1.f / d_a;
+            d_b = 1.f / d_b;
 #pragma unroll
             for (int n = 0; n < kDenTiles; ++n)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    float v = (st_a ? od[n][e] * inv_a : 0.f) + (st_b ? od[n][2 + e] * inv_b : 0.f);
+                    double v = (double)(st_a ? od[n][e] * d_a : 0.f) + (double)(st_b ? od[n][2 + e] * d_b : 0.f);
                     v += __shfl_xor_sync(0xffffffffu, v, 4);
                     v += __shfl_xor_sync(0xffffffffu, v, 8);
                     v += __shfl_xor_sync(0xffffffffu, v, 16);
-                    if (g == 0) atomicAdd(&den_sum[kDen ? n * 8 + 2 * q + e : 0], (double)v);
+                    if (g == 0) atomicAdd(&den_sum[kDen ? n * 8 + 2 * q + e : 0], v);
                 }
         }
     }
@@ -478,7 +495,7 @@ attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_
     if (kDen) {
         __syncthreads();
         if ((int)threadIdx.x < den.n_runs)
-            atomicAdd(den.out + (int64_t)head * den.n_runs + threadIdx.x, den_sum[kDen ? threadIdx.x : 0] * (double)den.weight[threadIdx.x]);
+            atomicAdd(den.out + (int64_t)head * den.n_runs + threadIdx.x, den_sum[kDen ? threadIdx.x : 0] * den.weight[threadIdx.x]);
     }
 }
 

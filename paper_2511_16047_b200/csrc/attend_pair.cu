@@ -1162,7 +1162,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
         if (cur || density->n_runs < 1 || density->n_runs > kMaxDenRuns || !density->out) return cudaErrorInvalidValue;
         den.out = density->out;
         den.n_runs = density->n_runs;
-        for (int i = 0; i < density->n_runs; ++i) den.weight[i] = density->weight[i];
+        for (int i = 0; i < density->n_runs; ++i) den.weight[i] = (float)density->weight[i];
         for (int i = 0; i < ranges.n; ++i) {
             if (density->run_of_range[i] < 0 || density->run_of_range[i] >= density->n_runs) return cudaErrorInvalidValue;
             den.run_of_range[i] = density->run_of_range[i];

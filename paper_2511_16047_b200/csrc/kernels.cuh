@@ -99,7 +99,7 @@ constexpr int kPairMaxDensityRuns = 16;
 struct PairDensity {
     double* out;
     int32_t n_runs;
-    float weight[kPairMaxDensityRuns];
+    double weight[kPairMaxDensityRuns];
     int8_t run_of_range[kMaxRanges];
 };
 

@@ -126,3 +126,32 @@ def test_key_tiles_of_several_runs(D, rows, budgets):
                 # runs and more rows average it down to the 2e-4 asked for above.
                 assert np.allclose(den.cpu().numpy(), want, rtol=1e-3, atol=1e-7), (layer, k)
         assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("path", [B.PATH_AUTO], ids=["auto"])
+@pytest.mark.parametrize("peaked", [False, True], ids=["flat", "peaked"])
+def test_masses_are_those_of_fp32_probabilities(D, path, peaked):
+    """Masses are sums of fp32 probabilities in every kernel, of runs of one key as of long ones: relative to the oracle an
+    exponential is off by 2^-22 (its instruction) and by the rounding of its argument, which is at most 2^-24 of a logit's size
+    (in units of log 2: under 2 for the flat inputs, under 48 for the peaked ones) times a few roundings; sums of up to 274
+    terms in fp32 add less.  Twice that: 1e-6 and 1e-5.  (Probabilities rounded to 16 bits are off by 2e-3, the polynomial that the
+    attention outputs take every sixth pair from by up to 8e-4, and two bf16 terms by 8e-6 of one probability.)"""
+    sides, rows, heads, scale = (1, 2, 3, 4, 5, 7, 10, 13), 1, 3, 1.0 / math.sqrt(D)
+    pols = [(2, 2, False), (0, 9, True)]
+    qkv = make_qkv(rows, heads, sides, D, seed=99, peaked=peaked)
+    Ks = [to_items(k) for _, k, _ in qkv]
+    worst = 0.0
+    with Cache(len(pols), heads, D, rows, sides, pols) as c:
+        B.amskv_set_attend_path(c.h, path)
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(pols)):
+                B.amskv_append(c.h, layer, k, kk, v)
+                runs = B.amskv_attended_tokens(c.h, layer, k)
+                out = torch.full_like(q, float("nan"))
+                den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+                B.amskv_attend_density(c.h, layer, k, q, out, den, den.numel())
+                torch.cuda.synchronize()
+                want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
+                worst = max(worst, np.abs(den.cpu().numpy() / want - 1).max())
+    assert worst <= (1e-5 if peaked else 1e-6), worst

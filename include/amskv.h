@@ -256,9 +256,10 @@ AMSKV_API int amskv_attention_density(amskv_cache* cache, int layer, int scale, 
  * probability mass of a query row on a run is a running sum of the box sums the softmax computes anyway;
  * the rows are normalised by their row sums in the epilogue and added up per (head, run).  One launch, no
  * second pass over the keys; the launch is somewhat longer than a plain amskv_attend (a few more, partly
- * filled key tiles, and the sums).  `out` is the same as amskv_attend's.  `density`, `density_entries` and the
- * meaning of the numbers are those of amskv_attention_density (probabilities after their rounding to bf16,
- * where that call uses them unrounded: they agree to about 1e-4 relative).  The warp-matrix kernel serves
+ * filled key tiles, and the sums).  `out` is amskv_attend's up to rounding (the key tiles may be others, and so may the
+ * kernel).  `density`, `density_entries` and the meaning of the numbers are those of amskv_attention_density: sums of
+ * fp32 probabilities, which no kernel rounds for them (both calls are within 1e-6 relative of exact sums where logits
+ * differ by units, 1e-5 where they differ by tens).  The warp-matrix kernel serves
  * scales of at most 16 queries and calls of few items the same way in one launch (the masses are products of
  * the probabilities with a 0/1 matrix of run membership).  The kernels of the other paths, and layers with
  * more than 16 runs, run as amskv_attend followed by amskv_attention_density.

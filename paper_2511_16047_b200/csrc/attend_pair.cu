@@ -49,7 +49,11 @@ constexpr int kMaxStages = 4;
 constexpr float kRescaleLog2 = 8.f;
 constexpr int kQSplitRows = 64;   // query tiles of at most this many rows are double-buffered inside their slot
 constexpr float kLazySumLimit = 1.8446744e19f;   // 2^64: see the kLazy form of the softmax loop
-constexpr int kPolyEvery = 6;     // every 6th pair of exponentials goes to the FMA pipe (0: none); swept 2, 3, 4, 6, 8
+// Every 6th pair of exponentials goes to the FMA pipe (0: none); swept 2, 3, 4, 6, 8.  None in density launches: a run of few keys
+// shows the polynomial's error (8e-4 at most), the more where it is not in the tile whose maximum is the reference.  Masses of 480
+// items, T = 256, peaked rows: off by 2.5e-5 with it (8e-6 when every run had tiles of its own and the first run the first), 4e-8
+// without.  512 items, T = 256: 51.4 -> 51.8 us a call, 128 channels 81.8 -> 83.0.
+constexpr int kPolyEvery = 6;
 
 // kWide: one CTA per SM with two S buffers per stream and an issuing warp per stream (below): the form
 // 128 channels use, and 64 channels in launches of at most one unit per SM; with more units 64 channels use the
@@ -899,11 +903,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                                 for (int ii = 0; ii < 8; ++ii) {
                                     const int i = (grp & 1) * 8 + ii;   // pair index within its 32-token half, as before
                                     const int c = grp * 16 + 2 * ii;
-                                    // every kPolyEvery-th pair takes its exponentials from a polynomial on the FMA pipe:
+                                    // (but in density launches) every kPolyEvery-th pair takes its exponentials from a polynomial on the FMA pipe:
                                     // the special-function unit (16 results per clock per SM) is the narrowest resource
                                     float x0, x1, p0, p1;
                                     fma2(x0, x1, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]), scale_log2, scale_log2, nb, nb);
-                                    if (kPolyEvery > 0 && (i % (kPolyEvery > 0 ? kPolyEvery : 1)) == 0) {
+                                    if (!kDen && kPolyEvery > 0 && (i % (kPolyEvery > 0 ? kPolyEvery : 1)) == 0) {
                                         exp2_poly2(p0, p1, x0, x1);
                                     } else {
                                         p0 = fast_exp2(x0);

@@ -121,15 +121,12 @@ def test_key_tiles_of_several_runs(D, rows, budgets):
                 tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
                 check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, scale), "layer %d scale %d" % (layer, k), max_abs=4e-2)
                 want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
-                # A run of one key is as exact as that key's exponential, and every sixth pair's comes from the cubic
-                # sum of f^n (ln 2)^n / n!, n <= 3, |f| <= 1/2: at most 7.9e-4 of 2^f too small (f = -1/2).  Longer
-                # runs and more rows average it down to the 2e-4 asked for above.
-                assert np.allclose(den.cpu().numpy(), want, rtol=1e-3, atol=1e-7), (layer, k)
+                assert np.allclose(den.cpu().numpy(), want, rtol=2e-4, atol=1e-7), (layer, k)
         assert B.amskv_status(c.h) == 0
 
 
 @pytest.mark.parametrize("D", [64, 128])
-@pytest.mark.parametrize("path", [B.PATH_AUTO], ids=["auto"])
+@pytest.mark.parametrize("path", [B.PATH_AUTO, B.PATH_TENSOR_PAIR], ids=["auto", "pair"])
 @pytest.mark.parametrize("peaked", [False, True], ids=["flat", "peaked"])
 def test_masses_are_those_of_fp32_probabilities(D, path, peaked):
     """Masses are sums of fp32 probabilities in every kernel, of runs of one key as of long ones: relative to the oracle an

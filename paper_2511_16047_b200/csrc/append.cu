@@ -16,7 +16,7 @@ static_assert(kThreads * kUnroll == kAppendBlockChunks, "blocks of a copy, as th
 // with density at T = 9, 512 items; 1 920 items, T = 25 19.9 -> 19.3; copies at the memory's rate are unchanged).
 template <int D, typename Index>
 __global__ void __launch_bounds__(kThreads)
-append_kernel(const uint4* __restrict__ Ksrc, const uint4* __restrict__ Vsrc, int64_t k_row, int64_t k_head,
+append_kernel(const uint4* Ksrc, const uint4* Vsrc, int64_t k_row, int64_t k_head,
               int64_t k_tok, int64_t v_row, int64_t v_head, int64_t v_tok, uint4* __restrict__ dst, int32_t capacity,
               int32_t token_offset, int32_t T, int32_t heads, int64_t total_chunks)
 {
@@ -43,8 +43,8 @@ append_kernel(const uint4* __restrict__ Ksrc, const uint4* __restrict__ Vsrc, in
                 // strides are in elements and multiples of 8, so they divide into chunks
                 const int64_t ks = (row * k_row + head * k_head + tok * k_tok) / 8 + ch;
                 const int64_t vs = (row * v_row + head * v_head + tok * v_tok) / 8 + ch;
-                kv[u] = __ldcs(Ksrc + ks);
-                vv[u] = __ldcs(Vsrc + vs);
+                kv[u] = load_16B_once(Ksrc + ks);
+                vv[u] = load_16B_once(Vsrc + vs);
                 d[u] = (int64_t)item * item_stride + (int64_t)(token_offset + tok) * CPT + ch;
             }
         }
@@ -73,7 +73,7 @@ constexpr uint32_t kBulkSpinLimit = 1u << 24;
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __global__ void __launch_bounds__(32)
-append_bulk_kernel(const char* __restrict__ Ksrc, const char* __restrict__ Vsrc, int64_t src_item_bytes,
+append_bulk_kernel(const char* Ksrc, const char* Vsrc, int64_t src_item_bytes,
                    char* __restrict__ dst, int64_t dst_item_bytes, int64_t v_shift_bytes, int64_t dst_offset_bytes,
                    uint32_t block_bytes, uint32_t chunks_per_block, int64_t total_chunks, int* __restrict__ status)
 {

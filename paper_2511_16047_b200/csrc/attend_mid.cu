@@ -153,7 +153,7 @@ __device__ __forceinline__ void scale_rows(float (&o)[N][4], float f_a, float f_
 
 template <int D, int NW, bool kDen>
 __global__ void __launch_bounds__(NW * 32, D == 64 ? 16 / NW : 2)
-attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
+attend_mid_kernel(const __nv_bfloat16* Q, int64_t q_row, int64_t q_head, int64_t q_tok,
                   __nv_bfloat16* __restrict__ O, int64_t o_row, int64_t o_head, int64_t o_tok,
                   __nv_bfloat16* __restrict__ region, int32_t capacity, const __grid_constant__ RangeList ranges,
                   int32_t T, int32_t heads, int32_t parts, int32_t n_rb, int32_t n_stages, float scale_log2,
@@ -266,8 +266,8 @@ attend_mid_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_
     uint4 qa0[kPieces], qa1[kPieces];
 #pragma unroll
     for (int h = 0; h < kPieces; ++h) {
-        qa0[h] = __ldg(q0 + 4 * h);
-        qa1[h] = __ldg(q1 + 4 * h);
+        qa0[h] = load_16B(q0 + 4 * h);
+        qa1[h] = load_16B(q1 + 4 * h);
     }
 #pragma unroll 1
     for (int c = 0; c < C::kStages; ++c) {

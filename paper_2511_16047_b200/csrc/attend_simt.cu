@@ -30,7 +30,7 @@ __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&f)[N])
     static_assert(N % 8 == 0, "16-byte granules");
 #pragma unroll
     for (int c = 0; c < N / 8; ++c) {
-        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(p) + c);
+        const uint4 raw = load_16B(reinterpret_cast<const uint4*>(p) + c);
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -43,11 +43,11 @@ __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&f)[N])
 
 template <int D>
 __global__ void __launch_bounds__(kThreads)
-attend_simt_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
+attend_simt_kernel(const __nv_bfloat16* Q, int64_t q_row, int64_t q_head, int64_t q_tok,
                    __nv_bfloat16* __restrict__ O, int64_t o_row, int64_t o_head, int64_t o_tok,
-                   const __nv_bfloat16* __restrict__ region, int32_t capacity, const RangeList ranges, int32_t T,
-                   int32_t heads, int64_t total_rows, float scale_log2, const __nv_bfloat16* __restrict__ ext_k,
-                   const __nv_bfloat16* __restrict__ ext_v, int64_t e_row, int64_t e_head, int64_t e_tok, int ext_range)
+                   const __nv_bfloat16* region, int32_t capacity, const RangeList ranges, int32_t T,
+                   int32_t heads, int64_t total_rows, float scale_log2, const __nv_bfloat16* ext_k,
+                   const __nv_bfloat16* ext_v, int64_t e_row, int64_t e_head, int64_t e_tok, int ext_range)
 {
     overlap_with_previous();
     constexpr int DPL = D / kLanesPerRow;  // channels per lane

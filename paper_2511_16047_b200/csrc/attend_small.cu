@@ -96,7 +96,7 @@ struct SmallExt {
 // us, 480 items 6.8 -> 5.8, 2 880 items 21.4 -> 18.5).
 template <int D, bool kExt, int kTiles, bool kEarlyV>
 __global__ void __launch_bounds__(kWarpsPerCta * 32, D == 64 ? (kTiles == 1 ? 6 : kTiles == 4 && kEarlyV ? 6 : 8) : (kTiles == 1 ? 6 : 4))
-attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
+attend_small_kernel(const __nv_bfloat16* Q, int64_t q_row, int64_t q_head, int64_t q_tok,
                     __nv_bfloat16* __restrict__ O, int64_t o_row, int64_t o_head, int64_t o_tok,
                     __nv_bfloat16* __restrict__ region, int32_t capacity, const RangeList ranges, int32_t T,
                     int32_t heads, int32_t n_items, float scale_log2, const SmallExt ext)
@@ -148,8 +148,8 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
         uint4 qa0[kPieces], qa1[kPieces];
 #pragma unroll
         for (int h = 0; h < kPieces; ++h) {
-            qa0[h] = __ldg(q0 + 4 * h);
-            qa1[h] = __ldg(q1 + 4 * h);
+            qa0[h] = load_16B(q0 + 4 * h);
+            qa1[h] = load_16B(q1 + 4 * h);
         }
         // ---- K pieces of every tile: all loads are issued before the first product needs one
         uint4 kk[kTiles][kPieces];
@@ -157,7 +157,7 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
         for (int t = 0; t < kTiles; ++t) {
             if (t < n_key_tiles) {
 #pragma unroll
-                for (int h = 0; h < kPieces; ++h) kk[t][h] = __ldg(kp[t] + 4 * h);
+                for (int h = 0; h < kPieces; ++h) kk[t][h] = load_16B(kp[t] + 4 * h);
             }
         }
         // ---- V pieces likewise (nothing the softmax computes is needed to fetch them)
@@ -166,7 +166,7 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
         for (int t = 0; t < kTiles; ++t) {
             if (kEarlyV && t < 2 * n_key_steps) {
 #pragma unroll
-                for (int h = 0; h < kPieces; ++h) vv[t][h] = __ldg(vp[t] + 4 * h);
+                for (int h = 0; h < kPieces; ++h) vv[t][h] = load_16B(vp[t] + 4 * h);
             }
         }
         // ---- S = Q K^T : this lane holds S[g][8t + 2q .. +1] and S[g + 8][same] of every tile t
@@ -233,8 +233,8 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
                 if (!kEarlyV) {
 #pragma unroll
                     for (int h = 0; h < kPieces; ++h) {
-                        vv[2 * st][h] = __ldg(vp[2 * st] + 4 * h);
-                        vv[kTiles > 1 ? 2 * st + 1 : 0][h] = __ldg(vp[kTiles > 1 ? 2 * st + 1 : 0] + 4 * h);
+                        vv[2 * st][h] = load_16B(vp[2 * st] + 4 * h);
+                        vv[kTiles > 1 ? 2 * st + 1 : 0][h] = load_16B(vp[kTiles > 1 ? 2 * st + 1 : 0] + 4 * h);
                     }
                 }
                 const uint4(&v0)[kPieces] = vv[2 * st];
@@ -282,7 +282,7 @@ attend_small_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t 
 // One 16-byte piece per thread.
 template <int D>
 __global__ void __launch_bounds__(256)
-single_key_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int64_t e_row, int64_t e_head,
+single_key_kernel(const uint4* K, const uint4* V, int64_t e_row, int64_t e_head,
                   uint4* __restrict__ O, int64_t o_row, int64_t o_head, uint4* __restrict__ region, int32_t capacity,
                   int32_t dst, int32_t store, int32_t heads, int64_t n_pieces)
 {
@@ -293,10 +293,10 @@ single_key_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V, int6
     const int64_t item = idx / CPT;
     const int32_t ch = (int32_t)(idx - item * CPT);
     const int32_t row = (int32_t)(item / heads), head = (int32_t)(item - (int64_t)row * heads);
-    const uint4 v = __ldg(V + (row * e_row + head * e_head) / 8 + ch);
+    const uint4 v = load_16B(V + (row * e_row + head * e_head) / 8 + ch);
     O[(row * o_row + head * o_head) / 8 + ch] = v;
     if (store) {
-        const uint4 k = __ldg(K + (row * e_row + head * e_head) / 8 + ch);
+        const uint4 k = load_16B(K + (row * e_row + head * e_head) / 8 + ch);
         uint4* kd = region + item * (2ll * capacity * CPT) + (int64_t)dst * CPT + ch;
         kd[0] = k;
         kd[(int64_t)capacity * CPT] = v;

@@ -29,7 +29,7 @@ __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&f)[N])
 {
 #pragma unroll
     for (int c = 0; c < N / 8; ++c) {
-        const uint4 raw = __ldg(reinterpret_cast<const uint4*>(p) + c);
+        const uint4 raw = load_16B(reinterpret_cast<const uint4*>(p) + c);
         const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -42,8 +42,8 @@ __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&f)[N])
 
 template <int D>
 __global__ void __launch_bounds__(kThreads)
-density_kernel(const __nv_bfloat16* __restrict__ Q, int64_t q_row, int64_t q_head, int64_t q_tok,
-               const __nv_bfloat16* __restrict__ region, int32_t capacity, const DensityPieces pieces, int32_t T,
+density_kernel(const __nv_bfloat16* Q, int64_t q_row, int64_t q_head, int64_t q_tok,
+               const __nv_bfloat16* region, int32_t capacity, const DensityPieces pieces, int32_t T,
                int32_t heads, int32_t ctas_per_item, float scale_log2, double inv_rows, double* __restrict__ out)
 {
     constexpr int DPL = D / kLanesPerRow;

@@ -210,6 +210,27 @@ __device__ __forceinline__ void overlap_with_previous()
     wait_for_previous();
     let_next_start();
 }
+// Loads of what an earlier launch wrote or the caller passed.  A kernel that is alive while its predecessor still writes may not
+// use the read-only path (ld.global.nc, which __ldg and const __restrict__ pointers lead to: the data must not change while
+// the kernel runs, and the compiler may move such a load above the wait).  These are ordinary loads that stay behind it.
+__device__ __forceinline__ uint4 load_16B(const void* p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 load_16B_once(const void* p)   // (data that no other load wants)
+{
+    uint4 v;
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double load_double(const double* p)
+{
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
 #endif
 
 // The attention of amskv_attend overlaps the copy of its scale's append where all blocks of that copy are resident at once

@@ -75,7 +75,7 @@ __device__ __forceinline__ void tap(int i, float ratio, int s_in, int& i0, int& 
 // multiply-adds per channel.
 template <int D>
 __global__ void __launch_bounds__(kThreads)
-similarity_partial_kernel(const uint4* __restrict__ K_prev, int32_t s_prev, const uint4* __restrict__ K_cur,
+similarity_partial_kernel(const uint4* K_prev, int32_t s_prev, const uint4* K_cur,
                           int32_t s_cur, int64_t items, int64_t units, int32_t parts, int32_t part_chunks,
                           int32_t items_per_unit, uint64_t inv_s_cur, double* __restrict__ partials)
 {
@@ -125,11 +125,11 @@ similarity_partial_kernel(const uint4* __restrict__ K_prev, int32_t s_prev, cons
             uint4 cur[2], t00[2], t01[2], t10[2], t11[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                cur[h] = __ldcs(C + 2 * idx + h);
-                t00[h] = __ldg(p00 + h);
-                t01[h] = __ldg(p01 + h);
-                t10[h] = __ldg(p10 + h);
-                t11[h] = __ldg(p11 + h);
+                cur[h] = load_16B_once(C + 2 * idx + h);
+                t00[h] = load_16B(p00 + h);
+                t01[h] = load_16B(p01 + h);
+                t10[h] = load_16B(p10 + h);
+                t11[h] = load_16B(p11 + h);
             }
             float p0 = 0.f, p1 = 0.f;
 #pragma unroll
@@ -158,12 +158,12 @@ similarity_partial_kernel(const uint4* __restrict__ K_prev, int32_t s_prev, cons
 }
 
 __global__ void __launch_bounds__(kThreads)
-similarity_final_kernel(const double* __restrict__ partials, int n, double* __restrict__ out)
+similarity_final_kernel(const double* partials, int n, double* __restrict__ out)
 {
     overlap_with_previous();
     __shared__ double smem[kThreads / 32];
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += kThreads) acc += partials[i];
+    for (int i = threadIdx.x; i < n; i += kThreads) acc += load_double(partials + i);
     const double total = block_sum(acc, smem);
     if (threadIdx.x == 0) *out = total;
 }

@@ -1,5 +1,5 @@
-"""Order of the launch-overlap instructions in the CUDA sources, checked on the text: what it guards against is a hang, which
-no test may provoke on a GPU."""
+"""Launch overlap in the CUDA sources, checked on the text: the order of its instructions, where what it guards against is a hang,
+which no test may provoke on a GPU, and the loads behind them, where it is a compiler's licence."""
 import glob
 import os
 import re
@@ -50,3 +50,13 @@ def test_the_next_launch_is_let_in_after_the_wait_and_after_the_tensor_memory_is
     if alloc:
         owned = re.search(r"__syncthreads\s*\(", body[alloc.end():])
         assert owned and release.start() > alloc.end() + owned.start()
+
+
+@pytest.mark.parametrize("path", sorted(glob.glob(os.path.join(CSRC, "*.cu*"))), ids=os.path.basename)
+def test_no_load_promises_that_its_data_is_read_only(path):
+    """A kernel is alive while the one before it still writes, so no load may go by the read-only path, which promises that the
+    data does not change and lets the compiler move the load above the wait."""
+    text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(path).read(), flags=re.S)
+    assert not re.search(r"__ld(g|cs|ca|cg|lu|cv)\s*\(|ld\.global\.nc", text)
+    for m in re.finditer(r"__global__", text):
+        assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", text[m.end():text.index("{", m.end())])

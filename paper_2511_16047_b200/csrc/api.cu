@@ -36,6 +36,7 @@ struct amskv_cache {
     float softmax_scale = 0.f;
     int path = AMSKV_PATH_AUTO;
     int sm_count = 0;
+    bool pageable_access = false;   // the device reads and writes pageable host memory
     std::vector<int32_t> sides, tokens;
     std::vector<LayerLayout> layout;
     std::vector<LayerLayout> layout0;   // as created: amskv_cache_reset undoes promotions
@@ -237,16 +238,18 @@ int amskv_cache_create(const amskv_desc* desc, void* dev_mem, size_t dev_bytes, 
     if (rc != AMSKV_OK) { delete c; return rc; }
     if (c->plan_only()) { *out = c; return AMSKV_OK; }
 
-    // (two attributes, not cudaGetDeviceProperties: it also queries clocks, which takes milliseconds a call; creating the
+    // (attributes, not cudaGetDeviceProperties: it also queries clocks, which takes milliseconds a call; creating the
     // cache of one layer for one image, arena included: 6 -> 0.7 ms)
-    int dev = 0, major = 0, sm_count = 0;
+    int dev = 0, major = 0, sm_count = 0, pageable = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) {
         (void)cudaGetLastError();
         delete c;
         return AMSKV_ERR_CUDA;
     }
     c->sm_count = sm_count;
+    c->pageable_access = pageable != 0;
     if (dev_mem) {
         if ((reinterpret_cast<uintptr_t>(dev_mem) % kAlign) != 0) { delete c; return AMSKV_ERR_INVALID; }
         if (dev_bytes < c->arena_bytes) { delete c; return AMSKV_ERR_NOMEM; }
@@ -639,7 +642,11 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
             den.run_of_range[i] = (int8_t)rp[i].run;
         }
         cudaStream_t st = static_cast<cudaStream_t>(stream);
-        cudaError_t e = launch_zero(density, (size_t)cache->heads * n_runs, st);
+        // pageable host memory, which the driver refuses to fill, must not reach a kernel
+        cudaPointerAttributes where;
+        cudaError_t e = cudaPointerGetAttributes(&where, density);
+        if (e == cudaSuccess && where.type == cudaMemoryTypeUnregistered && !cache->pageable_access) e = cudaErrorInvalidValue;
+        if (e == cudaSuccess) e = launch_zero(density, (size_t)cache->heads * n_runs, st);
         if (e == cudaSuccess && kernel == AttendKernel::Mid)
             e = launch_attend_mid(q, o, cache->region(layer), ranges, T, cache->rows, cache->heads, cache->head_dim,
                                   cache->softmax_scale, cache->sm_count, st, nullptr, nullptr, 0, &den);

@@ -152,3 +152,25 @@ def test_masses_are_those_of_fp32_probabilities(D, path, peaked):
                 want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
                 worst = max(worst, np.abs(den.cpu().numpy() / want - 1).max())
     assert worst <= (1e-5 if peaked else 1e-6), worst
+
+
+@pytest.mark.parametrize("side", [4, 10])
+def test_a_result_in_pageable_host_memory_is_refused(side):
+    """As a fill of it is; nothing is launched and the cache stays usable."""
+    qkv = make_qkv(1, 2, (side,), 64, seed=100)
+    q, kk, v = qkv[0]
+    with Cache(1, 2, 64, 1, (side,), [(1, 1, True)]) as c:
+        B.amskv_append(c.h, 0, 0, kk, v)
+        out = torch.empty_like(q)
+        runs = B.amskv_attended_tokens(c.h, 0, 0)
+        host = np.full(2, np.nan)
+        n0 = B.amskv_launch_count()
+        assert B.lib.amskv_attend_density(c.h, 0, 0, q.data_ptr(), out.data_ptr(), None, None, host.ctypes.data_as(B.ctypes.c_void_p),
+                                          2, None) == B.ERR_CUDA
+        assert B.amskv_launch_count() == n0
+        den = torch.full((2, 1), float("nan"), dtype=torch.float64, device="cuda")
+        B.amskv_attend_density(c.h, 0, 0, q, out, den, 2)
+        torch.cuda.synchronize()
+        want = oracle.attention_density(to_items(q), [to_items(kk)], runs, 0.125, 2)
+        assert np.allclose(den.cpu().numpy(), want, rtol=1e-5)
+        assert B.amskv_status(c.h) == 0

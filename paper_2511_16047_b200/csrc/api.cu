@@ -196,8 +196,9 @@ enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
 // (copies: the call includes an append of several copies, which only the warp-matrix kernel takes in)
 AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool copies = false)
 {
-    // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained)
-    if (cache->path == AMSKV_PATH_AUTO && (T > 1 || density) && cache->tc_ready &&
+    // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained); for a single query token,
+    // which is the CUDA-core kernel's with its fp32 probabilities, only where its one key makes the output a copy of V
+    if (cache->path == AMSKV_PATH_AUTO && (T > 1 || (density && total == 1)) && cache->tc_ready &&
         mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density, copies))
         return AttendKernel::Mid;
     // AUTO: the warp-per-item kernel wherever a scale's retained keys fit its register tile, the paired

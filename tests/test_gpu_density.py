@@ -174,3 +174,22 @@ def test_a_result_in_pageable_host_memory_is_refused(side):
         want = oracle.attention_density(to_items(q), [to_items(kk)], runs, 0.125, 2)
         assert np.allclose(den.cpu().numpy(), want, rtol=1e-5)
         assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_a_single_token_with_several_keys_keeps_fp32_probabilities(D):
+    """The output of the call with densities is amskv_attend's bit for bit: the CUDA-core kernel's, which rounds no probability."""
+    sides, rows, heads = (3, 1, 5, 1, 1), 2, 3
+    qkv = make_qkv(rows, heads, sides, D, seed=101, peaked=True)
+    with Cache(1, heads, D, rows, sides, [(0, 9, True)]) as c:
+        for k, (q, kk, v) in enumerate(qkv):
+            B.amskv_append(c.h, 0, k, kk, v)
+            runs = B.amskv_attended_tokens(c.h, 0, k)
+            den = torch.zeros((heads, len(runs)), dtype=torch.float64, device="cuda")
+            out, want = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+            B.amskv_attend_density(c.h, 0, k, q, out, den, den.numel())
+            B.amskv_attend(c.h, 0, k, q, want)
+            torch.cuda.synchronize()
+            if sides[k] == 1:
+                assert torch.equal(out, want)
+        assert B.amskv_status(c.h) == 0

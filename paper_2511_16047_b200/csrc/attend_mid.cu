@@ -533,13 +533,21 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // (128); none above 64 queries where the paired kernel has an SM for every tile: T = 81: 8.0 / 7.2 (16), 7.9 / 7.5 (32), 9.8 / 8.2 (64).
 // With the density (20 and 7 units; times with the append and the zeroed result): T = 36: 10.2 / 13.0 (120 items), 12.0 / 14.5
 // (256), 18.2 / 16.4 (384), 19.4 / 16.9 (512); T = 64: 15.3 / 18.2 (256), 21.7 / 19.8 (384); T = 100: 15.8 / 18.4 (120), 26.4 / 21.8
-// (256); T = 25: 18.9 / 21.0 (1 024); 128 channels, T = 64: 13.9 / 17.0 (120), 22.5 / 19.3 (256); and up to 16 queries the alternative is the
-// attention call plus the CUDA-core density pass (T = 4, 9, 16 at 512 items: 12.5 / 16.6, 13.5 / 23.6, 13.0 / 35.0): always this
-// one.  Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).  An append of several copies (`copies`),
+// (256); T = 25: 18.9 / 21.0 (1 024); 128 channels, T = 64: 13.9 / 17.0 (120), 22.5 / 19.3 (256).  Up to 16 queries with no more keys
+// than the warp-per-item kernel takes the alternative is the attention call plus the CUDA-core density pass, whose time grows
+// with the queries: always this one (T = 4, 9, 16 at 3 840 items: 23.3 / 27.1, 26.7 / 49.8, 31.8 / 90.5; 128 channels, T = 9 and 16:
+// 63.7 / 74.2 and 74.4 / 149), but for a single token up to 10 items per SM (1 024 items 10.0 / 11.4, 1 920 13.4 / 12.7) and, with 128
+// channels, where an SM holds two of its CTAs, up to two items per SM for a single token (300 items 10.8 / 11.6, 400 11.3 / 11.2,
+// 3 840 53.5 / 18.9) and five for four (700 items 15.9 / 16.3, 1 024 19.8 / 17.7, 3 840 58 / 37).  With more keys the alternative is the
+// paired kernel's one launch (T = 16, 916 keys: 400 items 28.9 / 41.0, 3 840 items 225 / 240; 128 channels 340 / 344).
+// Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).  An append of several copies (`copies`),
 // 2 us each beside the paired kernel, keeps the first lines.
 bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies)
 {
-    if (density && T <= kSmallMaxQueries) return true;
+    if (density && T <= kSmallMaxQueries) {
+        if (!small_supported(T, total_keys) || (T > 1 && D == 64) || T > 4) return true;
+        return items <= (int64_t)sm_count * (T > 1 ? 5 : D == 64 ? 10 : 2);
+    }
     if (!density && small_supported(T, total_keys)) return false;
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
     int line = D == 64 ? 19 : 6;

@@ -193,3 +193,26 @@ def test_a_single_token_with_several_keys_keeps_fp32_probabilities(D):
             if sides[k] == 1:
                 assert torch.equal(out, want)
         assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D,sides,items", [(64, (1, 2), (1480, 1488)), (128, (1, 2), (296, 304, 740, 744)), (128, (2, 3, 4), (740, 744))])
+def test_one_query_block_on_both_sides_of_the_lines(D, sides, items):
+    """Single tokens, four and more queries at the item counts where the kernel changes (10, 2 and 5 per SM of 148): the
+    densities of an item do not depend on it."""
+    for n in items:
+        heads, scale = 8, 1.0 / math.sqrt(D)
+        rows = n // heads
+        qkv = make_qkv(rows, heads, sides, D, seed=102)
+        with Cache(1, heads, D, rows, sides, [(0, 9, True)]) as c:
+            for k, (q, kk, v) in enumerate(qkv):
+                B.amskv_append(c.h, 0, k, kk, v)
+                runs = B.amskv_attended_tokens(c.h, 0, k)
+                out = torch.full_like(q, float("nan"))
+                den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+                B.amskv_attend_density(c.h, 0, k, q, out, den, den.numel())
+                torch.cuda.synchronize()
+                Ks, Vs = [to_items(t[1]) for t in qkv[:k + 1]], [to_items(t[2]) for t in qkv[:k + 1]]
+                check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, [(s, t) for s, f, m in runs for t in range(f, f + m)], scale),
+                            "%d items, scale %d" % (n, k))
+                assert np.allclose(den.cpu().numpy(), oracle.attention_density(to_items(q), Ks, runs, scale, heads), rtol=1e-6), (n, k)
+            assert B.amskv_status(c.h) == 0

@@ -521,27 +521,33 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 
 }  // namespace
 
-// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.
-// 64 channels: 19 units.  Below it the paired kernel (and, where the append cannot be fused into that, the copy before it)
-// costs 6 to 14 us whatever the size; above it the warp-level matrix instructions, a quarter of the tensor pipe's rate, are
-// what the call takes.  us per call, this kernel / the paired one, append included, in a graph: T = 25: 3.9 / 8.9 (60 items),
-// 6.4 / 11.2 (512), 11.5 / 14.9 (1 024), 19.7 / 19.8 (1 920); T = 36: 4.7 / 6.6 (60), 6.4 / 7.9 (256), 12.9 / 9.0 (512); T = 64: 8.9 /
-// 9.6 (256), 15.7 / 11.2 (512); T = 100: 16.1 / 12.4 (256).  7 units where the paired kernel has an SM for every query tile:
-// T = 64: 5.4 / 5.6 (48), 6.5 / 6.7 (96), 7.4 / 6.9 (120); T = 81: 6.1 / 6.4 (32), 7.6 / 6.7 (60); T = 100: 6.4 / 7.4 (16), 7.4 / 7.5 (32),
-// 8.8 / 7.7 (60); T = 144: 8.2 / 8.5 (16), 10.3 / 8.7 (32).
-// 128 channels: 6 units: T = 36: 5.2 / 10.2 (32), 6.2 / 10.8 (128), 20.5 / 17.1 (512); T = 64: 6.8 / 8.0 (32), 7.0 / 8.9 (64), 10.4 / 10.4
-// (128); none above 64 queries where the paired kernel has an SM for every tile: T = 81: 8.0 / 7.2 (16), 7.9 / 7.5 (32), 9.8 / 8.2 (64).
-// With the density (20 and 7 units; times with the append and the zeroed result): T = 36: 10.2 / 13.0 (120 items), 12.0 / 14.5
-// (256), 18.2 / 16.4 (384), 19.4 / 16.9 (512); T = 64: 15.3 / 18.2 (256), 21.7 / 19.8 (384); T = 100: 15.8 / 18.4 (120), 26.4 / 21.8
-// (256); T = 25: 18.9 / 21.0 (1 024); 128 channels, T = 64: 13.9 / 17.0 (120), 22.5 / 19.3 (256).  Up to 16 queries with no more keys
+// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.  Below the lines the paired
+// kernel costs 5 to 9 us whatever the size (and the copy before it, where the append is not fused into that); above them the
+// warp-level matrix instructions, a quarter of the tensor pipe's rate, are what the call takes.  us per call, this kernel / the
+// paired one, append included, in a graph:
+// 64 channels: 19 units, above 32 queries also no more CTAs (of eight warps, two to an SM) than are resident at once: T = 25: 3.6 /
+// 6.8 (60 items), 6.0 / 9.0 (512), 11.1 / 12.4 (1 024, 13.8 units), 19.4 / 17.6 (1 920, 25.9); T = 36: 4.4 / 5.7 (60), 5.9 / 7.9 (240), 9.8 / 8.0
+// (300, the second wave), 12.6 / 8.5 (512); T = 64: 8.2 / 8.5 (240, 13 units), 11.8 / 8.5 (300); T = 81: 7.7 / 8.9 (148), 12.4 / 11.1 (180).
+// Above 81 queries 7 units where the paired kernel has an SM for every query tile, because of calls behind a separate append
+// (fused, and append and attention apart: T = 100: 5.9 / 6.7 and 9.2 / 8.7 (60, 8.5 units), 7.7 / 7.4 and 9.8 / 9.8 (96, 13.6); T = 121:
+// 7.0 / 8.0 and 10.8 / 9.3 (60, 13.0); T = 169: 7.9 / 8.1 and 9.3 / 9.8 (32, 11.9), 10.5 / 9.1 and 12.2 / 11.1 (60, 22.3)).  An append of several
+// copies (`copies`), which is never apart and which the paired kernel writes partly row by row, keeps the 19: T = 100: 8.4 / 8.8 (120, 17 units), 9.0 / 9.3 (148,
+// 21); T = 121: 7.4 / 8.5 (60, 13), 9.9 / 9.6 (96, 20.8); T = 169: 8.8 / 9.3 (96, 21.4), 13.9 / 9.5 (120, 26.8).
+// 128 channels: 6 units: T = 25: 4.7 / 7.3 (60), 12.6 / 13.5 (512, 6.9 units), 17.4 / 16.2 (700); T = 36: 5.7 / 6.2 (60), 7.0 / 7.8 (148, 6.0),
+// 11.9 / 9.3 (180); T = 64: 6.0 / 6.4 (60), 7.5 / 7.5 (96, 5.2), 8.7 / 8.5 (148); none above 64 queries where the paired kernel has an SM
+// for every tile (T = 81: 7.0 / 7.0 (8), 7.1 / 7.2 (32), 8.6 / 8.0 (60); T = 100: 7.2 / 6.5 (8)) but for several copies (T = 100: 7.6 / 8.0 (32,
+// 4.5), 9.6 / 8.5 (60, 8.5); T = 169: 7.5 / 8.0 (8, 3.0), 9.2 / 8.5 (32, 7.1)).
+// With the density 20 and 7 units (times with the append and the zeroed result): T = 25: 18.2 / 18.7
+// (1 024 items), 27.8 / 29.3 (1 920, 25.9 units); T = 36: 10.4 / 12.4 (240), 15.0 / 13.1 (300); T = 64: 12.3 / 15.1 (240), 18.2 / 16.7 (300); T = 81:
+// 12.6 / 16.2 (148, 18 units), 18.0 / 16.9 (180); 128 channels: T = 25: 18.2 / 20.1 (512, 6.9 units), 23.6 / 25.3 (700), 49 / 49 (1 920); T = 36: 11.6 /
+// 13.6 (148), 17.4 / 14.0 (180); T = 64: 12.8 / 15.9 (120, 6.5), 20.7 / 17.1 (180).  Up to 16 queries with no more keys
 // than the warp-per-item kernel takes the alternative is the attention call plus the CUDA-core density pass, whose time grows
 // with the queries: always this one (T = 4, 9, 16 at 3 840 items: 23.3 / 27.1, 26.7 / 49.8, 31.8 / 90.5; 128 channels, T = 9 and 16:
 // 63.7 / 74.2 and 74.4 / 149), but for a single token up to 10 items per SM (1 024 items 10.0 / 11.4, 1 920 13.4 / 12.7) and, with 128
 // channels, where an SM holds two of its CTAs, up to two items per SM for a single token (300 items 10.8 / 11.6, 400 11.3 / 11.2,
 // 3 840 53.5 / 18.9) and five for four (700 items 15.9 / 16.3, 1 024 19.8 / 17.7, 3 840 58 / 37).  With more keys the alternative is the
 // paired kernel's one launch (T = 16, 916 keys: 400 items 28.9 / 41.0, 3 840 items 225 / 240; 128 channels 340 / 344).
-// Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).  An append of several copies (`copies`),
-// 2 us each beside the paired kernel, keeps the first lines.
+// Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).
 bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies)
 {
     if (density && T <= kSmallMaxQueries) {
@@ -552,8 +558,9 @@ bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int 
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
     int line = D == 64 ? 19 : 6;
     if (density) line = D == 64 ? 20 : 7;
-    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? 7 : (T > 64 ? 0 : 6);
-    return units <= (int64_t)sm_count * line;
+    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? (T > 81 ? 7 : 19) : (T > 64 ? 0 : 6);
+    const bool one_wave = D == 128 || T <= 32 || items * ((T + 63) / 64) <= 2 * (int64_t)sm_count;   // (of CTAs of 64 queries)
+    return units <= (int64_t)sm_count * line && one_wave;
 }
 
 cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges, int32_t T,

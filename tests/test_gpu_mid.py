@@ -186,3 +186,21 @@ def test_densities_of_one_query_block_with_two_and_with_four_warps(rows):
             want = oracle.attention_density(to_items(q), Ks, runs, 0.125, heads)
             assert np.allclose(den.cpu().numpy(), want, rtol=2e-4, atol=1e-7), k
         assert B.amskv_status(c.h) == 0
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("side,items", [(6, (148, 150, 296, 300)), (9, (148, 150)), (10, (72, 76)), (11, (42, 46))])
+def test_more_ctas_than_are_resident_at_once(D, side, items):
+    """T = 36, 81, 100 and 121 at the item counts where the kernel changes: the second wave of its CTAs, and 7 units per SM."""
+    sides = (5, side)
+    for n in items:
+        rows, heads = n // 4 if n % 4 == 0 else n // 2, 4 if n % 4 == 0 else 2
+        qkv = make_qkv(rows, heads, sides, D, seed=103)
+        pick = [0, n // 2, n - 1]
+        for fused in (False, True):
+            with Cache(1, heads, D, rows, sides, [(1, 2, False)]) as c:
+                outs = run_pass(c, qkv, fused=fused)
+                want = oracle_outputs(qkv, (1, 2, False), 1.0 / math.sqrt(D), items=pick)
+                for k in range(2):
+                    got = outs[0][k].reshape(n, -1, D)[pick].cpu().double()
+                    check_close(got, want[k], "%d items scale %d" % (n, k))

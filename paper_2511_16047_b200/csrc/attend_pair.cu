@@ -1142,10 +1142,20 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
     int64_t grid = (int64_t)sm_count * C::kCtasPerSm;
     if (kSplit) grid = pp.full > 0 ? ((int64_t)sm_count * C::kCtasPerSm) & ~1ll : 2ll * pp.n_pairs;
     else if (grid > pp.n_pairs) grid = pp.n_pairs;
-    // (With a second round for less than half of the CTAs it matters that those with two units do not share SMs: launched onto
-    // an idle chip they do not, but onto SMs that come free one by one they do: T = 361, 256 items 49.9 -> 54.6 us.)
-    const int64_t slots = (int64_t)sm_count * C::kCtasPerSm;
-    const bool overlap = kExt || kDen || (overlaps_append(pp.n_items, T, D, sm_count) && (pp.n_pairs <= slots || 2 * (int64_t)pp.n_pairs > 3 * slots));
+    // Where SMs hold two CTAs and an eighth to two thirds of the CTAs have a unit in the last round, it matters that those do not
+    // share SMs: launched onto an idle chip they do not, but onto SMs that come free one by one they do.  us per call, with /
+    // without the overlap, fused: 400 items (1.35 rounds), T = 256 32.9 / 28.2; 180 items (2.43), T = 1 024 119.6 / 105.4; 1 024 items (3.46),
+    // T = 169 41.7 / 39.7, T = 256 57.3 / 52.3; 512 items (2.59), T = 361 67.6 / 65.8; 1 920 items (6.49), T = 256 95.3 / 92.3.  With shorter units
+    // the launch latency that is hidden is worth more (700 items, 1.18 rounds, T = 36 11.9 / 13.2, T = 100, three key tiles, 21.2 / 22.0; 1 920
+    // items, 3.24 rounds, T = 64 27.6 / 29.2), and with fewer or more units in the last round (300 items, 1.01 rounds, T = 169 19.1 / 20.3,
+    // T = 256 25.3 / 26.3; 512 items, 1.73, T = 256 32.2 / 32.5).  Behind a copy, which leaves SMs one by one: T = 361, 256 items 54.6 / 49.9; 96
+    // items, 144 units 27.5 / 23.8; T = 576, 48 items, 120 units 31.6 / 26.8; T = 256, 180 units 23.2 / 25.0.  (A density launch follows the small
+    // kernel that zeroes its result, on an idle chip.)
+    const int64_t slots = (int64_t)sm_count * C::kCtasPerSm, rest = pp.n_pairs % slots;
+    const bool uneven = !kWide && n_tiles >= 5 && pp.n_pairs > slots && 8 * rest > slots && 3 * rest <= 2 * slots;
+    const bool overlap = kDen || (kExt ? !uneven
+                                       : overlaps_append(pp.n_items, T, D, sm_count) && (kWide || pp.n_pairs > sm_count) &&
+                                         (pp.n_pairs <= slots || 2 * (int64_t)pp.n_pairs > 3 * slots));
     return launch_kernel(overlap, attend_pair_kernel<D, kExt, kWide, kDen, kLazy, kShort, kPieces, kSplit>, dim3((unsigned)grid), dim3(C::kThreads),
                          KernelMemory(C::kSmemBytes, kSplit ? 2u : 1u), stream, qm, km, vm, km64, vm64, ext, (__nv_bfloat16*)O.ptr, O.row, O.head, O.token,
                          ranges, T, heads, pp, n_tiles, qpos, scale_log2, status, den);

@@ -70,6 +70,64 @@ def test_reference_maximum_moves_in_every_key_tile(D, path, fused, step):
             check_close(outs[0][k], want[k], "D=%d scale %d" % (D, k), max_abs=2e-2)
 
 
+@pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
+@pytest.mark.parametrize("D,rows,heads,sides,step", [
+    (64, 5, 31, (8, 18), 8),      # 233 units, seven key tiles: two CTAs per SM
+    (64, 5, 31, (8, 18), 48),
+    (64, 10, 31, (8, 10), 48),    # 155 units, three key tiles: the same with the producer of short units
+    (64, 5, 31, (8, 10), 48),     # 78 units of two streams with tiles of their own: one CTA per SM, two S buffers
+    (64, 1, 74, (8, 18), 48),     # as many pairs as 74 + 37: both kinds of pairs
+    (128, 5, 31, (8, 18), 8),     # two streams, both kinds of pairs
+    (128, 5, 31, (8, 18), 48),
+    (128, 8, 11, (12, 25), 48),   # 220 units on 148 SMs: the last 72, of both kinds, shared by two CTAs each
+])
+def test_reference_maximum_moves_in_the_forms_of_large_launches(D, rows, heads, sides, step, fused):
+    """As above in launches of more query tiles than SMs, which is what large batches run."""
+    _need(D)
+    scale = 1.0 / 8 if D == 64 else 1.0 / 16
+    qkv, level = [], 0
+    for k, s in enumerate(sides):
+        qkv.append(synth.growing_logit_qkv(rows, heads, s * s, D, 86, k, first_level=level, step=step, device="cuda"))
+        level += (s * s + 63) // 64
+    n = rows * heads
+    assert n * ((sides[1] ** 2 + 127) // 128) > 148
+    pick = sorted({0, 1, n // 2 - 1, n // 2, n * 27 // 32, n - 2, n - 1})
+    with Cache(1, heads, D, rows, sides, [(0, 9, True)], softmax_scale=scale) as cache:
+        outs = run_pass(cache, qkv, B.PATH_TENSOR_PAIR, fused=fused)
+        want = oracle_outputs(qkv, (0, 9, True), scale, items=pick)
+        for k in range(len(sides)):
+            check_close(outs[0][k].reshape(n, -1, D)[pick].cpu().double(), want[k], "D=%d scale %d" % (D, k), max_abs=2e-2)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("rows,heads", [(3, 5), (5, 31)])
+def test_densities_when_the_reference_maximum_moves(D, rows, heads):
+    """The masses of earlier runs are brought to the new reference with the output (logits up to 2^69 apart per key tile)."""
+    _need(D)
+    sides, scale = (8, 9, 13), 1.0 / 8 if D == 64 else 1.0 / 16
+    qkv, level = [], 0
+    for k, s in enumerate(sides):
+        qkv.append(synth.growing_logit_qkv(rows, heads, s * s, D, 87, k, first_level=level, step=8, device="cuda"))
+        level += (s * s + 63) // 64
+    n = rows * heads
+    with Cache(1, heads, D, rows, sides, [(0, 9, True)], softmax_scale=scale) as cache:
+        B.amskv_set_attend_path(cache.h, B.PATH_TENSOR_PAIR)
+        for k, (q, kk, v) in enumerate(qkv):
+            B.amskv_append(cache.h, 0, k, kk, v)
+            runs = B.amskv_attended_tokens(cache.h, 0, k)
+            out = torch.full_like(q, float("nan"))
+            den = torch.full((heads, len(runs)), float("nan"), dtype=torch.float64, device="cuda")
+            B.amskv_attend_density(cache.h, 0, k, q, out, den, den.numel())
+            torch.cuda.synchronize()
+            Ks, Vs = [to_items(t[1]) for t in qkv[:k + 1]], [to_items(t[2]) for t in qkv[:k + 1]]
+            tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
+            check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, scale), "scale %d" % k, max_abs=2e-2)
+            want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
+            # arguments of up to 140 in units of log 2 are rounded at 2^-17: 1e-5 of an exponential, and as much of the sum
+            assert np.allclose(den.cpu().numpy(), want, rtol=1e-4, atol=1e-7), k
+        assert B.amskv_status(cache.h) == 0
+
+
 def test_a_wait_that_runs_out_is_reported_and_the_cache_stays_usable():
     """A bounded wait nothing ever satisfies: the kernel gives up after its iteration limit, records its
     code and returns; amskv_status reports it once; an ordinary pass on the same cache then succeeds."""

@@ -143,11 +143,46 @@ def test_paired_kernel_writes_an_append_in_pieces(D):
     assert copies == {1, 2, 3}
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("rows,heads", [(5, 40), (10, 30)])
+def test_appends_in_pieces_of_launches_that_fill_the_chip(D, rows, heads):
+    """The same in the forms that large batches run: 64 channels, 100 units of two streams with tiles of their own, one CTA per SM
+    (T <= 121 of 200 items), and 150 to 300 units, two CTAs per SM, of both kinds of pairs; 128 channels with two streams."""
+    sides = (2, 8, 8, 9, 11, 8, 13, 12)
+    budgets = [(133, 5), (128, 64), (200, 70), (150, 0), (64, 64)]
+    pols = [(1, 1, False)] * len(budgets)
+    n = rows * heads
+    pick = [0, 1, n // 2, n - 1]
+    qkv = make_qkv(rows, heads, sides, D, seed=104, peaked=True)
+
+    def items(x):
+        return x.reshape(n, -1, D)[pick].cpu().double().numpy()
+
+    Ks, Vs = [items(k) for _, k, _ in qkv], [items(v) for _, _, v in qkv]
+    copies = set()
+    with Cache(len(pols), heads, D, rows, sides, pols, token_budgets=budgets) as c:
+        B.amskv_set_attend_path(c.h, B.PATH_TENSOR_PAIR)
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(pols)):
+                out = torch.full_like(q, float("nan"))
+                n0 = B.amskv_launch_count()
+                B.amskv_append_attend(c.h, layer, k, kk, v, q, out)
+                assert B.amskv_launch_count() - n0 == 1
+                copies.add(len(B.amskv_append_copies(c.h, layer, k)))
+                tokens = [(s, t) for s, first, count in B.amskv_attended_tokens(c.h, layer, k) for t in range(first, first + count)]
+                check_close(torch.from_numpy(items(out)), oracle.attend_tokens(items(q), Ks, Vs, tokens, 1.0 / math.sqrt(D)),
+                            "layer %d scale %d" % (layer, k), max_abs=4e-2)
+        assert B.amskv_status(c.h) == 0
+    assert copies == {1, 2, 3}
+
+
 @pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
 @pytest.mark.parametrize("rows,heads,sides", [
-    (5, 31, (3, 28)),          # 155 items, seven query tiles: 620 units, 28 left over after four rounds of 148
-    (2, 16, (16, 17, 25)),     # 32 items, five query tiles at the end, pairs of both kinds: 80 units, none whole
+    (5, 31, (3, 28)),          # 155 items, seven query tiles: 543 units, 99 left over after three rounds of 148: not split
+    (2, 16, (16, 17, 25)),     # 32 items, five query tiles at the end, pairs of both kinds: 80 units: not split
     (1, 150, (5, 27)),         # 150 items, six query tiles (the last ragged): 450 units, six left over
+    (8, 11, (12, 25)),         # 88 items, five query tiles: 220 units, of both kinds, 72 left over, 28 of two tiles of an item
+    (2, 35, (12, 25)),         # 70 items: 175 units, 27 left over, all of two items' last tiles
 ])
 def test_last_round_shared_by_two_ctas(rows, heads, sides, fused):
     """128 channels, launches whose last round of units is split over clusters of two CTAs: odd and even numbers of key tiles,

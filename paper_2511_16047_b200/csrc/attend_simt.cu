@@ -17,13 +17,6 @@ constexpr int kThreads = 128;
 constexpr int kLanesPerRow = 8;
 constexpr int kKeysPerStep = 4;
 
-__device__ __forceinline__ float fast_exp2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 template <int N>
 __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&f)[N])
 {

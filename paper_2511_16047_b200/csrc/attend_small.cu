@@ -34,13 +34,6 @@ namespace {
 constexpr int kWarpsPerCta = 2;     // (4: the same above 3 000 items, up to 10 % slower where the items leave SMs idle)
 static_assert(kSmallMaxKeys == 32, "the register tile is instantiated for 1, 2 and 4 eight-key tiles");
 
-__device__ __forceinline__ float fast_exp2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // D (16x8, fp32) += A (16x16, bf16, row-major) * B (16x8, bf16, column-major)
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                           uint32_t b1)

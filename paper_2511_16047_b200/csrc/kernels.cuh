@@ -210,6 +210,12 @@ __device__ __forceinline__ void overlap_with_previous()
     wait_for_previous();
     let_next_start();
 }
+__device__ __forceinline__ float fast_exp2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 // Loads of what an earlier launch wrote or the caller passed.  A kernel that is alive while its predecessor still writes may not
 // use the read-only path (ld.global.nc, which __ldg and const __restrict__ pointers lead to: the data must not change while
 // the kernel runs, and the compiler may move such a load above the wait).  These are ordinary loads that stay behind it.

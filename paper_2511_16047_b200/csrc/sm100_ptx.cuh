@@ -280,12 +280,6 @@ __device__ __forceinline__ void st_global_32B(void* p, uint32_t a, uint32_t b, u
                  : "memory");
 }
 
-__device__ __forceinline__ float fast_exp2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 // Packed single-precision pairs (two lanes per instruction on sm_100).
 __device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b0, float b1, float c0, float c1)
 {

@@ -38,7 +38,7 @@ FALLBACK_BF16_TFLOPS = 1400.0
 NCU_DOMINANT_KERNEL_TRAFFIC = {
     ("var_d30", "ams", "fused"): {
         "bytes_per_launch": 1.645e9,
-        "capture": "profiles/attention_dram_traffic_var_d30.md: 64-row, 2-layer case of the same shape, every launch of "
+        "capture": "ncu, attention_dram_traffic_var_d30 of profiles/: 64-row, 2-layer case of the same shape, every launch of "
                    "attend_pair_kernel<64, ext> of one step, scaled by rows (x 8) and by the layers of each class (21 + 9), "
                    "averaged over its 150 launches; reads exact, writes a lower bound (part of them still in L2 at that size)"},
 }

@@ -193,7 +193,7 @@ void note_appended(amskv_cache* cache, int layer, int scale)
 
 // which kernel amskv_attend uses for T query tokens over `total` keys
 enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
-// (copies: the call includes an append of several copies, which only the warp-matrix kernel takes in)
+// (copies: the call includes an append that is not one contiguous copy; see mid_preferred)
 AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool copies = false)
 {
     // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained); for a single query token,
@@ -461,9 +461,9 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         note_appended(cache, layer, scale);
         return AMSKV_OK;
     }
-    // One launch where the paired kernel serves this scale and the append is a single copy: the kernel
-    // reads the scale from K and V, attends to it together with the older retained tokens, and writes
-    // it to its place in the cache on the way.  Elsewhere: the two calls, one after the other.
+    // One launch where the warp-per-item, the warp-matrix or the paired kernel serves this scale: the kernel reads the scale
+    // from K and V, attends to it together with the older retained tokens, and writes it to its place in the cache on the
+    // way (the first only where the append is a single copy).  Elsewhere: the two calls, one after the other.
     RangeList after;
     after.n = lay.ranges(cache->tokens, scale, after.r);
     after.total = 0;
@@ -627,8 +627,8 @@ int amskv_attend_density(amskv_cache* cache, int layer, int scale, const void* Q
     if (n < 0) return AMSKV_ERR_UNSUPPORTED;   // the scale's own keys are not in the cache (never-stored last scale)
     int32_t total = 0;
     for (int32_t i = 0; i < n; ++i) total += rp[i].len;
-    // One launch where the paired or the warp-matrix kernel serves the scale: the former cuts its key tiles at the
-    // boundaries of the runs (one range per piece of a run), the latter multiplies P by the keys' run membership.
+    // One launch where the paired or the warp-matrix kernel serves the scale (one range per piece of a run): the former adds up
+    // the sums of 16-key boxes, which belong to one run each, the latter multiplies P by the keys' run membership.
     const AttendKernel kernel = choose_kernel(cache, T, total, true);
     if (cache->tc_ready && (kernel == AttendKernel::Pair || kernel == AttendKernel::Mid) && n_runs <= kPairMaxDensityRuns && n <= kMaxRanges) {
         RangeList ranges;

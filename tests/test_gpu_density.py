@@ -66,9 +66,7 @@ def test_order_and_argument_errors():
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("peaked", [False, True], ids=["flat", "peaked"])
 def test_density_as_a_by_product_of_the_attention_launch(D, peaked):
-    """amskv_attend_density: the output equals amskv_attend's bit for bit where both run the paired kernel on
-    the same tiles (and the oracle everywhere), and the density equals the oracle's -- whole scales and token
-    budgets, more units than CTAs, query tiles with idle warps, rows whose reference maximum moves (peaked)."""
+    """amskv_attend_density: the output and the density are the oracle's -- whole scales and token budgets, more units than CTAs, query tiles with idle warps, rows whose reference maximum moves (peaked)."""
     from gpu_common import check_close, oracle_outputs
     sides, rows, heads = (1, 2, 3, 5, 6, 8, 13), 6, 40
     qkv = make_qkv(rows, heads, sides, D, seed=63, peaked=peaked)

@@ -95,7 +95,7 @@ def test_left_over_cache_tokens_ride_in_the_spare_box_of_the_last_tile(D):
 
 
 def test_token_budgets_fused():
-    """Under token budgets the fused path takes the appends that are one copy; the rest run as two calls."""
+    """Under token budgets the fused path takes appends of one copy and of several."""
     _need()
     sides, rows, heads, D = (1, 2, 3, 4, 5, 6, 8, 10), 2, 6, 64
     budgets = [(500, 5), (100, 5), (70, 0), (13, 3), (64, 14), (120, 5)]

@@ -48,7 +48,6 @@ def _run(D, rows, heads, fused, budgets=None, flags=0, peaked=False, packed=Fals
                             "layer %d scale %d" % (layer, k), max_abs=4e-2 if peaked else 1e-2)
                 if density:
                     want = oracle.attention_density(to_items(q), Ks, runs, scale, heads)
-                    # masses from 16 bits of P and fp32 sums: the tolerance of the paired kernel's densities holds too
                     assert np.allclose(den.cpu().numpy(), want, rtol=2e-4, atol=1e-7), (layer, k)
         assert B.amskv_status(c.h) == 0
 
@@ -239,3 +238,25 @@ def test_more_ctas_than_are_resident_at_once(D, side, items):
                 for k in range(2):
                     got = outs[0][k].reshape(n, -1, D)[pick].cpu().double()
                     check_close(got, want[k], "%d items scale %d" % (n, k))
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("path", ["SIMT", "TENSOR", "AUTO", "TENSOR_PAIR"])
+def test_an_item_does_not_depend_on_the_values_of_others_nor_beyond_rounding_on_their_number(D, path):
+    """The items of one image alone and as the first of many, in all forms that the number of items chooses."""
+    sides, heads = (1, 3, 4, 6, 8, 11, 17), 4
+    most = make_qkv(80, heads, sides, D, seed=105)
+    outs = {}
+    for rows in (1, 13, 40, 80):
+        qkv = [tuple(x[:rows].contiguous() for x in t) for t in most]
+        with Cache(1, heads, D, rows, sides, [(2, 2, False)]) as c:
+            outs[rows] = [o[:1].double() for o in run_pass(c, qkv, getattr(B, "PATH_" + path), fused=path in ("AUTO", "TENSOR_PAIR"))[0]]
+            again = run_pass(c, [(t[0], t[1], torch.cat([t[2][:1], -t[2][1:]])) for t in qkv], getattr(B, "PATH_" + path),
+                             fused=path in ("AUTO", "TENSOR_PAIR"))[0]
+            assert all(torch.equal(x, y[:1].double()) for x, y in zip(outs[rows], again))
+    for rows in (13, 40, 80):
+        for x, y in zip(outs[1], outs[rows]):
+            if path in ("SIMT", "TENSOR"):
+                assert torch.equal(x, y)
+            else:   # each within 2.5e-3 of exact sums
+                assert (x - y).norm() <= 5e-3 * x.norm()

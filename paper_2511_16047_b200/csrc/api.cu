@@ -537,6 +537,10 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         // five, 256 items: 26.7 / 23.6).  Appends of several copies, which the producer writes partly row by row, take it above
         // 128 queries only (1 920 items, ten layers: T = 256 1 046 / 1 028, T = 100 487 / 554).  A launch of at most one unit per
         // SM fuses anyway: another key tile is 0.8 us there, the copy 2 (T = 100, 256 items: 16.9 / 13.6).
+        // Swept with the append fused wherever it can be against two calls, 240 to 3 840 items: 64 channels win fused at every T of the
+        // schedules (T = 36 to 361, by 1 to 40 %) but T = 100 with 255 keys at 1 920 items (55.4 / 53.4); 128 channels but T = 81 with
+        // three tiles from 700 items up (35.4 / 35.0, 1 920 96 / 90); several copies lose at T = 100, 64 channels from 700 items (28.8 /
+        // 24.8), 128 from 300 (28.1 / 25.9), at T = 36 from 700 to 1 920 items (128 channels 24.5 / 22.4), and win at T = 169 (700 items 27.8 / 33.9).
         // (AMSKV_PATH_TENSOR_PAIR fuses wherever it can.)
         auto tiles = [](const RangeList& rl) {
             int32_t n = 0;

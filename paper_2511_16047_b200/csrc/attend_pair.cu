@@ -1148,9 +1148,11 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
     // T = 169 41.7 / 39.7, T = 256 57.3 / 52.3; 512 items (2.59), T = 361 67.6 / 65.8; 1 920 items (6.49), T = 256 95.3 / 92.3.  With shorter units
     // the launch latency that is hidden is worth more (700 items, 1.18 rounds, T = 36 11.9 / 13.2, T = 100, three key tiles, 21.2 / 22.0; 1 920
     // items, 3.24 rounds, T = 64 27.6 / 29.2), and with fewer or more units in the last round (300 items, 1.01 rounds, T = 169 19.1 / 20.3,
-    // T = 256 25.3 / 26.3; 512 items, 1.73, T = 256 32.2 / 32.5).  Behind a copy, which leaves SMs one by one: T = 361, 256 items 54.6 / 49.9; 96
-    // items, 144 units 27.5 / 23.8; T = 576, 48 items, 120 units 31.6 / 26.8; T = 256, 180 units 23.2 / 25.0.  (A density launch follows the small
-    // kernel that zeroes its result, on an idle chip.)
+    // T = 256 25.3 / 26.3; 512 items, 1.73, T = 256 32.2 / 32.5).
+    // Behind a copy, which leaves SMs one by one: up to a unit per SM, 80 units (T = 576) 29.8 / 24.9, 111 (T = 361) 25.0 / 22.6, 144 (T = 361) 27.1 /
+    // 23.3, but 90 (T = 324) 17.5 / 18.9; beyond, 180 (T = 225) 22.9 / 23.6, 256 (T = 121) 20.4 / 22.2; 350 (T = 100) 29.4 / 30.4, 384 (T = 1 024) 90.2 /
+    // 79.1, 400 (T = 169, 225, 256) 34.5 / 33.1, 37.6 / 35.6, 51.9 / 46.6; 512 (T = 256) 52.7 / 55.6.  (A density launch follows the small kernel that
+    // zeroes its result, on an idle chip.)
     const int64_t slots = (int64_t)sm_count * C::kCtasPerSm, rest = pp.n_pairs % slots;
     const bool uneven = !kWide && n_tiles >= 5 && pp.n_pairs > slots && 8 * rest > slots && 3 * rest <= 2 * slots;
     const bool overlap = kDen || (kExt ? !uneven

@@ -241,13 +241,15 @@ attend_mid_kernel(const __nv_bfloat16* Q, int64_t q_row, int64_t q_head, int64_t
         for (int i = 0; i < kRows; ++i) {
             const int32_t j = c * kChunk + cp_row0 + i * kStep - Lc;
             if (j < 0 || j >= ext.len) continue;
-            int32_t d = -1;
-            for (int n = 0; n < ext.n_pieces; ++n)
-                if (j >= ext.piece[n].src && j < ext.piece[n].src + ext.piece[n].len) d = ext.piece[n].dst + j - ext.piece[n].src;
-            if (d < 0) continue;
-            __nv_bfloat16* kd = kbase + (int64_t)d * D + cp_piece * 8;
-            *reinterpret_cast<uint4*>(kd) = *reinterpret_cast<const uint4*>(tile + k_slot + i * kStep * C::kRowBytes);
-            *reinterpret_cast<uint4*>(kd + v_shift) = *reinterpret_cast<const uint4*>(tile + v_slot + i * kStep * C::kRowBytes);
+            const uint4 kv = *reinterpret_cast<const uint4*>(tile + k_slot + i * kStep * C::kRowBytes);
+            const uint4 vv = *reinterpret_cast<const uint4*>(tile + v_slot + i * kStep * C::kRowBytes);
+            // (a token can have two places: in the ring or its head, and in the slot of a scale that is attended from there)
+            for (int n = 0; n < ext.n_pieces; ++n) {
+                if (j < ext.piece[n].src || j >= ext.piece[n].src + ext.piece[n].len) continue;
+                __nv_bfloat16* kd = kbase + (int64_t)(ext.piece[n].dst + j - ext.piece[n].src) * D + cp_piece * 8;
+                *reinterpret_cast<uint4*>(kd) = kv;
+                *reinterpret_cast<uint4*>(kd + v_shift) = vv;
+            }
         }
     };
 

@@ -66,6 +66,36 @@ def test_appends_of_several_copies_are_one_launch(D):
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("path", [B.PATH_AUTO, B.PATH_TENSOR_PAIR], ids=["auto", "pair"])
+def test_tokens_with_two_places(D, path):
+    """Scales that are attended from a slot of their own and also leave tokens in the ring or its pinned head: those tokens are
+    written twice by one append, and later scales read them from the ring."""
+    budgets = [(58, 12), (40, 30), (70, 60), (100, 95), (45, 20), (30, 7)]
+    rows, heads, scale = 2, 3, 1.0 / math.sqrt(D)
+    qkv = make_qkv(rows, heads, SIDES, D, seed=106, peaked=True)
+    Ks, Vs = [to_items(k) for _, k, _ in qkv], [to_items(v) for _, _, v in qkv]
+    twice, read_later = [set() for _ in budgets], [False] * len(budgets)
+    with Cache(len(budgets), heads, D, rows, SIDES, [(1, 1, False)] * len(budgets), token_budgets=budgets) as c:
+        c.arena.fill_(0x3f)                                    # a place that is not written holds 0.75
+        torch.cuda.synchronize()
+        c.arena[:4].zero_()                                    # (the status word)
+        B.amskv_set_attend_path(c.h, path)
+        for k, (q, kk, v) in enumerate(qkv):
+            for layer in range(len(budgets)):
+                out = torch.full_like(q, float("nan"))
+                B.amskv_append_attend(c.h, layer, k, kk, v, q, out)
+                runs = B.amskv_attended_tokens(c.h, layer, k)
+                copies = sorted((src, src + n) for src, _, n in B.amskv_append_copies(c.h, layer, k))
+                if any(b[0] < a[1] for a, b in zip(copies, copies[1:])):
+                    twice[layer].add(k)
+                read_later[layer] |= any(s in twice[layer] and s != k for s, _, _ in runs)
+                tokens = [(s, t) for s, first, count in runs for t in range(first, first + count)]
+                check_close(out, oracle.attend_tokens(to_items(q), Ks, Vs, tokens, scale), "layer %d scale %d" % (layer, k), max_abs=4e-2)
+        assert B.amskv_status(c.h) == 0
+    assert all(read_later)
+
+
+@pytest.mark.parametrize("D", [64, 128])
 def test_never_stored_last_scale(D):
     _run(D, 2, 3, True, flags=B.FLAG_TRANSIENT_LAST_SCALE)
 

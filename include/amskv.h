@@ -91,14 +91,12 @@ extern "C" {
                                idle in the paired tcgen05 kernel, that kernel otherwise             */
 #define AMSKV_PATH_SIMT 1   /* always the CUDA-core kernel                                     */
 #define AMSKV_PATH_TENSOR 2 /* always the single-stream tcgen05 kernel                         */
-#define AMSKV_PATH_TENSOR_PAIR 3 /* always the paired tcgen05 kernel (two query tiles per CTA; one where
-                                    a launch has an SM for every tile)                              */
+#define AMSKV_PATH_TENSOR_PAIR 3 /* always the paired tcgen05 kernel (two query tiles per CTA)  */
 #define AMSKV_PATH_SMALL 4  /* the warp-per-item kernel wherever it applies (paired kernel elsewhere) */
-/* Outputs do not depend on the values of other rows and heads, and a call repeated is bit-equal.  Under AUTO,
- * TENSOR_PAIR and SMALL the kernel, its form and the order of its key tiles are chosen by rows x heads and the number
- * of SMs as well as by the scale, so the outputs of an image computed together with other numbers of images may
- * differ in rounding (2e-3 in the 2-norm, as both do from exact sums).  Under SIMT and TENSOR they depend on the image
- * alone. */
+/* Outputs do not depend on the values of other rows and heads, and a call repeated is bit-equal.  Under AUTO the kernel,
+ * its form and the order of its key tiles are chosen by rows x heads and the number of SMs as well as by the scale, so the
+ * outputs of an image computed together with other numbers of images may differ in rounding (2e-3 in the 2-norm, as both
+ * do from exact sums).  Under every other path the scale alone decides, and they are bit-equal. */
 
 typedef struct amskv_cache amskv_cache; /* opaque; owned by the library */
 

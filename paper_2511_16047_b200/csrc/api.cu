@@ -401,7 +401,7 @@ int amskv_attend(amskv_cache* cache, int layer, int scale, const void* Q, void* 
         e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes,
                                cache->k_maps64[layer].bytes, cache->v_maps64[layer].bytes, ranges, T, cache->rows,
                                cache->heads, cache->head_dim, cache->softmax_scale, cache->status_word(),
-                               cache->sm_count, static_cast<cudaStream_t>(stream));
+                               cache->sm_count, static_cast<cudaStream_t>(stream), nullptr, nullptr, cache->path != AMSKV_PATH_AUTO);
     } else if (kernel == AttendKernel::Tensor) {
         e = launch_attend_tc(q, o, cache->region(layer), cache->k_maps[layer].bytes, cache->v_maps[layer].bytes, ranges,
                              T, cache->rows, cache->heads, cache->head_dim, cache->softmax_scale, cache->status_word(),
@@ -453,7 +453,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
             e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes, cache->k_maps64[layer].bytes,
                                    cache->v_maps64[layer].bytes, rl, T, cache->rows, cache->heads, cache->head_dim,
                                    cache->softmax_scale, cache->status_word(), cache->sm_count,
-                                   static_cast<cudaStream_t>(stream), &src);
+                                   static_cast<cudaStream_t>(stream), &src, nullptr, cache->path != AMSKV_PATH_AUTO);
         else
             e = launch_attend_simt(q, o, cache->region(layer), rl, T, cache->rows, cache->heads, cache->head_dim,
                                    cache->softmax_scale, static_cast<cudaStream_t>(stream), &src);
@@ -573,7 +573,8 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
     cudaError_t e = launch_attend_pair(q, o, cache->k_maps[layer].bytes, cache->v_maps[layer].bytes,
                                        cache->k_maps64[layer].bytes, cache->v_maps64[layer].bytes, ranges, T, cache->rows,
                                        cache->heads, cache->head_dim, cache->softmax_scale, cache->status_word(),
-                                       cache->sm_count, static_cast<cudaStream_t>(stream), &cur);
+                                       cache->sm_count, static_cast<cudaStream_t>(stream), &cur, nullptr,
+                                       cache->path != AMSKV_PATH_AUTO);
     if (e != cudaSuccess) { (void)cudaGetLastError(); return AMSKV_ERR_CUDA; }
     note_appended(cache, layer, scale);
     return AMSKV_OK;

@@ -1168,7 +1168,7 @@ cudaError_t launch(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorM
 cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k_map, const void* v_map,
                                const void* k_map64, const void* v_map64, const RangeList& ranges, int32_t T, int32_t rows, int32_t heads, int32_t D,
                                float softmax_scale, int* status, int sm_count, cudaStream_t stream,
-                               const CurrentScaleSource* cur, const PairDensity* density)
+                               const CurrentScaleSource* cur, const PairDensity* density, bool fixed_form)
 {
     if (ranges.n < 1 || ranges.total < 1 || T < 1) return cudaErrorInvalidValue;
     DenArgs<true> den;
@@ -1253,7 +1253,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // 10.1 / 7.7, T = 169 11.1 / 9.6, T = 256 14.2 / 11.7; 32 items, T = 256 13.2 / 10.9; 128 channels, 32 items: T = 144 12.9 /
     // 10.3, T = 256 14.5 / 12.3, T = 400 23.6 / 20.7; 16 items, T = 576 35.3 / 22.6.  With more tiles than SMs the pairs win (128
     // channels, 32 items, T = 576, 160 tiles: 38.3 / 40.9).
-    if (!density && pair_one_tile_per_sm(pp.n_items, T, sm_count)) {
+    if (!density && !fixed_form && pair_one_tile_per_sm(pp.n_items, T, sm_count)) {
         pp.kind = 3;
         pp.n_shared = 0;
         pp.n_pairs = pp.n_items * pp.nqt;
@@ -1291,7 +1291,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // measured 2 % faster there).
     // Writes in several pieces are instantiated for the lazy form only.
     constexpr int lazy_min = 3, lazy128_min = 3, short_max = 4, split_min = 12;
-    if (D == 128 && !density && ext.n_pieces == 0 && pp.kind != 3) {
+    if (D == 128 && !density && !fixed_form && ext.n_pieces == 0 && pp.kind != 3) {
         // The last round of units often leaves most SMs idle.  Where at most half of them have a unit in it (and there is
         // something to halve: a merge costs about five key tiles), two CTAs share each of its units.  us per call, before /
         // after: 32 items, T = 1 600 (208 units on 148 SMs) 139 / 105, T = 4 096 (512) 535 / 491; 48 items, T = 1 024 (192) 82 / 68;
@@ -1319,7 +1319,7 @@ cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k
     // the next tile off the chain, costs no parallelism (T = 256, 60 items 13.8 -> 12.8 us, 128 items 15.2 -> 14.6; T = 1 024, 36
     // items, 144 units 37.9 -> 33.4; with 256 units 21.0 -> 24.3).  Not for launches of both kinds of pairs (T = 576, 36 items:
     // 23.6 -> 24.7).
-    if (pp.n_pairs <= sm_count && pp.kind != 2) {
+    if (!fixed_form && pp.n_pairs <= sm_count && pp.kind != 2) {
         if (ext.n_pieces > 0) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true, true);
         if (cur) AMSKV_PAIR_LAUNCH(64, true, true, false, true, true, false);
         AMSKV_PAIR_LAUNCH(64, false, true, false, true, true, false);

@@ -112,11 +112,12 @@ inline int64_t pair_units(int64_t items, int32_t T)
     return items * (nqt / 2) + ((nqt & 1) ? (items + 1) / 2 : 0);
 }
 
-// Paired tensor-core kernel: two softmax groups per CTA, probabilities kept in tensor memory.
+// Paired tensor-core kernel: two softmax groups per CTA, probabilities kept in tensor memory.  fixed_form: the form is chosen by the
+// scale alone (two query tiles per CTA), so that an item's result does not depend on the number of items.
 cudaError_t launch_attend_pair(const Strided& Q, const Strided& O, const void* k_map16, const void* v_map16,
                                const void* k_map64, const void* v_map64, const RangeList& ranges, int32_t T, int32_t rows, int32_t heads, int32_t D,
                                float softmax_scale, int* status, int sm_count, cudaStream_t stream,
-                               const CurrentScaleSource* cur = nullptr, const PairDensity* density = nullptr);
+                               const CurrentScaleSource* cur = nullptr, const PairDensity* density = nullptr, bool fixed_form = false);
 
 // Warp-per-item kernel for the coarse scales: every retained key in one register tile.
 constexpr int kSmallMaxKeys = 32;

@@ -70,18 +70,19 @@ def test_reference_maximum_moves_in_every_key_tile(D, path, fused, step):
             check_close(outs[0][k], want[k], "D=%d scale %d" % (D, k), max_abs=2e-2)
 
 
+@pytest.mark.parametrize("path", [B.PATH_AUTO, B.PATH_TENSOR_PAIR], ids=["auto", "pair"])
 @pytest.mark.parametrize("fused", [False, True], ids=["separate", "fused"])
 @pytest.mark.parametrize("D,rows,heads,sides,step", [
     (64, 5, 31, (8, 18), 8),      # 233 units, seven key tiles: two CTAs per SM
     (64, 5, 31, (8, 18), 48),
     (64, 10, 31, (8, 10), 48),    # 155 units, three key tiles: the same with the producer of short units
-    (64, 5, 31, (8, 10), 48),     # 78 units of two streams with tiles of their own: one CTA per SM, two S buffers
+    (64, 5, 31, (8, 10), 48),     # 78 units of two streams with tiles of their own: one CTA per SM, two S buffers (auto)
     (64, 1, 74, (8, 18), 48),     # as many pairs as 74 + 37: both kinds of pairs
     (128, 5, 31, (8, 18), 8),     # two streams, both kinds of pairs
     (128, 5, 31, (8, 18), 48),
-    (128, 8, 11, (12, 25), 48),   # 220 units on 148 SMs: the last 72, of both kinds, shared by two CTAs each
+    (128, 8, 11, (12, 25), 48),   # 220 units on 148 SMs: the last 72, of both kinds, shared by two CTAs each (auto)
 ])
-def test_reference_maximum_moves_in_the_forms_of_large_launches(D, rows, heads, sides, step, fused):
+def test_reference_maximum_moves_in_the_forms_of_large_launches(D, rows, heads, sides, step, fused, path):
     """As above in launches of more query tiles than SMs, which is what large batches run."""
     _need(D)
     scale = 1.0 / 8 if D == 64 else 1.0 / 16
@@ -93,7 +94,7 @@ def test_reference_maximum_moves_in_the_forms_of_large_launches(D, rows, heads, 
     assert n * ((sides[1] ** 2 + 127) // 128) > 148
     pick = sorted({0, 1, n // 2 - 1, n // 2, n * 27 // 32, n - 2, n - 1})
     with Cache(1, heads, D, rows, sides, [(0, 9, True)], softmax_scale=scale) as cache:
-        outs = run_pass(cache, qkv, B.PATH_TENSOR_PAIR, fused=fused)
+        outs = run_pass(cache, qkv, path, fused=fused)
         want = oracle_outputs(qkv, (0, 9, True), scale, items=pick)
         for k in range(len(sides)):
             check_close(outs[0][k].reshape(n, -1, D)[pick].cpu().double(), want[k], "D=%d scale %d" % (D, k), max_abs=2e-2)

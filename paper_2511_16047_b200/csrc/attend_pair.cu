@@ -111,7 +111,7 @@ struct Barriers {
     uint64_t q_full[2][2];     // [stream][half]: see kQSplitRows
     uint64_t kv_full[kMaxStages], kv_empty[kMaxStages];
     uint64_t s_full[2][2], p_full[2][2];   // [stream][S buffer]
-    uint64_t o_full[2], pv_done[2];
+    uint64_t o_full[2], pv_done[2], drained[2];
     uint32_t tmem_base;
     int abort_flag;
     int2 tile_tab[kTileTab];
@@ -282,6 +282,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
             mbar_init(smem_u32(&bars->pv_done[g]), 1);
             mbar_init(smem_u32(&bars->o_full[g]), 1);
+            mbar_init(smem_u32(&bars->drained[g]), 1);
         }
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(smem_u32(&bars->kv_full[s]), 1);
@@ -604,72 +605,78 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // stage counter advances alike in both.  A commit covers the issuing thread's own instructions only,
         // hence a key/value stage is released by one arrival per issuing warp: each commits its own P V on a
         // shared tile, and the one stream that uses a tile of its own commits twice.
-        const int my_g = C::kMmaWarps == 2 ? warp - kMmaWarp : -1;   // -1: this warp issues for both streams
+        //
+        // A warp's own instructions are what a tile costs here: a satisfied wait of a voting warp 220 clocks, a branch into the
+        // elected lane and back 130, the bookkeeping of a tile 500, against 320 (64 channels) and 640 clocks of products.  So a
+        // wait that gives up does not change the course (it sets the abort flag, after which no wait waits), a product's
+        // instructions and commits are one predicated block, and a tile's length is fetched a tile ahead.  Eight images, T = 4 096,
+        // 128 channels: 4 836 -> 4 717 us a call at the same power; one image, T = 576 and 1 600: 35.7 -> 31.5 and 98.3 -> 93.4; 64
+        // channels, 256 items, T = 64 and 100: 9.35 -> 9.05 and 11.9 -> 11.6, and no change where the softmax warps fill the SM.
+        const int my_g = C::kMmaWarps == 2 ? warp - kMmaWarp : 0;
         if (my_pairs > 0) {
-            bool ok = true;
+            constexpr int kStreams = C::kMmaWarps == 2 ? 1 : 2;   // streams this warp issues for
+            
             const uint32_t idesc_pv = make_idesc(kQRows, D, 1);
             const uint32_t k_lo0 = desc_lo(kv_smem, 16);                             // K tile of stage 0, K-major
             const uint32_t v_lo0 = desc_lo(kv_smem + C::kKVBytes, C::kKVHalfBytes);  // V tile of stage 0, MN-major
             const uint32_t q_lo0 = desc_lo(q_smem, 16);
             constexpr uint32_t kStageLo = C::kStageBytes >> 4, kQLo = C::kQBytes >> 4;
+            auto await = [&](const uint32_t bar, const uint32_t parity) { wait_through(bar, parity, status, kStatusMmaTimeout, abort_flag); };
             // per stream: the tile whose S was issued last and whose P V is still to be issued
-            uint32_t pv_stage[2] = {0, 0}, pv_nch[2] = {0, 0}, pv_t[2] = {0, 0};
-            bool pv_live[2] = {false, false}, pv_first[2] = {false, false}, pv_release[2] = {false, false},
-                 pv_last[2] = {false, false}, pv_twice[2] = {false, false};
-            uint32_t tcount[2] = {0, 0};   // tiles issued per stream
-            uint32_t ucount[2] = {0, 0};   // units started per stream
-            uint32_t q_half[2] = {0, 0};   // half of the query slot the current unit of each stream uses
+            uint32_t pv_stage[kStreams] = {}, pv_nch[kStreams] = {}, pv_first[kStreams] = {}, pv_last[kStreams] = {},
+                     pv_release[kStreams] = {}, pv_twice[kStreams] = {};
+            bool pv_live[kStreams] = {};
+            uint32_t tcount[kStreams] = {};   // tiles issued per stream
+            uint32_t ucount[kStreams] = {};   // units started per stream
+            uint32_t q_half[kStreams] = {};   // half of the query slot the current unit of each stream uses
             uint32_t sq = 0;
 
             // O (+)= P V : M = 128, N = D channels, K = 16 * nch tokens; P from TMEM (packed over S),
             // V read MN-major from its stage
-            auto issue_pv = [&](const int g) -> bool {
-                const uint32_t t = pv_t[g];  // flat tile index of this stream
-                if (!warp_wait(p_full0 + 16 * g + 8 * buf_of(t), par_of(t), abort_flag)) return false;
+            auto issue_pv = [&](const int i) {
+                const int g = kStreams == 2 ? i : my_g;
+                const uint32_t t = tcount[i] - 1u;  // flat tile index of this stream
+                await(p_full0 + 16 * g + 8 * buf_of(t), par_of(t));
                 // (a unit's first P V overwrites O: every warp of the group arrives on p_full for that tile
                 // only after its epilogue of the previous unit, so O has been read by then)
                 tc_fence_after();
-                const uint32_t v_lo = v_lo0 + pv_stage[g] * kStageLo;
-                const uint32_t p_tmem = tmem + C::kSCol + (g * C::kSBufs + buf_of(t)) * kKT;
-                const uint32_t o_tmem = tmem + C::kOCol + g * D;
-                const uint32_t nch = pv_nch[g];
-                if (elect_one()) {
-                    umma_ts(o_tmem, p_tmem, v_lo, kDescHi, idesc_pv, pv_first[g] ? 0u : 1u);
-                    if (nch > 1) umma_ts(o_tmem, p_tmem + 8, v_lo + (2048 >> 4), kDescHi, idesc_pv, 1u);
-                    if (nch > 2) umma_ts(o_tmem, p_tmem + 16, v_lo + (4096 >> 4), kDescHi, idesc_pv, 1u);
-                    if (nch > 3) umma_ts(o_tmem, p_tmem + 24, v_lo + (6144 >> 4), kDescHi, idesc_pv, 1u);
-                    if (pv_release[g]) umma_commit(kv_empty0 + 8 * pv_stage[g]);
-                    if (C::kMmaWarps == 2 && pv_twice[g]) umma_commit(kv_empty0 + 8 * pv_stage[g]);
-                    if (pv_last[g]) umma_commit(o_full0 + 8 * g);
-                    if (C::kSBufs == 2) umma_commit(pv_done0 + 8 * g);   // read by the (rare) rescale of O only
+                const uint32_t empty = kv_empty0 + 8 * pv_stage[i];
+                umma_pv(tmem + C::kOCol + g * D, tmem + C::kSCol + (g * C::kSBufs + buf_of(t)) * kKT,
+                             v_lo0 + pv_stage[i] * kStageLo, kDescHi, idesc_pv, pv_first[i] ^ 1u, pv_nch[i], pv_release[i], empty,
+                             pv_last[i], o_full0 + 8 * g);
+                if (C::kMmaWarps == 2) {
+                    if (pv_twice[i]) umma_commit_elected(empty);
+                    umma_commit_elected(pv_done0 + 8 * g);   // read by the (rare) rescale of O only
                 }
-                __syncwarp();
-                return true;
+            };
+            auto tile_steps = [&](const int j) -> uint32_t {   // 16-token steps of tile j
+                int32_t t0, valid;
+                tile_of(j, t0, valid);
+                (void)tile_run(valid);
+                return ((uint32_t)(valid + 15) >> 4) + ((kExt && ext.rider_valid > 0 && j == n_tiles - 1) ? 1u : 0u);
             };
 
-            for (uint32_t n = 0; ok && n < my_pairs; ++n) {
+            for (uint32_t n = 0; n < my_pairs; ++n) {
                 const int32_t pair = pair_at(n);
                 const int j_begin = tiles_begin(n), j_end = tiles_end(n);
-                const int ng = stream_of<kWide>(pp, pair, 1).valid ? 2 : 1;
                 const bool shared = pair_is_shared(pp, pair);
-                for (int j = j_begin; ok && j < j_end; ++j) {
-                    int32_t t0, valid;
-                    tile_of(j, t0, valid);
-                    (void)tile_run(valid);
-                    const uint32_t nch = ((uint32_t)(valid + 15) >> 4) +
-                                         ((kExt && ext.rider_valid > 0 && j == n_tiles - 1) ? 1u : 0u);
+                const bool two = shared || (!(kWide && pp.kind == 3) && 2 * (pair - pp.n_shared) + 1 < pp.n_items);   // stream B is there
+                // One S buffer: the pending P V of the previous tile goes first, because this S overwrites its P.  Two buffers: this S
+                // goes first and runs on the tensor pipe while the softmax of the previous tile finishes (streams with
+                // tiles of their own keep the first order: they need their key/value stages back sooner).
+                const bool s_first = C::kSBufs == 2 && (shared || pp.kind == 3);
+                const uint32_t per_tile = shared || !two ? 1u : 2u;
+                uint32_t nch = tile_steps(j_begin);
+                for (int j = j_begin; j < j_end; ++j, sq += per_tile) {
                     const uint32_t idesc_s = make_idesc(kQRows, nch * 16, 0);
 #pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        if (!ok) continue;
-                        if (my_g >= 0 && g != my_g) continue;
-                        if (g >= ng) {
+                    for (int i = 0; i < kStreams; ++i) {
+                        const int g = kStreams == 2 ? i : my_g;
+                        if (g == 1 && !two) {
                             // the stream is absent from this pair: its last P V of the previous pair must not
                             // wait for a next S that is not coming soon (it also holds a key/value stage)
-                            if (pv_live[g]) {
-                                if (!issue_pv(g)) ok = false;
-                                pv_live[g] = false;
-                            }
+                            if (pv_live[i]) issue_pv(i);
+                            pv_live[i] = false;
                             continue;
                         }
                         // S = Q K^T for (stream g, tile j).  Its operands are waited for first: they have
@@ -677,55 +684,38 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         const uint32_t seq = shared ? sq : sq + g;
                         const uint32_t stage = seq % C::kStages, use = seq / C::kStages;
                         if (j == j_begin) {
-                            const uint32_t u = ucount[g];
-                            q_half[g] = q_split ? (u & 1u) : 0u;
-                            const uint32_t parity = q_split ? ((u >> 1) & 1u) : (u & 1u);
-                            if (!warp_wait(q_full0 + 16 * g + 8 * q_half[g], parity, abort_flag)) { ok = false; continue; }
-                            ++ucount[g];
+                            const uint32_t u = ucount[i]++;
+                            q_half[i] = q_split ? (u & 1u) : 0u;
+                            await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u);
                         }
-                        if (!(shared && g == 1 && my_g < 0)) {  // one issuer: the second stream of a shared tile finds it landed
-                            if (!warp_wait(kv_full0 + 8 * stage, use & 1u, abort_flag)) { ok = false; continue; }
-                        }
-                        // One S buffer: the pending P V of the previous tile goes first, because this S
-                        // overwrites its P.  Two buffers: this S goes first and runs on the tensor pipe while
-                        // the softmax of the previous tile finishes (streams with tiles of their own keep the
-                        // first order: they need their key/value stages back sooner).
-                        const bool s_first = C::kSBufs == 2 && (shared || pp.kind == 3);
-                        if (!s_first && pv_live[g] && !issue_pv(g)) { ok = false; continue; }
+                        if (!(shared && i == 1)) await(kv_full0 + 8 * stage, use & 1u);   // one issuer: the second stream of a shared tile finds it landed
+                        if (!s_first && pv_live[i]) issue_pv(i);
                         tc_fence_after();
-                        const uint32_t t_now = tcount[g];
-                        const uint32_t q_lo = q_lo0 + g * kQLo + q_half[g] * (kQHalfSlot >> 4);
-                        const uint32_t k_lo = k_lo0 + stage * kStageLo;
-                        const uint32_t d = tmem + C::kSCol + (g * C::kSBufs + buf_of(t_now)) * kKT;
-                        if (elect_one()) {
-                            umma_ss<false>(d, q_lo, k_lo, kDescHi, idesc_s);
-#pragma unroll
-                            for (int ks = 1; ks < D / 16; ++ks) {
-                                constexpr uint32_t kQH = C::kQHalfBytes >> 4, kKH = C::kKVHalfBytes >> 4;
-                                umma_ss<true>(d, q_lo + (ks >> 2) * kQH + (ks & 3) * 2,
-                                              k_lo + (ks >> 2) * kKH + (ks & 3) * 2, kDescHi, idesc_s);
-                            }
-                            umma_commit(s_full0 + 16 * g + 8 * buf_of(t_now));
-                        }
-                        __syncwarp();
-                        if (s_first && pv_live[g] && !issue_pv(g)) { ok = false; continue; }
-                        pv_live[g] = true;
-                        pv_stage[g] = stage;
-                        pv_nch[g] = nch;
-                        pv_t[g] = t_now;
-                        pv_first[g] = (j == j_begin);
-                        pv_last[g] = (j == j_end - 1);
-                        pv_release[g] = (shared && my_g < 0) ? (g == ng - 1) : true;
-                        pv_twice[g] = !shared;
-                        ++tcount[g];
+                        const uint32_t buf = buf_of(tcount[i]);
+                        umma_s<D, C::kQHalfBytes, C::kKVHalfBytes>(tmem + C::kSCol + (g * C::kSBufs + buf) * kKT,
+                                                                  q_lo0 + g * kQLo + q_half[i] * (kQHalfSlot >> 4), k_lo0 + stage * kStageLo,
+                                                                  kDescHi, idesc_s, s_full0 + 16 * g + 8 * buf);
+                        if (s_first && pv_live[i]) issue_pv(i);
+                        pv_live[i] = true;
+                        pv_stage[i] = stage;
+                        pv_nch[i] = nch;
+                        pv_first[i] = j == j_begin;
+                        pv_last[i] = j == j_end - 1;
+                        pv_release[i] = !(shared && kStreams == 2 && i == 0);
+                        pv_twice[i] = !shared;
+                        ++tcount[i];
                     }
-                    sq += shared ? 1 : ng;
+                    if (j + 1 < j_end) nch = tile_steps(j + 1);
                 }
             }
 #pragma unroll
-            for (int g = 0; g < 2; ++g)
-                if (ok && (my_g < 0 || g == my_g) && pv_live[g] && !issue_pv(g)) ok = false;
-            if (!ok && lane == 0) report(status, kStatusMmaTimeout, abort_flag);
+            for (int i = 0; i < kStreams; ++i)
+                if (pv_live[i]) issue_pv(i);
+            if (__any_sync(0xffffffffu, *abort_flag)) {   // nothing else waits for the last products then: they end before the tensor memory is freed
+                umma_commit_elected(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]));
+                for (uint32_t i = 0; i < kSpinLimit; ++i)
+                    if (mbar_try_wait(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]), 0u)) break;
+            }
         }
     } else if (layout_ok) {
         // ------------------------------------------------------------ softmax + epilogue (warps 0-7)

@@ -68,6 +68,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+__device__ __forceinline__ void report(int* status, int code, volatile int* abort_flag)
+{
+    atomicCAS(status, 0, code);
+    *abort_flag = 1;
+}
+// Bounded wait that does not tell how it ended: one that gives up sets the abort flag, and with the flag set no wait waits.  What
+// follows is the same code either way, so a warp stays on one path.
+__device__ __forceinline__ void wait_through(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
+{
+    if (mbar_try_wait(bar, parity)) return;
+    for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
+        if ((i & 255u) != 0u) continue;
+        if (*abort_flag) break;
+        if (i >= kSpinLimit) {
+            report(status, code, abort_flag);
+            break;
+        }
+    }
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2)
 {
     asm volatile(
@@ -188,6 +208,99 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32
 __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// The same from a converged warp, by one of its lanes.
+__device__ __forceinline__ void umma_commit_elected(uint32_t bar)
+{
+    asm volatile(
+        "{\n"
+        ".reg .pred e;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(bar)
+        : "memory");
+}
+// S = Q K^T of one tile, D channels, and its commit: one predicated block from a converged warp (operands are the same in
+// all lanes), without a branch into the elected lane.
+#define AMSKV_SS_STEP(qo, ko, acc)                                                   \
+    "add.u32 t, %1, " qo ";\n"                                                       \
+    "mov.b64 da, {t, %3};\n"                                                         \
+    "add.u32 t, %2, " ko ";\n"                                                       \
+    "mov.b64 db, {t, %3};\n"                                                         \
+    "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " acc ";\n"
+template <int D, uint32_t kQHalfBytes, uint32_t kKVHalfBytes>
+__device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc, uint32_t bar)
+{
+    static_assert(D == 64 || D == 128, "one or two 128-byte swizzle atoms per row");
+    if (D == 64)
+        asm volatile(
+            "{\n"
+            ".reg .pred e, yes, no;\n"
+            ".reg .b32 t;\n"
+            ".reg .b64 da, db;\n"
+            "elect.sync _|e, 0xffffffff;\n"
+            "setp.eq.u32 yes, 0, 0;\n"
+            "setp.ne.u32 no, 0, 0;\n"
+            AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar)
+            : "memory");
+    else
+        asm volatile(
+            "{\n"
+            ".reg .pred e, yes, no;\n"
+            ".reg .b32 t;\n"
+            ".reg .b64 da, db;\n"
+            "elect.sync _|e, 0xffffffff;\n"
+            "setp.eq.u32 yes, 0, 0;\n"
+            "setp.ne.u32 no, 0, 0;\n"
+            AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
+            AMSKV_SS_STEP("%6", "%7", "yes") AMSKV_SS_STEP("%6 + 2", "%7 + 2", "yes") AMSKV_SS_STEP("%6 + 4", "%7 + 4", "yes")
+            AMSKV_SS_STEP("%6 + 6", "%7 + 6", "yes")
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "n"(kQHalfBytes >> 4), "n"(kKVHalfBytes >> 4)
+            : "memory");
+}
+#undef AMSKV_SS_STEP
+// O (+)= P V of one tile of `steps` 16-token steps, P in tensor memory, and its commits: to
+// `empty` where `release` is set, to `full` where `last` is.
+__device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t desc_hi, uint32_t idesc,
+                                        uint32_t accumulate, uint32_t steps, uint32_t release, uint32_t empty, uint32_t last,
+                                        uint32_t full)
+{
+    asm volatile(
+        "{\n"
+        ".reg .pred e, acc, yes, s1, s2, s3, r, l;\n"
+        ".reg .b32 t, a;\n"
+        ".reg .b64 db;\n"
+        "elect.sync _|e, 0xffffffff;\n"
+        "setp.ne.u32 acc, %5, 0;\n"
+        "setp.eq.u32 yes, 0, 0;\n"
+        "setp.gt.and.u32 s1, %6, 1, e;\n"
+        "setp.gt.and.u32 s2, %6, 2, e;\n"
+        "setp.gt.and.u32 s3, %6, 3, e;\n"
+        "setp.ne.and.u32 r, %7, 0, e;\n"
+        "setp.ne.and.u32 l, %9, 0, e;\n"
+        "mov.b64 db, {%2, %3};\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, acc;\n"
+        "add.u32 t, %2, 128;\n"
+        "add.u32 a, %1, 8;\n"
+        "mov.b64 db, {t, %3};\n"
+        "@s1 tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, yes;\n"
+        "add.u32 t, %2, 256;\n"
+        "add.u32 a, %1, 16;\n"
+        "mov.b64 db, {t, %3};\n"
+        "@s2 tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, yes;\n"
+        "add.u32 t, %2, 384;\n"
+        "add.u32 a, %1, 24;\n"
+        "mov.b64 db, {t, %3};\n"
+        "@s3 tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, yes;\n"
+        "@r tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n"
+        "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%10];\n"
+        "}\n" ::"r"(o_tmem), "r"(p_tmem), "r"(v_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(steps), "r"(release), "r"(empty),
+        "r"(last), "r"(full)
+        : "memory");
 }
 
 #define AMSKV_R32(r, o)                                                                                               \
@@ -344,12 +457,6 @@ constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t make_idesc(uint32_t M, uint32_t N, uint32_t b_mn_major)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major << 16) | ((N >> 3) << 17) | ((M >> 4) << 24);
-}
-
-__device__ __forceinline__ void report(int* status, int code, volatile int* abort_flag)
-{
-    atomicCAS(status, 0, code);
-    *abort_flag = 1;
 }
 
 }  // namespace ptx

@@ -307,21 +307,37 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         }
         fence_async_smem();
     }
-    if (warp == kProducerWarp) {
+    // Everything up to a role's first load touches only this CTA's own memory, so it runs while the kernel before this one
+    // ends: the threads that issue this CTA's loads wait for that kernel right before the first of them, and what the others
+    // read or write follows from those loads.  By then the code up to there, its launch parameters and its tensor maps have
+    // been fetched.  With one wait for all here, a launch issued its first loads 2 000 to 3 800 clocks after it: 60 items, T =
+    // 100, 169 and 256 6.86 / 9.55 / 11.1 -> 6.05 / 8.95 / 10.0 us a call, 256 items, T = 64 and 100 9.05 / 11.6 -> 8.76 / 11.0, 1 920 items, T =
+    // 25 and 36 19.1 / 23.7 -> 17.3 / 22.6, 128 channels, 32 items, T = 144 and 400 8.74 / 16.5 -> 7.8 / 15.7; neutral at large launches.
+    // Tensor memory is owned before the roles split, but in the two-CTA form's long launches (kOwnLate), where the producer
+    // allocates behind its preparations and the other warps meet it there, the softmax warps after the wait: 256 items, T = 169 and
+    // 256 14.8 / 21.3 -> 14.3 / 20.6, 2 304 items, T = 324 223 -> 218, but in the other forms 60 items, T = 100 6.05 -> 6.88 and 256
+    // items, T = 64 8.76 -> 8.95.
+    constexpr bool kOwnLate = !kWide && !kShort;
+    uint32_t tmem = 0;
+    auto allocate = [&]() {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
                      "r"(C::kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    };
+    if (!kOwnLate && warp == kProducerWarp) allocate();
     tc_fence_before();
-    // everything up to here touches only this CTA's own memory, so it runs while the kernel before this one ends
-    wait_for_previous();
     __syncthreads();
-    // The next kernel comes in only now that this CTA owns its tensor memory.  Let in earlier, a CTA of it could take columns
-    // that this one is still waiting for, and keep them while it waits for this launch to end.
-    let_next_start();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+    if (!kOwnLate) tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+    auto own_late = [&]() {   // (once by every warp)
+        if (!kOwnLate) return;
+        if (warp == kProducerWarp) allocate();
+        tc_fence_before();
+        barrier_of(1, C::kThreads);
+        tc_fence_after();
+        tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+    };
     // (in a density launch `valid` also carries the tile's run, or that the tile is a mixed one; tile_run() strips that)
     auto tile_of = [&](int j, int32_t& t0, int32_t& valid) {
         if (j < kTileTab) {
@@ -379,7 +395,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // requested (it has landed by then, so the wait costs nothing), by lane 0, as one bulk group per
         // stage; before a stage is refilled, every group but the two newest has finished reading it.
         const bool storing = kExt && ext.store != 0;
-        if (kShort && lane == 0) {
+        if (lane == 0) {
             prefetch_tensormap(&k_map);
             prefetch_tensormap(&v_map);
             prefetch_tensormap(&k_map64);
@@ -395,6 +411,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 }
             }
         }
+        own_late();
         uint32_t st_sq[2] = {0, 0};
         int32_t st_tok[2] = {0, 0}, st_item[2] = {0, 0};
         int st_n = 0;
@@ -477,6 +494,12 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                     if (!warp_wait(kv_empty0 + 8 * stage, (use & 1u) ^ 1u, abort_flag)) {
                         ok = false;
                         break;
+                    }
+                    if (sq == 0) {
+                        wait_for_previous();
+                        // The next kernel comes in only now that this CTA owns its tensor memory.  Let in earlier, a CTA of it could take
+                        // columns that this one is still waiting for, and keep them while it waits for this launch to end.
+                        let_next_start();
                     }
                     const uint32_t full = kv_full0 + 8 * stage;
                     const uint32_t k_dst = kv_smem + stage * C::kStageBytes, v_dst = k_dst + C::kKVBytes;
@@ -630,6 +653,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             uint32_t ucount[kStreams] = {};   // units started per stream
             uint32_t q_half[kStreams] = {};   // half of the query slot the current unit of each stream uses
             uint32_t sq = 0;
+            bool owned = !kOwnLate;
 
             // O (+)= P V : M = 128, N = D channels, K = 16 * nch tokens; P from TMEM (packed over S),
             // V read MN-major from its stage
@@ -683,7 +707,12 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         // almost always landed, and this keeps the two waits out of the P -> P V -> S chain.
                         const uint32_t seq = shared ? sq : sq + g;
                         const uint32_t stage = seq % C::kStages, use = seq / C::kStages;
+                        if (!owned) {
+                            own_late();
+                            owned = true;
+                        }
                         if (j == j_begin) {
+                            if (tcount[i] == 0) wait_for_previous();   // (the waits that follow have a limit, the launch before has none)
                             const uint32_t u = ucount[i]++;
                             q_half[i] = q_split ? (u & 1u) : 0u;
                             await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u);
@@ -711,19 +740,20 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 #pragma unroll
             for (int i = 0; i < kStreams; ++i)
                 if (pv_live[i]) issue_pv(i);
+            if (!owned) own_late();
             if (__any_sync(0xffffffffu, *abort_flag)) {   // nothing else waits for the last products then: they end before the tensor memory is freed
                 umma_commit_elected(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]));
                 for (uint32_t i = 0; i < kSpinLimit; ++i)
                     if (mbar_try_wait(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]), 0u)) break;
             }
+        } else {
+            own_late();
         }
     } else if (layout_ok) {
         // ------------------------------------------------------------ softmax + epilogue (warps 0-7)
         const int g = warp >> 2, wq = warp & 3;
         const uint32_t lane_base = ((uint32_t)(wq * 32)) << 16;
         const int r = wq * 32 + lane;  // query row inside the tile = TMEM lane
-        const uint32_t s_tmem0 = tmem + C::kSCol + g * C::kSBufs * kKT + lane_base;   // + kKT per S buffer
-        const uint32_t o_tmem = tmem + C::kOCol + g * D + lane_base;
         const uint32_t o_full = o_full0 + 8 * g;
         const bool q_loader = (wq == 0 && lane == 0);
         // the output rows start on 32-byte boundaries (the interface only promises 16)
@@ -735,7 +765,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         uint32_t q_next_n = 0;    // first pair index not yet searched for a query tile
 
         // request the query tile of this stream's next unit not yet requested (first lane of the group only)
-        if (kShort && q_loader) prefetch_tensormap(&q_map);
+        if (q_loader) prefetch_tensormap(&q_map);
         auto load_next_q = [&]() {
             for (; q_next_n < my_pairs; ++q_next_n) {
                 const int32_t pair = pair_at(q_next_n);
@@ -747,6 +777,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 const uint32_t half = q_split ? (q_armed & 1u) : 0u;
                 const uint32_t bar = q_full0 + 16 * g + 8 * half;
                 const uint32_t dst = q_smem + g * C::kQBytes + half * kQHalfSlot;
+                if (q_armed == 0) wait_for_previous();
                 mbar_expect_tx(bar, (uint32_t)qboxes * kQBoxRows * D * 2);
                 int c[4] = {0, 0, 0, 0};
                 c[qpos.y] = head;
@@ -766,6 +797,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             load_next_q();
             if (q_split) load_next_q();
         }
+        __syncwarp();
+        own_late();
+        if (kOwnLate) wait_for_previous();
+        const uint32_t s_tmem0 = tmem + C::kSCol + g * C::kSBufs * kKT + lane_base;   // + kKT per S buffer
+        const uint32_t o_tmem = tmem + C::kOCol + g * D + lane_base;
 
         uint32_t t = 0;   // flat tile counter of this stream
         uint32_t un = 0;  // units done by this stream
@@ -788,7 +824,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 const int run = tile_run(valid);
                 const uint32_t s_tmem = s_tmem0 + buf_of(t) * kKT;
                 const uint32_t s_full = s_full0 + 16 * g + 8 * buf_of(t), p_full = p_full0 + 16 * g + 8 * buf_of(t);
-                if (!__all_sync(0xffffffffu, mbar_wait(s_full, par_of(t), abort_flag))) {
+                // (the first wait may span the end of the launch before; the issuing warp's limit, through the abort flag, ends it too)
+                if (!__all_sync(0xffffffffu, mbar_wait(s_full, par_of(t), abort_flag, !kOwnLate && t == 0 ? ~0u : kSpinLimit))) {
                     report(status, kStatusSyncTimeout, abort_flag);
                     ok = false;
                     break;
@@ -1109,7 +1146,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
-    if (warp == kProducerWarp) {
+    if (warp == kProducerWarp && (layout_ok || !kOwnLate)) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::kTmemCols) : "memory");
     }

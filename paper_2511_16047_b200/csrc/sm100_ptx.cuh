@@ -148,6 +148,13 @@ __device__ __forceinline__ void st_cluster_8B(uint32_t addr, float a, float b)
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
 }
 
+// A named barrier of `threads` threads of the CTA.
+__device__ __forceinline__ void barrier_of(uint32_t id, uint32_t threads)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one()
 {

@@ -522,17 +522,21 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // warp-level matrix instructions, a quarter of the tensor pipe's rate, are what the call takes.  us per call, this kernel / the
 // paired one, append included, in a graph:
 // 64 channels: 19 units, above 32 queries also no more CTAs (of eight warps, two to an SM) than are resident at once: T = 25: 3.6 /
-// 6.8 (60 items), 6.0 / 9.0 (512), 11.1 / 12.4 (1 024, 13.8 units), 19.4 / 17.6 (1 920, 25.9); T = 36: 4.4 / 5.7 (60), 5.9 / 7.9 (240), 9.8 / 8.0
-// (300, the second wave), 12.6 / 8.5 (512); T = 64: 8.2 / 8.5 (240, 13 units), 11.8 / 8.5 (300); T = 81: 7.7 / 8.9 (148), 12.4 / 11.1 (180).
-// Above 81 queries 7 units where the paired kernel has an SM for every query tile, because of calls behind a separate append
-// (fused, and append and attention apart: T = 100: 5.9 / 6.7 and 9.2 / 8.7 (60, 8.5 units), 7.7 / 7.4 and 9.8 / 9.8 (96, 13.6); T = 121:
-// 7.0 / 8.0 and 10.8 / 9.3 (60, 13.0); T = 169: 7.9 / 8.1 and 9.3 / 9.8 (32, 11.9), 10.5 / 9.1 and 12.2 / 11.1 (60, 22.3)).  An append of several
-// copies (`copies`), which is never apart and which the paired kernel writes partly row by row, keeps the 19: T = 100: 8.4 / 8.8 (120, 17 units), 9.0 / 9.3 (148,
+// 5.9 (60 items), 6.1 / 8.6 (512), 11.1 / 12.4 (1 024, 13.8 units), 19.4 / 17.6 (1 920, 25.9); T = 36: 4.4 / 4.7 (60), 5.9 / 7.0 (256), 9.5 / 8.0
+// (300, the second wave); T = 49: 4.4 / 4.9 (60), 7.0 / 7.5 (256), 11.1 / 8.3 (300); T = 64: 4.7 / 4.7 (60), 5.5 / 6.7 (148).  An append fused
+// into the paired kernel takes 10 units above 49 queries (T = 64: 7.5 / 7.2 (200, 10.8 units), 8.3 / 7.6 (256); behind a separate
+// append 9.1 / 9.9 and 9.8 / 10.7), and every call above 64 where it has an SM for every query tile (T = 81: 5.4 / 4.9 (8), 5.9 /
+// 5.2 (60), 7.7 / 7.4 (148); T = 100: 5.4 / 5.2 (8), 6.0 / 5.4 (60), 8.8 / 7.8 (148); T = 169: 6.8 / 6.7 (8), 8.0 / 7.0 (32)).  Apart from the append this
+// kernel keeps 7 units there (T = 81: 6.4 / 7.2 (32, 3.9 units), 8.2 / 7.2 (60, 7.3); T = 100: 7.0 / 7.5 (32), 9.0 / 7.6 (60, 8.5); T = 121: 7.7 /
+// 8.0 (32, 6.9), 10.6 / 8.5 (60); T = 169: 7.7 / 8.5 (16, 5.9), 9.0 / 8.7 (32, 11.9)).  An append of several copies (`copies`), which is
+// never apart and which the paired kernel writes partly row by row, keeps the 19: T = 100: 8.4 / 8.8 (120, 17 units), 9.0 / 9.3 (148,
 // 21); T = 121: 7.4 / 8.5 (60, 13), 9.9 / 9.6 (96, 20.8); T = 169: 8.8 / 9.3 (96, 21.4), 13.9 / 9.5 (120, 26.8).
-// 128 channels: 6 units: T = 25: 4.7 / 7.3 (60), 12.6 / 13.5 (512, 6.9 units), 17.4 / 16.2 (700); T = 36: 5.7 / 6.2 (60), 7.0 / 7.8 (148, 6.0),
-// 11.9 / 9.3 (180); T = 64: 6.0 / 6.4 (60), 7.5 / 7.5 (96, 5.2), 8.7 / 8.5 (148); none above 64 queries where the paired kernel has an SM
-// for every tile (T = 81: 7.0 / 7.0 (8), 7.1 / 7.2 (32), 8.6 / 8.0 (60); T = 100: 7.2 / 6.5 (8)) but for several copies (T = 100: 7.6 / 8.0 (32,
-// 4.5), 9.6 / 8.5 (60, 8.5); T = 169: 7.5 / 8.0 (8, 3.0), 9.2 / 8.5 (32, 7.1)).
+// 128 channels: 6 units: T = 25: 4.7 / 6.8 (60), 12.6 / 12.8 (512, 6.9 units), 17.4 / 16.2 (700); T = 36 apart from the append: 6.8 / 7.5 (32),
+// 8.2 / 8.2 (96), 8.3 / 9.3 (148), 12.6 / 10.8 (200).  Fused, above 32 queries, only where the paired kernel's tiles take more than two
+// thirds of the SMs, which leaves the next launch's no room (T = 36: 5.6 / 4.8 (8), 5.7 / 5.2 (60), 6.4 / 6.3 (96), 6.9 / 7.8 (148, 6.0 units); T = 49:
+// 5.5 / 5.4 (60), 7.1 / 7.2 (120); T = 64: 5.9 / 4.9 (8), 6.0 / 5.4 (60), 8.7 / 8.2 (148, 8.0)).  None above 64 queries where the paired
+// kernel has an SM for every tile (T = 81: 7.3 / 5.7 (8), 8.5 / 6.1 (60); T = 100: 7.2 / 5.9 (8)) but for several copies (T = 100: 7.6 / 8.0
+// (32, 4.5), 9.6 / 8.5 (60, 8.5); T = 169: 7.5 / 8.0 (8, 3.0), 9.2 / 8.5 (32, 7.1)).
 // With the density 20 and 7 units (times with the append and the zeroed result): T = 25: 18.2 / 18.7
 // (1 024 items), 27.8 / 29.3 (1 920, 25.9 units); T = 36: 10.4 / 12.4 (240), 15.0 / 13.1 (300); T = 64: 12.3 / 15.1 (240), 18.2 / 16.7 (300); T = 81:
 // 12.6 / 16.2 (148, 18 units), 18.0 / 16.9 (180); 128 channels: T = 25: 18.2 / 20.1 (512, 6.9 units), 23.6 / 25.3 (700), 49 / 49 (1 920); T = 36: 11.6 /
@@ -544,7 +548,7 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // 3 840 53.5 / 18.9) and five for four (700 items 15.9 / 16.3, 1 024 19.8 / 17.7, 3 840 58 / 37).  With more keys the alternative is the
 // paired kernel's one launch (T = 16, 916 keys: 400 items 28.9 / 41.0, 3 840 items 225 / 240; 128 channels 340 / 344).
 // Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).
-bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies)
+bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool fused, bool copies)
 {
     if (density && T <= kSmallMaxQueries) {
         if (!small_supported(T, total_keys) || (T > 1 && D == 64) || T > 4) return true;
@@ -554,7 +558,10 @@ bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int 
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
     int line = D == 64 ? 19 : 6;
     if (density) line = D == 64 ? 20 : 7;
-    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? (T > 81 ? 7 : 19) : (T > 64 ? 0 : 6);
+    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) {
+        if (T > 64) line = D == 64 && !fused ? 7 : 0;
+        else if (D == 128 && T > 32 && fused && 3 * items <= 2 * sm_count) line = 0;
+    } else if (!copies && D == 64 && fused && T > 49) line = 10;
     const bool one_wave = D == 128 || T <= 32 || items * ((T + 63) / 64) <= 2 * (int64_t)sm_count;   // (of CTAs of 64 queries)
     return units <= (int64_t)sm_count * line && one_wave;
 }

@@ -295,3 +295,21 @@ def test_an_item_does_not_depend_on_the_values_of_others_nor_beyond_rounding_on_
                 assert (x - y).norm() <= 5e-3 * x.norm()
             else:
                 assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("D,side,items", [(64, 8, (184, 186)), (64, 9, (148, 150)), (128, 6, (98, 100)), (128, 8, (98, 100))])
+def test_lines_between_the_kernels_of_fused_and_separate_appends(D, side, items):
+    """T = 64 at ten units of the warp-matrix kernel per SM (185 items of 4 x 2 blocks are 1 480), T = 81 with and without an SM for
+    every query tile, T = 36 and 64 of 128 channels at two thirds of the SMs (98): fused and separate appends choose apart."""
+    sides = (5, side)
+    for n in items:
+        rows, heads = n // 2, 2
+        qkv = make_qkv(rows, heads, sides, D, seed=108)
+        pick = [0, n // 2, n - 1]
+        want = oracle_outputs(qkv, (1, 2, False), 1.0 / math.sqrt(D), items=pick)
+        for fused in (False, True):
+            with Cache(1, heads, D, rows, sides, [(1, 2, False)]) as c:
+                outs = run_pass(c, qkv, fused=fused)
+                for k in range(2):
+                    got = outs[0][k].reshape(n, -1, D)[pick].cpu().double()
+                    check_close(got, want[k], "%d items scale %d" % (n, k))

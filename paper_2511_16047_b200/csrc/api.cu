@@ -193,14 +193,13 @@ void note_appended(amskv_cache* cache, int layer, int scale)
 
 // which kernel amskv_attend uses for T query tokens over `total` keys
 enum class AttendKernel { Small, Mid, Simt, Pair, Tensor };
-// (fused: the kernel takes the scale from the caller's tensors; copies: and appends it, as more than one contiguous copy; see
-// mid_preferred)
-AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool fused = false, bool copies = false)
+// (copies: the call includes an append that is not one contiguous copy; see mid_preferred)
+AttendKernel choose_kernel(const amskv_cache* cache, int32_t T, int32_t total, bool density = false, bool copies = false)
 {
     // few items or few queries: the warp-matrix kernel (attend_mid.cu, where the line is explained); for a single query token,
     // which is the CUDA-core kernel's with its fp32 probabilities, only where its one key makes the output a copy of V
     if (cache->path == AMSKV_PATH_AUTO && (T > 1 || (density && total == 1)) && cache->tc_ready &&
-        mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density, fused, copies))
+        mid_preferred(T, total, cache->items(), cache->head_dim, cache->sm_count, density, copies))
         return AttendKernel::Mid;
     // AUTO: the warp-per-item kernel wherever a scale's retained keys fit its register tile, the paired
     // tcgen05 kernel elsewhere (the CUDA-core kernel only where tensor maps are unavailable)
@@ -445,7 +444,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
         for (int i = 0; i < rl.n; ++i) rl.total += rl.r[i].len;
         CurrentScaleSource src{ks, vs, false, 0, cache->region(layer)};
         cudaError_t e;
-        if (choose_kernel(cache, T, rl.total, false, true) == AttendKernel::Mid) {
+        if (choose_kernel(cache, T, rl.total) == AttendKernel::Mid) {
             --rl.n;   // the kernel takes the scale itself from `src`
             rl.total -= T;
             e = launch_attend_mid(q, o, cache->region(layer), rl, T, cache->rows, cache->heads, cache->head_dim,
@@ -472,7 +471,7 @@ int amskv_append_attend(amskv_cache* cache, int layer, int scale, const void* K,
     Piece piece[LayerLayout::kMaxPieces];
     const int32_t n_pieces = lay.pieces(cache->tokens, scale, piece);
     const bool one_copy = n_pieces == 1 && piece[0].src == 0 && piece[0].len == T;
-    AttendKernel kernel = choose_kernel(cache, T, after.total, false, true, !one_copy);
+    AttendKernel kernel = choose_kernel(cache, T, after.total, false, !one_copy);
     // a single-token scale that is its own only key (the first scale): out = V, one copy kernel does both calls
     if (cache->path == AMSKV_PATH_AUTO && T == 1 && after.total == 1) kernel = AttendKernel::Small;
     if (kernel == AttendKernel::Small && one_copy) {

@@ -517,26 +517,32 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 
 }  // namespace
 
-// Where this kernel is the faster one, in units of work (16 queries x 64 keys of one item) per SM.  Below the lines the paired
-// kernel costs 5 to 9 us whatever the size (and the copy before it, where the append is not fused into that); above them the
-// warp-level matrix instructions, a quarter of the tensor pipe's rate, are what the call takes.  us per call, this kernel / the
-// paired one, append included, in a graph:
-// 64 channels: 19 units, above 32 queries also no more CTAs (of eight warps, two to an SM) than are resident at once: T = 25: 3.6 /
-// 5.9 (60 items), 6.1 / 8.6 (512), 11.1 / 12.4 (1 024, 13.8 units), 19.4 / 17.6 (1 920, 25.9); T = 36: 4.4 / 4.7 (60), 5.9 / 7.0 (256), 9.5 / 8.0
-// (300, the second wave); T = 49: 4.4 / 4.9 (60), 7.0 / 7.5 (256), 11.1 / 8.3 (300); T = 64: 4.7 / 4.7 (60), 5.5 / 6.7 (148).  An append fused
-// into the paired kernel takes 10 units above 49 queries (T = 64: 7.5 / 7.2 (200, 10.8 units), 8.3 / 7.6 (256); behind a separate
-// append 9.1 / 9.9 and 9.8 / 10.7), and every call above 64 where it has an SM for every query tile (T = 81: 5.4 / 4.9 (8), 5.9 /
-// 5.2 (60), 7.7 / 7.4 (148); T = 100: 5.4 / 5.2 (8), 6.0 / 5.4 (60), 8.8 / 7.8 (148); T = 169: 6.8 / 6.7 (8), 8.0 / 7.0 (32)).  Apart from the append this
-// kernel keeps 7 units there (T = 81: 6.4 / 7.2 (32, 3.9 units), 8.2 / 7.2 (60, 7.3); T = 100: 7.0 / 7.5 (32), 9.0 / 7.6 (60, 8.5); T = 121: 7.7 /
-// 8.0 (32, 6.9), 10.6 / 8.5 (60); T = 169: 7.7 / 8.5 (16, 5.9), 9.0 / 8.7 (32, 11.9)).  An append of several copies (`copies`), which is
-// never apart and which the paired kernel writes partly row by row, keeps the 19: T = 100: 8.4 / 8.8 (120, 17 units), 9.0 / 9.3 (148,
-// 21); T = 121: 7.4 / 8.5 (60, 13), 9.9 / 9.6 (96, 20.8); T = 169: 8.8 / 9.3 (96, 21.4), 13.9 / 9.5 (120, 26.8).
-// 128 channels: 6 units: T = 25: 4.7 / 6.8 (60), 12.6 / 12.8 (512, 6.9 units), 17.4 / 16.2 (700); T = 36 apart from the append: 6.8 / 7.5 (32),
-// 8.2 / 8.2 (96), 8.3 / 9.3 (148), 12.6 / 10.8 (200).  Fused, above 32 queries, only where the paired kernel's tiles take more than two
-// thirds of the SMs, which leaves the next launch's no room (T = 36: 5.6 / 4.8 (8), 5.7 / 5.2 (60), 6.4 / 6.3 (96), 6.9 / 7.8 (148, 6.0 units); T = 49:
-// 5.5 / 5.4 (60), 7.1 / 7.2 (120); T = 64: 5.9 / 4.9 (8), 6.0 / 5.4 (60), 8.7 / 8.2 (148, 8.0)).  None above 64 queries where the paired
-// kernel has an SM for every tile (T = 81: 7.3 / 5.7 (8), 8.5 / 6.1 (60); T = 100: 7.2 / 5.9 (8)) but for several copies (T = 100: 7.6 / 8.0
-// (32, 4.5), 9.6 / 8.5 (60, 8.5); T = 169: 7.5 / 8.0 (8, 3.0), 9.2 / 8.5 (32, 7.1)).
+// Where this kernel serves a call, in units of work (16 queries x 64 keys of one item) per SM.  Below the lines the paired kernel
+// costs 5 to 9 us whatever the size (and the copy before it, where the append is not fused into that); above them the warp-level
+// matrix instructions, a quarter of the tensor pipe's rate, are what the call takes.
+//   64 channels   19 units; above 32 queries no more CTAs (of eight warps, two to an SM) than are resident at once; 7 units above 81
+//                 queries where the paired kernel has an SM for every query tile, 19 there too for an append of several copies
+//   128 channels  6 units; none above 64 queries where the paired kernel has an SM for every tile, but for several copies
+// us per call, this kernel / the paired one, in a graph, append included: f fused, s a call of its own, c of several copies.
+//     T   64 channels                                                 128 channels
+//    25   f 60 items 3.6 / 5.9, 512 6.1 / 8.6, 1 024 (13.8 units)     f 60 4.7 / 6.8, 512 (6.9 units) 12.6 / 12.8, 700 17.4 / 16.2
+//         11.1 / 12.4, 1 920 (25.9) 19.4 / 17.6
+//    36   f 60 4.4 / 4.7, 256 5.9 / 7.0, 300 (second wave) 9.5 / 8.0  f 8 5.6 / 4.8, 60 5.7 / 5.2, 96 6.4 / 6.3, 148 (6.0) 6.9 / 7.8
+//                                                                     s 32 6.8 / 7.5, 96 8.2 / 8.2, 148 8.3 / 9.3, 200 12.6 / 10.8
+//    49   f 60 4.4 / 4.9, 256 7.0 / 7.5, 300 11.1 / 8.3               f 60 5.5 / 5.4, 120 7.1 / 7.2
+//    64   f 60 4.7 / 4.7, 148 5.5 / 6.7, 200 (10.8) 7.5 / 7.2,        f 8 5.9 / 4.9, 60 6.0 / 5.4, 148 (8.0) 8.7 / 8.2
+//         256 8.3 / 7.6; s 200 9.1 / 9.9, 256 9.8 / 10.7
+//    81   f 8 5.4 / 4.9, 60 5.9 / 5.2, 148 7.7 / 7.4;                 f 8 7.3 / 5.7, 60 8.5 / 6.1
+//         s 32 (3.9) 6.4 / 7.2, 60 (7.3) 8.2 / 7.2
+//   100   f 8 5.4 / 5.2, 60 (8.5) 6.0 / 5.4, 148 8.8 / 7.8;           f 8 7.2 / 5.9; c 32 (4.5) 7.6 / 8.0, 60 (8.5) 9.6 / 8.5
+//         s 32 7.0 / 7.5, 60 9.0 / 7.6; c 120 (17) 8.4 / 8.8, 148 (21) 9.0 / 9.3
+//   121   s 32 (6.9) 7.7 / 8.0, 60 10.6 / 8.5; c 60 (13) 7.4 / 8.5, 96 (20.8) 9.9 / 9.6
+//   169   f 8 6.8 / 6.7, 32 8.0 / 7.0; s 16 (5.9) 7.7 / 8.5,          c 8 (3.0) 7.5 / 8.0, 32 (7.1) 9.2 / 8.5
+//         32 (11.9) 9.0 / 8.7; c 96 (21.4) 8.8 / 9.3, 120 (26.8) 13.9 / 9.5
+// The lines were drawn when the paired kernel took 0.5 to 1.5 us more behind another launch than it does in this table.  Fused
+// appends by which it would now win below them (by up to 17 %) stay here all the same: they keep this kernel's weights (every
+// exponential from the special-function unit, the reference a maximum over 32 keys of each half, where the paired kernel's may be
+// that of a tile of 21), and fused and separate calls choose alike.
 // With the density 20 and 7 units (times with the append and the zeroed result): T = 25: 18.2 / 18.7
 // (1 024 items), 27.8 / 29.3 (1 920, 25.9 units); T = 36: 10.4 / 12.4 (240), 15.0 / 13.1 (300); T = 64: 12.3 / 15.1 (240), 18.2 / 16.7 (300); T = 81:
 // 12.6 / 16.2 (148, 18 units), 18.0 / 16.9 (180); 128 channels: T = 25: 18.2 / 20.1 (512, 6.9 units), 23.6 / 25.3 (700), 49 / 49 (1 920); T = 36: 11.6 /
@@ -548,7 +554,7 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // 3 840 53.5 / 18.9) and five for four (700 items 15.9 / 16.3, 1 024 19.8 / 17.7, 3 840 58 / 37).  With more keys the alternative is the
 // paired kernel's one launch (T = 16, 916 keys: 400 items 28.9 / 41.0, 3 840 items 225 / 240; 128 channels 340 / 344).
 // Without the density the warp-per-item kernel keeps its scales (T = 9: 2.6 / 3.5).
-bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool fused, bool copies)
+bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies)
 {
     if (density && T <= kSmallMaxQueries) {
         if (!small_supported(T, total_keys) || (T > 1 && D == 64) || T > 4) return true;
@@ -558,10 +564,7 @@ bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int 
     const int64_t units = items * ((T + 15) / 16) * (((int64_t)total_keys + kChunk - 1) / kChunk);
     int line = D == 64 ? 19 : 6;
     if (density) line = D == 64 ? 20 : 7;
-    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) {
-        if (T > 64) line = D == 64 && !fused ? 7 : 0;
-        else if (D == 128 && T > 32 && fused && 3 * items <= 2 * sm_count) line = 0;
-    } else if (!copies && D == 64 && fused && T > 49) line = 10;
+    else if (!copies && pair_one_tile_per_sm(items, T, sm_count)) line = D == 64 ? (T > 81 ? 7 : 19) : (T > 64 ? 0 : 6);
     const bool one_wave = D == 128 || T <= 32 || items * ((T + 63) / 64) <= 2 * (int64_t)sm_count;   // (of CTAs of 64 queries)
     return units <= (int64_t)sm_count * line && one_wave;
 }

@@ -134,7 +134,7 @@ cudaError_t launch_attend_small(const Strided& Q, const Strided& O, const LayerR
 // instructions.  With `cur`, `ranges` lists the cached keys only and the current scale's tokens come from the caller's
 // tensors; `piece` says where they go in the region (n_pieces = 0: nowhere).  With `density` (then without `cur`) an entry
 // of `ranges` belongs to one run, as for the paired kernel.
-bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool fused, bool copies);
+bool mid_preferred(int32_t T, int32_t total_keys, int64_t items, int32_t D, int sm_count, bool density, bool copies);
 cudaError_t launch_attend_mid(const Strided& Q, const Strided& O, const LayerRegion& region, const RangeList& ranges, int32_t T,
                               int32_t rows, int32_t heads, int32_t D, float softmax_scale, int sm_count, cudaStream_t stream,
                               const CurrentScaleSource* cur = nullptr, const Piece* piece = nullptr, int32_t n_pieces = 0,

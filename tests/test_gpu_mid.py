@@ -299,8 +299,8 @@ def test_an_item_does_not_depend_on_the_values_of_others_nor_beyond_rounding_on_
 
 @pytest.mark.parametrize("D,side,items", [(64, 8, (184, 186)), (64, 9, (148, 150)), (128, 6, (98, 100)), (128, 8, (98, 100))])
 def test_lines_between_the_kernels_of_fused_and_separate_appends(D, side, items):
-    """T = 64 at ten units of the warp-matrix kernel per SM (185 items of 4 x 2 blocks are 1 480), T = 81 with and without an SM for
-    every query tile, T = 36 and 64 of 128 channels at two thirds of the SMs (98): fused and separate appends choose apart."""
+    """T = 64 of 185 items, T = 81 with and without an SM for every query tile, T = 36 and 64 of 128 channels at two thirds of the SMs:
+    the outputs of fused and of separate appends, whatever kernel serves them, against the oracle."""
     sides = (5, side)
     for n in items:
         rows, heads = n // 2, 2
@@ -313,3 +313,18 @@ def test_lines_between_the_kernels_of_fused_and_separate_appends(D, side, items)
                 for k in range(2):
                     got = outs[0][k].reshape(n, -1, D)[pick].cpu().double()
                     check_close(got, want[k], "%d items scale %d" % (n, k))
+
+
+@pytest.mark.parametrize("D,side,share", [(64, 8, 240 / 148), (64, 9, 100 / 148), (64, 10, 60 / 148), (128, 6, 60 / 148), (128, 8, 60 / 148)])
+def test_fused_and_separate_appends_choose_the_same_kernel(D, side, share):
+    """T = 64, 81, 100 and, 128 channels, 36 and 64, at item counts (per SM) that the lines of the warp-matrix kernel leave to it whether
+    or not the append is fused: its packed key sequence is then the same, so the outputs are, bit for bit.  (The paired kernel's,
+    asked for by its path, are not.)"""
+    items = int(torch.cuda.get_device_properties(0).multi_processor_count * share)
+    qkv = make_qkv(items, 1, (5, side), D, seed=108, peaked=True)
+    outs = []
+    with Cache(1, 1, D, items, (5, side), [(1, 2, False)]) as c:
+        for path, fused in ((B.PATH_AUTO, False), (B.PATH_AUTO, True), (B.PATH_TENSOR_PAIR, True)):
+            outs.append(run_pass(c, qkv, path, fused=fused)[0][1])
+    assert torch.equal(outs[0], outs[1])
+    assert not torch.equal(outs[1], outs[2])

@@ -25,8 +25,9 @@
 // stands, and only a row whose tile sum leaves the range (beyond 2^64, or not a number) makes
 // its warp take the true maxima, rescale and form the tile again.  The first lane of each group fetches its
 // next query tile as soon as the last S of the current one has landed.
-// Every wait is bounded: a wait that gives up records a status code, all roles wind down,
-// copies in flight are awaited and the tensor memory is freed.
+// Every wait is bounded: a wait that gives up records a status code and sets a flag; no role issues another load, product,
+// commit or store on what that wait was for, so all of them stop, and then the copies and products still
+// under way are awaited and the tensor memory is freed.
 #include <algorithm>
 #include <type_traits>
 
@@ -113,6 +114,7 @@ struct Barriers {
     uint64_t s_full[2][2], p_full[2][2];   // [stream][S buffer]
     uint64_t o_full[2], pv_done[2], drained[2];
     uint32_t tmem_base;
+    uint32_t issued;           // stages the producer has filled, for the end of a launch that gave up
     int abort_flag;
     int2 tile_tab[kTileTab];
 };
@@ -612,15 +614,9 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
             __syncwarp();
         }
-        if (!ok) {
-            if (lane == 0) report(status, kStatusTmaTimeout, abort_flag);
-            // wind down: let the copies that were issued land before the CTA gives its shared memory back
-            const uint32_t first = sq > (uint32_t)C::kStages ? sq - C::kStages : 0u;
-            for (uint32_t q = first; q < sq; ++q) {
-                const uint32_t stage = q % C::kStages, use = q / C::kStages;
-                for (uint32_t i = 0; i < kSpinLimit; ++i)
-                    if (mbar_try_wait(kv_full0 + 8 * stage, use & 1u)) break;
-            }
+        if (lane == 0) {
+            if (!ok) report(status, kStatusTmaTimeout, abort_flag);
+            bars->issued = sq;
         }
     } else if (layout_ok && warp >= kMmaWarp) {
         // ------------------------------------------------------------ MMA issuer(s)
@@ -631,20 +627,22 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         //
         // A warp's own instructions are what a tile costs here: a satisfied wait of a voting warp 220 clocks, a branch into the
         // elected lane and back 130, the bookkeeping of a tile 500, against 320 (64 channels) and 640 clocks of products.  So a
-        // wait that gives up does not change the course (it sets the abort flag, after which no wait waits), a product's
+        // wait that gives up does not change the course (the lane's `go` ends, and with it what it issues), a product's
         // instructions and commits are one predicated block, and a tile's length is fetched a tile ahead.  Eight images, T = 4 096,
         // 128 channels: 4 836 -> 4 717 us a call at the same power; one image, T = 576 and 1 600: 35.7 -> 31.5 and 98.3 -> 93.4; 64
         // channels, 256 items, T = 64 and 100: 9.35 -> 9.05 and 11.9 -> 11.6, and no change where the softmax warps fill the SM.
         const int my_g = C::kMmaWarps == 2 ? warp - kMmaWarp : 0;
         if (my_pairs > 0) {
             constexpr int kStreams = C::kMmaWarps == 2 ? 1 : 2;   // streams this warp issues for
-            
             const uint32_t idesc_pv = make_idesc(kQRows, D, 1);
             const uint32_t k_lo0 = desc_lo(kv_smem, 16);                             // K tile of stage 0, K-major
             const uint32_t v_lo0 = desc_lo(kv_smem + C::kKVBytes, C::kKVHalfBytes);  // V tile of stage 0, MN-major
             const uint32_t q_lo0 = desc_lo(q_smem, 16);
             constexpr uint32_t kStageLo = C::kStageBytes >> 4, kQLo = C::kQBytes >> 4;
-            auto await = [&](const uint32_t bar, const uint32_t parity) { wait_through(bar, parity, status, kStatusMmaTimeout, abort_flag); };
+            bool go = true;   // no wait of this lane has given up
+            auto await = [&](const uint32_t bar, const uint32_t parity) {
+                if (go) go = wait_through(bar, parity, status, kStatusMmaTimeout, abort_flag);
+            };
             // per stream: the tile whose S was issued last and whose P V is still to be issued
             uint32_t pv_stage[kStreams] = {}, pv_nch[kStreams] = {}, pv_first[kStreams] = {}, pv_last[kStreams] = {},
                      pv_release[kStreams] = {}, pv_twice[kStreams] = {};
@@ -666,11 +664,11 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 tc_fence_after();
                 const uint32_t empty = kv_empty0 + 8 * pv_stage[i];
                 umma_pv(tmem + C::kOCol + g * D, tmem + C::kSCol + (g * C::kSBufs + buf_of(t)) * kKT,
-                             v_lo0 + pv_stage[i] * kStageLo, kDescHi, idesc_pv, pv_first[i] ^ 1u, pv_nch[i], pv_release[i], empty,
-                             pv_last[i], o_full0 + 8 * g);
+                        v_lo0 + pv_stage[i] * kStageLo, kDescHi, idesc_pv, pv_first[i] ^ 1u, pv_nch[i], pv_release[i], empty,
+                        pv_last[i], o_full0 + 8 * g, go);
                 if (C::kMmaWarps == 2) {
-                    if (pv_twice[i]) umma_commit_elected(empty);
-                    umma_commit_elected(pv_done0 + 8 * g);   // read by the (rare) rescale of O only
+                    if (pv_twice[i]) umma_commit_elected(empty, go);
+                    umma_commit_elected(pv_done0 + 8 * g, go);   // read by the (rare) rescale of O only
                 }
             };
             auto tile_steps = [&](const int j) -> uint32_t {   // 16-token steps of tile j
@@ -723,7 +721,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         const uint32_t buf = buf_of(tcount[i]);
                         umma_s<D, C::kQHalfBytes, C::kKVHalfBytes>(tmem + C::kSCol + (g * C::kSBufs + buf) * kKT,
                                                                   q_lo0 + g * kQLo + q_half[i] * (kQHalfSlot >> 4), k_lo0 + stage * kStageLo,
-                                                                  kDescHi, idesc_s, s_full0 + 16 * g + 8 * buf);
+                                                                  kDescHi, idesc_s, s_full0 + 16 * g + 8 * buf, go);
                         if (s_first && pv_live[i]) issue_pv(i);
                         pv_live[i] = true;
                         pv_stage[i] = stage;
@@ -741,11 +739,6 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             for (int i = 0; i < kStreams; ++i)
                 if (pv_live[i]) issue_pv(i);
             if (!owned) own_late();
-            if (__any_sync(0xffffffffu, *abort_flag)) {   // nothing else waits for the last products then: they end before the tensor memory is freed
-                umma_commit_elected(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]));
-                for (uint32_t i = 0; i < kSpinLimit; ++i)
-                    if (mbar_try_wait(smem_u32(&bars->drained[C::kMmaWarps == 2 ? my_g : 0]), 0u)) break;
-            }
         } else {
             own_late();
         }
@@ -1146,6 +1139,24 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
+    if (layout_ok && *abort_flag) {   // (the same for all threads: no role is left to set it)
+        // A launch that gave up.  Nothing issues any more; what nobody may have waited for, the newest copy into each stage and
+        // the products, ends before shared and tensor memory are given back (query tiles: at the end of the softmax role).
+        auto until = [](const uint32_t bar, const uint32_t parity) {
+            for (uint32_t i = 0; i < kSpinLimit; ++i)
+                if (mbar_try_wait(bar, parity)) break;
+        };
+        if (warp == kProducerWarp) {
+            const uint32_t issued = bars->issued;
+            for (uint32_t q = issued > (uint32_t)C::kStages ? issued - C::kStages : 0u; q < issued; ++q)
+                until(kv_full0 + 8 * (q % C::kStages), (q / C::kStages) & 1u);
+        } else if (warp >= kMmaWarp) {
+            const uint32_t drained = smem_u32(&bars->drained[warp - kMmaWarp]);
+            umma_commit_elected(drained, true);
+            until(drained, 0u);
+        }
+        __syncthreads();
+    }
     if (warp == kProducerWarp && (layout_ok || !kOwnLate)) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::kTmemCols) : "memory");

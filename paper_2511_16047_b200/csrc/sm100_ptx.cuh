@@ -73,19 +73,20 @@ __device__ __forceinline__ void report(int* status, int code, volatile int* abor
     atomicCAS(status, 0, code);
     *abort_flag = 1;
 }
-// Bounded wait that does not tell how it ended: one that gives up sets the abort flag, and with the flag set no wait waits.  What
-// follows is the same code either way, so a warp stays on one path.
-__device__ __forceinline__ void wait_through(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
+// Bounded wait of a warp that stays on one path: what follows is the same code however it ended.  False in a lane that gave up
+// (it sets the abort flag) or saw the flag set; the blocks below then issue nothing (`go`).
+__device__ __forceinline__ bool wait_through(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
 {
-    if (mbar_try_wait(bar, parity)) return;
+    if (mbar_try_wait(bar, parity)) return true;
     for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
         if ((i & 255u) != 0u) continue;
-        if (*abort_flag) break;
+        if (*abort_flag) return false;
         if (i >= kSpinLimit) {
             report(status, code, abort_flag);
-            break;
+            return false;
         }
     }
+    return true;
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2)
@@ -184,15 +185,17 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// The same from a converged warp, by one of its lanes.
-__device__ __forceinline__ void umma_commit_elected(uint32_t bar)
+// The blocks below are issued from a converged warp by one of its lanes, always the same one, and only if that lane's `go` is set:
+// its own waits have all ended well, so what it issues reads data that has landed.
+__device__ __forceinline__ void umma_commit_elected(uint32_t bar, bool go)
 {
     asm volatile(
         "{\n"
         ".reg .pred e;\n"
         "elect.sync _|e, 0xffffffff;\n"
+        "setp.ne.and.u32 e, %1, 0, e;\n"
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-        "}\n" ::"r"(bar)
+        "}\n" ::"r"(bar), "r"((uint32_t)go)
         : "memory");
 }
 // Shared-memory matrix descriptors are passed as two 32-bit halves: the low half carries the
@@ -206,7 +209,8 @@ __device__ __forceinline__ void umma_commit_elected(uint32_t bar)
     "mov.b64 db, {t, %3};\n"                                                         \
     "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " acc ";\n"
 template <int D, uint32_t kQHalfBytes, uint32_t kKVHalfBytes>
-__device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc, uint32_t bar)
+__device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc, uint32_t bar,
+                                       bool go)
 {
     static_assert(D == 64 || D == 128, "one or two 128-byte swizzle atoms per row");
     if (D == 64)
@@ -216,11 +220,12 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
             ".reg .b32 t;\n"
             ".reg .b64 da, db;\n"
             "elect.sync _|e, 0xffffffff;\n"
+            "setp.ne.and.u32 e, %6, 0, e;\n"
             "setp.eq.u32 yes, 0, 0;\n"
             "setp.ne.u32 no, 0, 0;\n"
             AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
             "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
-            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar)
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "r"((uint32_t)go)
             : "memory");
     else
         asm volatile(
@@ -229,13 +234,15 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
             ".reg .b32 t;\n"
             ".reg .b64 da, db;\n"
             "elect.sync _|e, 0xffffffff;\n"
+            "setp.ne.and.u32 e, %6, 0, e;\n"
             "setp.eq.u32 yes, 0, 0;\n"
             "setp.ne.u32 no, 0, 0;\n"
             AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
-            AMSKV_SS_STEP("%6", "%7", "yes") AMSKV_SS_STEP("%6 + 2", "%7 + 2", "yes") AMSKV_SS_STEP("%6 + 4", "%7 + 4", "yes")
-            AMSKV_SS_STEP("%6 + 6", "%7 + 6", "yes")
+            AMSKV_SS_STEP("%7", "%8", "yes") AMSKV_SS_STEP("%7 + 2", "%8 + 2", "yes") AMSKV_SS_STEP("%7 + 4", "%8 + 4", "yes")
+            AMSKV_SS_STEP("%7 + 6", "%8 + 6", "yes")
             "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
-            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "n"(kQHalfBytes >> 4), "n"(kKVHalfBytes >> 4)
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "r"((uint32_t)go),
+            "n"(kQHalfBytes >> 4), "n"(kKVHalfBytes >> 4)
             : "memory");
 }
 #undef AMSKV_SS_STEP
@@ -243,7 +250,7 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
 // `empty` where `release` is set, to `full` where `last` is.
 __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t desc_hi, uint32_t idesc,
                                         uint32_t accumulate, uint32_t steps, uint32_t release, uint32_t empty, uint32_t last,
-                                        uint32_t full)
+                                        uint32_t full, bool go)
 {
     asm volatile(
         "{\n"
@@ -251,6 +258,7 @@ __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32
         ".reg .b32 t, a;\n"
         ".reg .b64 db;\n"
         "elect.sync _|e, 0xffffffff;\n"
+        "setp.ne.and.u32 e, %11, 0, e;\n"
         "setp.ne.u32 acc, %5, 0;\n"
         "setp.eq.u32 yes, 0, 0;\n"
         "setp.gt.and.u32 s1, %6, 1, e;\n"
@@ -275,7 +283,7 @@ __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32
         "@r tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n"
         "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%10];\n"
         "}\n" ::"r"(o_tmem), "r"(p_tmem), "r"(v_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(steps), "r"(release), "r"(empty),
-        "r"(last), "r"(full)
+        "r"(last), "r"(full), "r"((uint32_t)go)
         : "memory");
 }
 

@@ -322,6 +322,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     constexpr bool kOwnLate = !kWide && !kShort;
     uint32_t tmem = 0;
     auto allocate = [&]() {
+        __syncwarp();   // (an aligned instruction; loops and a branch of one lane lie before)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)),
                      "r"(C::kTmemCols)
                      : "memory");

@@ -67,6 +67,13 @@ def test_no_load_promises_that_its_data_is_read_only(path):
         assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", text[m.end():text.index("{", m.end())])
 
 
+def test_the_producer_of_the_paired_kernel_allocates_as_a_whole_warp():
+    """tcgen05.alloc is an aligned instruction, and loops of unequal length or a branch of one lane come before it."""
+    body = [b for _, n, b in KERNELS if n == "attend_pair_kernel"][0]
+    assert body.count("tcgen05.alloc") == 1
+    assert re.search(r"__syncwarp\(\);\s*asm volatile\(\"tcgen05\.alloc", body)
+
+
 def _check_end_of_a_launch_that_gave_up(header, body):
     """The issuing warps of the paired kernel issue nothing more once a wait of theirs has given up -- their commits are what the other
     roles take for landed data and free stages -- and what is under way then ends before memory is given back."""

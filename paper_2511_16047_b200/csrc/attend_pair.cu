@@ -25,9 +25,8 @@
 // stands, and only a row whose tile sum leaves the range (beyond 2^64, or not a number) makes
 // its warp take the true maxima, rescale and form the tile again.  The first lane of each group fetches its
 // next query tile as soon as the last S of the current one has landed.
-// Every wait is bounded: a wait that gives up records a status code and sets a flag; no role issues another load, product,
-// commit or store on what that wait was for, so all of them stop, and then the copies and products still
-// under way are awaited and the tensor memory is freed.
+// Every wait is bounded: one that gives up records a status code and sets a flag, its role stops, and so do the others at
+// their next wait for it.  Copies and products still under way then are awaited, and the tensor memory is freed.
 #include <algorithm>
 #include <type_traits>
 
@@ -626,12 +625,14 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
         // hence a key/value stage is released by one arrival per issuing warp: each commits its own P V on a
         // shared tile, and the one stream that uses a tile of its own commits twice.
         //
-        // A warp's own instructions are what a tile costs here: a satisfied wait of a voting warp 220 clocks, a branch into the
-        // elected lane and back 130, the bookkeeping of a tile 500, against 320 (64 channels) and 640 clocks of products.  So a
-        // wait that gives up does not change the course (the lane's `go` ends, and with it what it issues), a product's
-        // instructions and commits are one predicated block, and a tile's length is fetched a tile ahead.  Eight images, T = 4 096,
-        // 128 channels: 4 836 -> 4 717 us a call at the same power; one image, T = 576 and 1 600: 35.7 -> 31.5 and 98.3 -> 93.4; 64
-        // channels, 256 items, T = 64 and 100: 9.35 -> 9.05 and 11.9 -> 11.6, and no change where the softmax warps fill the SM.
+        // A warp's own instructions are what a tile costs here: a satisfied wait in the other roles' form 220 clocks, a branch into
+        // the elected lane and back 130, the bookkeeping of a tile 500, against 320 (64 channels) and 640 clocks of products.  So
+        // a satisfied wait is a poll, a vote and a branch, a product's instructions and commits are one predicated block, and a
+        // tile's length is fetched a tile ahead.  Eight images, T = 4 096, 128 channels: 4 836 -> 4 717 us a call at the same
+        // power; one image, T = 576 and 1 600: 35.7 -> 31.5 and 98.3 -> 93.4; 64 channels, 256 items, T = 64 and 100: 9.35 -> 9.05
+        // and 11.9 -> 11.6, and no change where the softmax warps fill the SM.  (Those without the votes, by which the warp stops
+        // as one behind a wait that gives up: they cost 0.3 to 0.8 % of a pass of few items.  Lanes that each remember how their
+        // waits ended, and predicates on that in the blocks: 7 130 -> 7 550 us a 256x256 pass of 15 360 items, three layers.)
         const int my_g = C::kMmaWarps == 2 ? warp - kMmaWarp : 0;
         if (my_pairs > 0) {
             constexpr int kStreams = C::kMmaWarps == 2 ? 1 : 2;   // streams this warp issues for
@@ -640,9 +641,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             const uint32_t v_lo0 = desc_lo(kv_smem + C::kKVBytes, C::kKVHalfBytes);  // V tile of stage 0, MN-major
             const uint32_t q_lo0 = desc_lo(q_smem, 16);
             constexpr uint32_t kStageLo = C::kStageBytes >> 4, kQLo = C::kQBytes >> 4;
-            bool go = true;   // no wait of this lane has given up
-            auto await = [&](const uint32_t bar, const uint32_t parity) {
-                if (go) go = wait_through(bar, parity, status, kStatusMmaTimeout, abort_flag);
+            auto await = [&](const uint32_t bar, const uint32_t parity) -> bool {
+                return warp_wait_lean(bar, parity, status, kStatusMmaTimeout, abort_flag);
             };
             // per stream: the tile whose S was issued last and whose P V is still to be issued
             uint32_t pv_stage[kStreams] = {}, pv_nch[kStreams] = {}, pv_first[kStreams] = {}, pv_last[kStreams] = {},
@@ -656,21 +656,22 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
 
             // O (+)= P V : M = 128, N = D channels, K = 16 * nch tokens; P from TMEM (packed over S),
             // V read MN-major from its stage
-            auto issue_pv = [&](const int i) {
+            auto issue_pv = [&](const int i) -> bool {
                 const int g = kStreams == 2 ? i : my_g;
                 const uint32_t t = tcount[i] - 1u;  // flat tile index of this stream
-                await(p_full0 + 16 * g + 8 * buf_of(t), par_of(t));
+                if (!await(p_full0 + 16 * g + 8 * buf_of(t), par_of(t))) return false;
                 // (a unit's first P V overwrites O: every warp of the group arrives on p_full for that tile
                 // only after its epilogue of the previous unit, so O has been read by then)
                 tc_fence_after();
                 const uint32_t empty = kv_empty0 + 8 * pv_stage[i];
                 umma_pv(tmem + C::kOCol + g * D, tmem + C::kSCol + (g * C::kSBufs + buf_of(t)) * kKT,
                         v_lo0 + pv_stage[i] * kStageLo, kDescHi, idesc_pv, pv_first[i] ^ 1u, pv_nch[i], pv_release[i], empty,
-                        pv_last[i], o_full0 + 8 * g, go);
+                        pv_last[i], o_full0 + 8 * g);
                 if (C::kMmaWarps == 2) {
-                    if (pv_twice[i]) umma_commit_elected(empty, go);
-                    umma_commit_elected(pv_done0 + 8 * g, go);   // read by the (rare) rescale of O only
+                    if (pv_twice[i]) umma_commit_elected(empty);
+                    umma_commit_elected(pv_done0 + 8 * g);   // read by the (rare) rescale of O only
                 }
+                return true;
             };
             auto tile_steps = [&](const int j) -> uint32_t {   // 16-token steps of tile j
                 int32_t t0, valid;
@@ -698,7 +699,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                         if (g == 1 && !two) {
                             // the stream is absent from this pair: its last P V of the previous pair must not
                             // wait for a next S that is not coming soon (it also holds a key/value stage)
-                            if (pv_live[i]) issue_pv(i);
+                            if (pv_live[i] && !issue_pv(i)) goto stopped;
                             pv_live[i] = false;
                             continue;
                         }
@@ -714,16 +715,17 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                             if (tcount[i] == 0) wait_for_previous();   // (the waits that follow have a limit, the launch before has none)
                             const uint32_t u = ucount[i]++;
                             q_half[i] = q_split ? (u & 1u) : 0u;
-                            await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u);
+                            if (!await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u)) goto stopped;
                         }
-                        if (!(shared && i == 1)) await(kv_full0 + 8 * stage, use & 1u);   // one issuer: the second stream of a shared tile finds it landed
-                        if (!s_first && pv_live[i]) issue_pv(i);
+                        // (one issuer: the second stream of a shared tile finds it landed)
+                        if (!(shared && i == 1) && !await(kv_full0 + 8 * stage, use & 1u)) goto stopped;
+                        if (!s_first && pv_live[i] && !issue_pv(i)) goto stopped;
                         tc_fence_after();
                         const uint32_t buf = buf_of(tcount[i]);
                         umma_s<D, C::kQHalfBytes, C::kKVHalfBytes>(tmem + C::kSCol + (g * C::kSBufs + buf) * kKT,
                                                                   q_lo0 + g * kQLo + q_half[i] * (kQHalfSlot >> 4), k_lo0 + stage * kStageLo,
-                                                                  kDescHi, idesc_s, s_full0 + 16 * g + 8 * buf, go);
-                        if (s_first && pv_live[i]) issue_pv(i);
+                                                                  kDescHi, idesc_s, s_full0 + 16 * g + 8 * buf);
+                        if (s_first && pv_live[i] && !issue_pv(i)) goto stopped;
                         pv_live[i] = true;
                         pv_stage[i] = stage;
                         pv_nch[i] = nch;
@@ -738,7 +740,8 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
             }
 #pragma unroll
             for (int i = 0; i < kStreams; ++i)
-                if (pv_live[i]) issue_pv(i);
+                if (pv_live[i] && !issue_pv(i)) goto stopped;
+        stopped:
             if (!owned) own_late();
         } else {
             own_late();
@@ -1141,7 +1144,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     tc_fence_before();
     __syncthreads();
     if (layout_ok && *abort_flag) {   // (the same for all threads: no role is left to set it)
-        // A launch that gave up.  Nothing issues any more; what nobody may have waited for, the newest copy into each stage and
+        // A launch that gave up.  Nothing is issued any more; what nobody may have waited for, the newest copy into each stage and
         // the products, ends before shared and tensor memory are given back (query tiles: at the end of the softmax role).
         auto until = [](const uint32_t bar, const uint32_t parity) {
             for (uint32_t i = 0; i < kSpinLimit; ++i)
@@ -1153,7 +1156,7 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
                 until(kv_full0 + 8 * (q % C::kStages), (q / C::kStages) & 1u);
         } else if (warp >= kMmaWarp) {
             const uint32_t drained = smem_u32(&bars->drained[warp - kMmaWarp]);
-            umma_commit_elected(drained, true);
+            umma_commit_elected(drained);
             until(drained, 0u);
         }
         __syncthreads();

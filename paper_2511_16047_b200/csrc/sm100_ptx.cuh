@@ -73,22 +73,6 @@ __device__ __forceinline__ void report(int* status, int code, volatile int* abor
     atomicCAS(status, 0, code);
     *abort_flag = 1;
 }
-// Bounded wait of a warp that stays on one path: what follows is the same code however it ended.  False in a lane that gave up
-// (it sets the abort flag) or saw the flag set; the blocks below then issue nothing (`go`).
-__device__ __forceinline__ bool wait_through(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    for (uint32_t i = 1; !mbar_try_wait(bar, parity); ++i) {
-        if ((i & 255u) != 0u) continue;
-        if (*abort_flag) return false;
-        if (i >= kSpinLimit) {
-            report(status, code, abort_flag);
-            return false;
-        }
-    }
-    return true;
-}
-
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2)
 {
     asm volatile(
@@ -175,6 +159,22 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
 {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
 }
+// The same for a warp whose own instructions are what its work waits for: one poll, one vote and one uniform branch where the phase is
+// complete already.  It reports a wait that runs out itself.
+__device__ __forceinline__ bool warp_wait_lean(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+#pragma unroll 1
+    for (uint32_t i = 1; !__all_sync(0xffffffffu, mbar_try_wait(bar, parity)); ++i) {
+        if ((i & 255u) != 0u) continue;
+        if (__any_sync(0xffffffffu, *abort_flag)) return false;
+        if (i >= kSpinLimit) {
+            report(status, code, abort_flag);
+            return false;
+        }
+    }
+    return true;
+}
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -185,17 +185,15 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// The blocks below are issued from a converged warp by one of its lanes, always the same one, and only if that lane's `go` is set:
-// its own waits have all ended well, so what it issues reads data that has landed.
-__device__ __forceinline__ void umma_commit_elected(uint32_t bar, bool go)
+// The same from a converged warp, by one of its lanes.
+__device__ __forceinline__ void umma_commit_elected(uint32_t bar)
 {
     asm volatile(
         "{\n"
         ".reg .pred e;\n"
         "elect.sync _|e, 0xffffffff;\n"
-        "setp.ne.and.u32 e, %1, 0, e;\n"
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-        "}\n" ::"r"(bar), "r"((uint32_t)go)
+        "}\n" ::"r"(bar)
         : "memory");
 }
 // Shared-memory matrix descriptors are passed as two 32-bit halves: the low half carries the
@@ -209,8 +207,7 @@ __device__ __forceinline__ void umma_commit_elected(uint32_t bar, bool go)
     "mov.b64 db, {t, %3};\n"                                                         \
     "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " acc ";\n"
 template <int D, uint32_t kQHalfBytes, uint32_t kKVHalfBytes>
-__device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc, uint32_t bar,
-                                       bool go)
+__device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t desc_hi, uint32_t idesc, uint32_t bar)
 {
     static_assert(D == 64 || D == 128, "one or two 128-byte swizzle atoms per row");
     if (D == 64)
@@ -220,12 +217,11 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
             ".reg .b32 t;\n"
             ".reg .b64 da, db;\n"
             "elect.sync _|e, 0xffffffff;\n"
-            "setp.ne.and.u32 e, %6, 0, e;\n"
             "setp.eq.u32 yes, 0, 0;\n"
             "setp.ne.u32 no, 0, 0;\n"
             AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
             "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
-            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "r"((uint32_t)go)
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar)
             : "memory");
     else
         asm volatile(
@@ -234,15 +230,13 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
             ".reg .b32 t;\n"
             ".reg .b64 da, db;\n"
             "elect.sync _|e, 0xffffffff;\n"
-            "setp.ne.and.u32 e, %6, 0, e;\n"
             "setp.eq.u32 yes, 0, 0;\n"
             "setp.ne.u32 no, 0, 0;\n"
             AMSKV_SS_STEP("0", "0", "no") AMSKV_SS_STEP("2", "2", "yes") AMSKV_SS_STEP("4", "4", "yes") AMSKV_SS_STEP("6", "6", "yes")
-            AMSKV_SS_STEP("%7", "%8", "yes") AMSKV_SS_STEP("%7 + 2", "%8 + 2", "yes") AMSKV_SS_STEP("%7 + 4", "%8 + 4", "yes")
-            AMSKV_SS_STEP("%7 + 6", "%8 + 6", "yes")
+            AMSKV_SS_STEP("%6", "%7", "yes") AMSKV_SS_STEP("%6 + 2", "%7 + 2", "yes") AMSKV_SS_STEP("%6 + 4", "%7 + 4", "yes")
+            AMSKV_SS_STEP("%6 + 6", "%7 + 6", "yes")
             "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n"
-            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "r"((uint32_t)go),
-            "n"(kQHalfBytes >> 4), "n"(kKVHalfBytes >> 4)
+            "}\n" ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(desc_hi), "r"(idesc), "r"(bar), "n"(kQHalfBytes >> 4), "n"(kKVHalfBytes >> 4)
             : "memory");
 }
 #undef AMSKV_SS_STEP
@@ -250,7 +244,7 @@ __device__ __forceinline__ void umma_s(uint32_t d_tmem, uint32_t q_lo, uint32_t 
 // `empty` where `release` is set, to `full` where `last` is.
 __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t desc_hi, uint32_t idesc,
                                         uint32_t accumulate, uint32_t steps, uint32_t release, uint32_t empty, uint32_t last,
-                                        uint32_t full, bool go)
+                                        uint32_t full)
 {
     asm volatile(
         "{\n"
@@ -258,7 +252,6 @@ __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32
         ".reg .b32 t, a;\n"
         ".reg .b64 db;\n"
         "elect.sync _|e, 0xffffffff;\n"
-        "setp.ne.and.u32 e, %11, 0, e;\n"
         "setp.ne.u32 acc, %5, 0;\n"
         "setp.eq.u32 yes, 0, 0;\n"
         "setp.gt.and.u32 s1, %6, 1, e;\n"
@@ -283,7 +276,7 @@ __device__ __forceinline__ void umma_pv(uint32_t o_tmem, uint32_t p_tmem, uint32
         "@r tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n"
         "@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%10];\n"
         "}\n" ::"r"(o_tmem), "r"(p_tmem), "r"(v_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate), "r"(steps), "r"(release), "r"(empty),
-        "r"(last), "r"(full), "r"((uint32_t)go)
+        "r"(last), "r"(full)
         : "memory");
 }
 

@@ -77,20 +77,23 @@ def test_the_producer_of_the_paired_kernel_allocates_as_a_whole_warp():
 def _check_end_of_a_launch_that_gave_up(header, body):
     """The issuing warps of the paired kernel issue nothing more once a wait of theirs has given up -- their commits are what the other
     roles take for landed data and free stages -- and what is under way then ends before memory is given back."""
-    blocks = [m.group(0) for m in re.finditer(r"asm volatile\((?:[^;]|;(?!\n\s*(?:\}|else)))*?elect\.sync _\|e.*?\"memory\"\);", header, flags=re.S)]
-    assert len(blocks) == 4                                    # a commit, S with 64 and with 128 channels, P V
-    for block in blocks:
-        assert re.search(r"elect\.sync _\|e, 0xffffffff;\\n\"\s*\"setp\.ne\.and\.u32 e, %\d+, 0, e;", block) and "(uint32_t)go" in block
-        assert all(p for p in re.findall(r"(@\w+ )?tcgen05\.(?:mma|commit)", block))
-    assert re.search(r"bool wait_through\([^}]*report\([^;]*;\s*return false;", header)
-    assert re.search(r"if \(go\) go = wait_through\(", body) and body.count("wait_through(") == 1
+    wait = re.search(r"bool warp_wait_lean\(.*?\n}", header, flags=re.S).group(0)
+    assert wait.count("__all_sync(0xffffffffu, mbar_try_wait(bar, parity))") == 2 and "__any_sync(0xffffffffu, *abort_flag)" in wait
+    assert wait.count("return true;") == 2 and re.search(r"report\([^;]*;\s*return false;", wait)
     role, end = body[: body.rindex("dealloc")].rsplit("if (layout_ok && *abort_flag) {", 1)
-    issued = re.findall(r"umma_(?:s|pv|commit_elected)\b[^;]*;", role)
-    assert len(issued) == 4 and all(re.search(r", go\);", call) for call in issued)
+    issuer = role[role.index("warp >= kMmaWarp"):]
+    issuer = issuer[: issuer.index("stopped:")]
+    assert body.count("warp_wait_lean(") == issuer.count("return warp_wait_lean(") == 1
+    for call in ("await", "issue_pv"):
+        uses = re.findall(r"(\S*)\b%s\([^;]*;" % call, issuer)
+        tails = re.findall(r"\b%s\([^;]*\) (goto stopped|return false);" % call, issuer)
+        assert len(uses) == len(tails) >= 3 and all(u.endswith("!") for u in uses)
+    assert len(re.findall(r"umma_(?:s|pv|commit_elected)\b[^;]*;", role)) == 4 == len(re.findall(r"umma_(?:s|pv|commit_elected)\b[^;]*;", issuer))
+    assert re.search(r"stopped:\s*if \(!owned\) own_late\(\);\s*\}", role)
     assert re.search(r"__syncthreads\(\);\s*$", role)           # all roles have stopped
     assert re.search(r"if \(!ok\) report\([^;]*;\s*bars->issued = sq;", role)
     assert re.search(r"for \(uint32_t q = un; q < q_armed; \+\+q\)", role)
-    assert re.search(r"bars->issued.*until\(kv_full0.*umma_commit_elected\(drained, true\);\s*until\(drained.*__syncthreads\(\);\s*\}\s*if", end, flags=re.S)
+    assert re.search(r"bars->issued.*until\(kv_full0.*umma_commit_elected\(drained\);\s*until\(drained.*__syncthreads\(\);\s*\}\s*if", end, flags=re.S)
 
 
 def _pair():
@@ -102,11 +105,11 @@ def test_a_launch_that_gave_up_issues_nothing_more_and_ends_its_copies():
 
 
 @pytest.mark.parametrize("old,new", [
-    ("if (go) go = wait_through(", "wait_through("),                            # products behind a wait that gave up
-    ("s_full0 + 16 * g + 8 * buf, go);", "s_full0 + 16 * g + 8 * buf, true);"),
-    ("umma_commit_elected(empty, go);", "umma_commit_elected(empty, true);"),
-    ('"setp.ne.and.u32 e, %11, 0, e;\\n"', ""),
-    ('"@r tcgen05.commit', '"tcgen05.commit'),
+    ("!await(kv_full0 + 8 * stage, use & 1u)) goto stopped;", "!await(kv_full0 + 8 * stage, use & 1u)) tc_fence_after();"),
+    ("if (!await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u)) goto stopped;",
+     "await(q_full0 + 16 * g + 8 * q_half[i], (q_split ? u >> 1 : u) & 1u);"),
+    ("if (s_first && pv_live[i] && !issue_pv(i)) goto stopped;", "if (s_first && pv_live[i]) issue_pv(i);"),
+    ("if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;", "if (mbar_try_wait(bar, parity)) return true;"),
     ("report(status, code, abort_flag);\n            return false;", "report(status, code, abort_flag);\n            break;"),
     ("if (!ok) report(status, kStatusTmaTimeout, abort_flag);\n            bars->issued = sq;",
      "if (!ok) { report(status, kStatusTmaTimeout, abort_flag); bars->issued = sq; }"),

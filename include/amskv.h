@@ -403,9 +403,10 @@ AMSKV_API int amskv_cache_bytes(const amskv_cache* cache, size_t* allocated, siz
  * return AMSKV_OK regardless, and only this call tells.  amskv_cache_reset does not touch the word. */
 AMSKV_API int amskv_status(amskv_cache* cache, int* device_status);
 
-/* Diagnostic (the paper has no counterpart): enqueues one 32-thread kernel whose bounded wait -- the same
- * helper every attention kernel waits with -- runs out after `iterations` polls (1 .. 2^20) of a barrier
- * that nothing arrives at.  The kernel records code 3 in the cache's status word and returns normally;
+/* Diagnostic (the paper has no counterpart): enqueues one 32-thread kernel whose bounded waits -- the same
+ * helpers the attention kernels wait with, that of the issuing warps first -- run out after `iterations` polls
+ * (1 .. 2^20) of a barrier that nothing arrives at.  The kernel records code 3 in the cache's status word
+ * (2 if the issuing warps' wait did not record its own as it should) and returns normally;
  * nothing faults or hangs.  Lets a caller (and the tests) check the whole reporting chain:
  * amskv_status must then return AMSKV_ERR_DEVICE_TIMEOUT once, and AMSKV_OK afterwards. */
 AMSKV_API int amskv_selftest_wait_timeout(amskv_cache* cache, uint32_t iterations, void* stream);

@@ -161,14 +161,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
 }
 // The same for a warp whose own instructions are what its work waits for: one poll, one vote and one uniform branch where the phase is
 // complete already.  It reports a wait that runs out itself.
-__device__ __forceinline__ bool warp_wait_lean(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag)
+__device__ __forceinline__ bool warp_wait_lean(uint32_t bar, uint32_t parity, int* status, int code, volatile int* abort_flag,
+                                               uint32_t limit = kSpinLimit)
 {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
 #pragma unroll 1
     for (uint32_t i = 1; !__all_sync(0xffffffffu, mbar_try_wait(bar, parity)); ++i) {
-        if ((i & 255u) != 0u) continue;
-        if (__any_sync(0xffffffffu, *abort_flag)) return false;
-        if (i >= kSpinLimit) {
+        if ((i & 255u) == 0u && __any_sync(0xffffffffu, *abort_flag)) return false;
+        if (i >= limit) {
             report(status, code, abort_flag);
             return false;
         }

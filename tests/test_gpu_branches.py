@@ -130,8 +130,9 @@ def test_densities_when_the_reference_maximum_moves(D, rows, heads):
 
 
 def test_a_wait_that_runs_out_is_reported_and_the_cache_stays_usable():
-    """A bounded wait nothing ever satisfies: the kernel gives up after its iteration limit, records its
-    code and returns; amskv_status reports it once; an ordinary pass on the same cache then succeeds."""
+    """A bounded wait nothing ever satisfies, in the issuing warps' form and in the other roles': the kernel gives up after its
+    iteration limit, records its code (another one where the issuing warps' form told less than it should) and returns;
+    amskv_status reports it once; an ordinary pass on the same cache then succeeds."""
     _need(64)
     sides, rows, heads, D = (2, 9), 2, 3, 64
     qkv = make_qkv(rows, heads, sides, D, seed=83)

@@ -32,6 +32,12 @@ def _kernels():
 
 
 KERNELS = _kernels()
+
+
+def _pair():
+    return _text(os.path.join(CSRC, "sm100_ptx.cuh")), [b for _, n, b in KERNELS if n == "attend_pair_kernel"][0]
+
+
 RELEASE = r"launch_dependents|overlap_with_previous\s*\(|let_next_start\s*\("
 WAIT = r"griddepcontrol\.wait|overlap_with_previous\s*\(|wait_for_previous\s*\("
 
@@ -67,6 +73,65 @@ def test_no_load_promises_that_its_data_is_read_only(path):
         assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", text[m.end():text.index("{", m.end())])
 
 
+def _check_order_of_the_paired_kernel(body):
+    """The same for the paired kernel, whose CTAs allocate either ahead of the roles or, in the two-CTA form's long launches, in the
+    producer's branch, and whose roles wait for the launch before on their own, right before what needs it."""
+    one = re.compile(r"if \(!kOwnLate && warp == kProducerWarp\) allocate\(\);\s*tc_fence_before\(\);\s*__syncthreads\(\);")
+    late = re.compile(r"auto own_late = \[&\]\(\) \{\s*if \(!kOwnLate\) return;\s*if \(warp == kProducerWarp\) allocate\(\);\s*"
+                      r"tc_fence_before\(\);\s*barrier_of\(1, C::kThreads\);")
+    early, later = one.search(body), late.search(body)
+    assert early and later and len(re.findall(r"\ballocate\(\)", body)) == 2
+    cuts = [body.index(t) for t in ("if (layout_ok && warp == kProducerWarp) {", "} else if (layout_ok && warp >= kMmaWarp) {", "} else if (layout_ok) {",
+                                    "if constexpr (kSplit) {")]
+    assert later.end() < cuts[0] and cuts == sorted(cuts)
+    before, producer, issuer, softmax = (body[a:b] for a, b in zip([0] + cuts, cuts))
+    assert not re.search(r"tma_load|wait_for_previous|let_next_start", before)
+    # the producer: owns, waits, lets the next launch in, loads
+    assert len(re.findall(RELEASE, body)) == 1
+    order = [producer.index(t) for t in ("own_late();", "if (sq == 0) {", "wait_for_previous();", "let_next_start();", "tma_load")]
+    assert order == sorted(order) and producer.count("own_late();") == 1
+    assert re.search(r"if \(sq == 0\) \{\s*wait_for_previous\(\);\s*let_next_start\(\);\s*\}", producer)
+    # an issuing warp: owns, waits for the launch before, and only then in a wait that has a limit
+    order = [issuer.index(t) for t in ("own_late();", "if (tcount[i] == 0) wait_for_previous();", "if (!await(q_full0", "!await(kv_full0", "umma_s<")]
+    assert order == sorted(order)
+    # the softmax warps: the one that loads queries waits before its first load, all of them before their first S where they own late
+    order = [softmax.index(t) for t in ("if (q_armed == 0) wait_for_previous();", "mbar_expect_tx", "tma_load", "own_late();", "mbar_wait(s_full")]
+    assert order == sorted(order)
+    assert re.search(r"own_late\(\);\s*if \(kOwnLate\) wait_for_previous\(\);", softmax)
+
+
+def test_the_roles_of_the_paired_kernel_own_and_wait_before_they_load():
+    _check_order_of_the_paired_kernel(_pair()[1])
+
+
+@pytest.mark.parametrize("old,new", [
+    ("allocate();\n    tc_fence_before();\n    __syncthreads();", "{}\n    tc_fence_before();\n    __syncthreads();\n    allocate();"),
+    ("        barrier_of(1, C::kThreads);\n", ""),
+    ("        own_late();\n        uint32_t st_sq", "        uint32_t st_sq"),
+    ("                        let_next_start();\n", "                        let_next_start();\n                        own_late();\n"),
+    ("if (sq == 0) {\n                        wait_for_previous();", "if (sq == 0) {"),
+    ("if (sq == 0) {\n", "if (sq == 1) {\n"),
+    ("if (tcount[i] == 0) wait_for_previous();", ""),
+    ("if (q_armed == 0) wait_for_previous();", ""),
+    ("if (kOwnLate) wait_for_previous();", ""),
+    ("auto own_late = [&]() {", "let_next_start();\n    auto own_late = [&]() {"),
+])
+def test_the_check_of_the_roles_order_rejects(old, new):
+    body = _pair()[1]
+    assert body.count(old) == 1
+    with pytest.raises((AssertionError, ValueError)):
+        _check_order_of_the_paired_kernel(body.replace(old, new))
+
+
+def test_a_producer_that_owns_its_columns_behind_the_release_is_rejected():
+    body = _pair()[1]
+    moved = body.replace("        own_late();\n        uint32_t st_sq", "        uint32_t st_sq")
+    moved = moved.replace("let_next_start();\n", "let_next_start();\n                        own_late();\n")
+    assert moved != body and moved.count("own_late();") == body.count("own_late();")
+    with pytest.raises(AssertionError):
+        _check_order_of_the_paired_kernel(moved)
+
+
 def test_the_producer_of_the_paired_kernel_allocates_as_a_whole_warp():
     """tcgen05.alloc is an aligned instruction, and loops of unequal length or a branch of one lane come before it."""
     body = [b for _, n, b in KERNELS if n == "attend_pair_kernel"][0]
@@ -94,10 +159,6 @@ def _check_end_of_a_launch_that_gave_up(header, body):
     assert re.search(r"if \(!ok\) report\([^;]*;\s*bars->issued = sq;", role)
     assert re.search(r"for \(uint32_t q = un; q < q_armed; \+\+q\)", role)
     assert re.search(r"bars->issued.*until\(kv_full0.*umma_commit_elected\(drained\);\s*until\(drained.*__syncthreads\(\);\s*\}\s*if", end, flags=re.S)
-
-
-def _pair():
-    return _text(os.path.join(CSRC, "sm100_ptx.cuh")), [b for _, n, b in KERNELS if n == "attend_pair_kernel"][0]
 
 
 def test_a_launch_that_gave_up_issues_nothing_more_and_ends_its_copies():

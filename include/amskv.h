@@ -96,7 +96,9 @@ extern "C" {
 /* Outputs do not depend on the values of other rows and heads, and a call repeated is bit-equal.  Under AUTO the kernel,
  * its form and the order of its key tiles are chosen by rows x heads and the number of SMs as well as by the scale, so the
  * outputs of an image computed together with other numbers of images may differ in rounding (2e-3 in the 2-norm, as both
- * do from exact sums).  Under every other path the scale alone decides, and they are bit-equal. */
+ * do from exact sums).  Under every other path the scale alone decides, and they are bit-equal.  amskv_append_attend and
+ * the two calls it stands for choose the same kernel unless the append is several copies, but the paired kernel takes the
+ * current scale's keys as tiles of their own when it appends them, so their outputs may differ in rounding too. */
 
 typedef struct amskv_cache amskv_cache; /* opaque; owned by the library */
 
@@ -214,7 +216,7 @@ AMSKV_API int amskv_attend(amskv_cache* cache, int layer, int scale, const void*
 
 /*
  * amskv_append(layer, scale, K, V) followed by amskv_attend(layer, scale, Q, out), with the same
- * results, cache state and order contract (scale must be the layer's next scale), in one kernel
+ * results (up to the rounding that another order of key tiles brings), cache state and order contract (scale must be the layer's next scale), in one kernel
  * launch where possible: Algorithm 1 appends a scale right before that scale attends, so the
  * paired tensor-core kernel can read the scale's K and V from the caller's tensors, use them as
  * keys and values beside the older retained tokens it reads from the cache, and write them to
@@ -398,7 +400,7 @@ AMSKV_API int amskv_cache_bytes(const amskv_cache* cache, size_t* allocated, siz
  * kernel reported a problem since the last call; otherwise it is the code of the first bounded wait that
  * gave up (1: a key/value or query copy did not arrive, 2: the MMA-issuing warp gave up, 3: a softmax
  * group or another role gave up) and the return value is AMSKV_ERR_DEVICE_TIMEOUT.  A kernel that gives
- * up still returns normally (its roles wind down, copies in flight are awaited, tensor memory is freed),
+ * up still returns normally (its roles stop, copies and products in flight are awaited, tensor memory is freed),
  * so the context stays usable, but the outputs of that launch are undefined: the calls that enqueue work
  * return AMSKV_OK regardless, and only this call tells.  amskv_cache_reset does not touch the word. */
 AMSKV_API int amskv_status(amskv_cache* cache, int* device_status);

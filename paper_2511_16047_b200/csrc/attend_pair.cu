@@ -311,13 +311,16 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_const
     // Everything up to a role's first load touches only this CTA's own memory, so it runs while the kernel before this one
     // ends: the threads that issue this CTA's loads wait for that kernel right before the first of them, and what the others
     // read or write follows from those loads.  By then the code up to there, its launch parameters and its tensor maps have
-    // been fetched.  With one wait for all here, a launch issued its first loads 2 000 to 3 800 clocks after it: 60 items, T =
-    // 100, 169 and 256 6.86 / 9.55 / 11.1 -> 6.05 / 8.95 / 10.0 us a call, 256 items, T = 64 and 100 9.05 / 11.6 -> 8.76 / 11.0, 1 920 items, T =
-    // 25 and 36 19.1 / 23.7 -> 17.3 / 22.6, 128 channels, 32 items, T = 144 and 400 8.74 / 16.5 -> 7.8 / 15.7; neutral at large launches.
+    // been fetched.  With one wait for all here, a launch issued its first loads 2 000 to 3 800 clocks after it.  us a call, before
+    // and after (neutral at large launches):
+    //   64 channels, 60 items      T = 100   6.86 -> 6.05    T = 169  9.55 -> 8.95    T = 256  11.1 -> 10.0
+    //   64 channels, 256 items     T =  64   9.05 -> 8.76    T = 100  11.6 -> 11.0
+    //   64 channels, 1 920 items   T =  25   19.1 -> 17.3    T =  36  23.7 -> 22.6
+    //   128 channels, 32 items     T = 144   8.74 -> 7.8     T = 400  16.5 -> 15.7
     // Tensor memory is owned before the roles split, but in the two-CTA form's long launches (kOwnLate), where the producer
-    // allocates behind its preparations and the other warps meet it there, the softmax warps after the wait: 256 items, T = 169 and
-    // 256 14.8 / 21.3 -> 14.3 / 20.6, 2 304 items, T = 324 223 -> 218, but in the other forms 60 items, T = 100 6.05 -> 6.88 and 256
-    // items, T = 64 8.76 -> 8.95.
+    // allocates behind its preparations and the other warps meet it there, the softmax warps after the wait:
+    //   where it is done so        256 items, T = 169  14.8 -> 14.3, T = 256  21.3 -> 20.6;  2 304 items, T = 324  223 -> 218
+    //   in the other forms         60 items, T = 100   6.05 -> 6.88;  256 items, T = 64  8.76 -> 8.95
     constexpr bool kOwnLate = !kWide && !kShort;
     uint32_t tmem = 0;
     auto allocate = [&]() {

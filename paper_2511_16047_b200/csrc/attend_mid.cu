@@ -543,7 +543,7 @@ cudaError_t launch(bool overlap, const Strided& Q, const Strided& O, const Layer
 // appends by which it would now win below them (by up to 17 %) stay here all the same: they keep this kernel's weights (every
 // exponential from the special-function unit, the reference a maximum over 32 keys of each half, where the paired kernel's may be
 // that of a tile of 21; peaked rows, off exact sums: T = 36, 57 keys, 128 channels 1.67e-3 / 1.97e-3, T = 64, 105 keys, 64
-// channels 1.84e-3 / 1.96e-3, from 129 keys with 64 channels the same), and fused and separate appends of one copy choose alike.
+// channels 1.84e-3 / 1.96e-3, at 134 and more the same), and fused and separate appends of one copy choose alike.
 // With the density 20 and 7 units (times with the append and the zeroed result): T = 25: 18.2 / 18.7
 // (1 024 items), 27.8 / 29.3 (1 920, 25.9 units); T = 36: 10.4 / 12.4 (240), 15.0 / 13.1 (300); T = 64: 12.3 / 15.1 (240), 18.2 / 16.7 (300); T = 81:
 // 12.6 / 16.2 (148, 18 units), 18.0 / 16.9 (180); 128 channels: T = 25: 18.2 / 20.1 (512, 6.9 units), 23.6 / 25.3 (700), 49 / 49 (1 920); T = 36: 11.6 /
